@@ -77,8 +77,9 @@ typedef struct {
   int groups;        /* right-hand sides per sweep team (1, 2, 4, 5 or 8; 0 = automatic) */
   int sweep_kernel;  /* 0: automatic (default): with strong_rank > 0 the sweep on the strongly
                            admissible format (hsweep_strong_export) where its plan fits, then
-                           the bulk-copy-staged sweep on cooperative teams where its
-                           shared-memory plan fits, else the basic sweep;
+                           the bulk-copy-staged sweep on teams of CTAs (dense-diagonal
+                           slabs, else the sibling-pair factors) where its shared-memory
+                           plan fits, else the basic sweep;
                         1: the basic sweep that reads the factors from global memory;
                         2: the team sweep on the sibling-pair factors (for strong_rank > 0:
                            the stored, recompressed expansion), else the basic sweep */
@@ -226,8 +227,9 @@ HSWEEP_API int hsweep_create(const double* c_dev, double omega, int n, int pml_w
  * T~_m u_m, backward sweep), for nrhs vectors at once.
  *   r, z  device [nrhs][N]; r is not modified; r and z must not overlap.
  * Stream-ordered; returns after enqueue.
- * CUDA graphs: for an upward handle (sweep_dir = +1) the call enqueues one memset of the
- * exchange slots and one cooperative kernel launch on the handle's stream, and may be
+ * CUDA graphs: for an upward handle (sweep_dir = +1) the call enqueues only sweep launches
+ * (one, or a few when the teams of a large batch run in turns) and, where the sweep exchanges
+ * through global memory, memsets of its slots, on the handle's stream, and may be
  * captured into a graph on that stream (replays repeat the call on the captured r and
  * z).  A capture allocates nothing: size the handle's buffers first with one call
  * outside the capture with at least as many right-hand sides; a capture that would
@@ -350,13 +352,15 @@ HSWEEP_API int hsweep_stats(hsweep_t h, int reset, long long* launches, long lon
 
 /*
  * The launch plan the apply would use for nrhs right-hand sides (diagnostics):
- * out[0] the sweep kernel (0: basic, 2: bulk-copy-staged on cooperative teams exchanging
- * tagged partial sums, 3: the same on the strongly admissible format; 1 is not used),
+ * out[0] the sweep kernel (0: basic, 2: bulk-copy-staged teams of CTAs exchanging partial
+ * sums, 3: the same on the strongly admissible format; 1 is not used),
  * out[1] CTAs per team, out[2] right-hand sides per team,
- * out[3] teams, out[4] for the basic kernel 1 when its team is the whole grid (a grid barrier),
+ * out[3] teams of a launch, out[4] for the basic kernel 1 when its team is the whole grid (a grid barrier),
  * for the team kernels the threads per CTA (512: one CTA per SM, 256: two), out[5] dynamic shared
  * memory per CTA in bytes, out[6] largest per-step factor record of one CTA in bytes,
- * out[7] column slices per row in the expansion (0 for the basic kernel).
+ * out[7] column slices per row in the expansion (0 for the basic kernel); for kernel 2 on
+ * dense-diagonal slabs, the automatic choice up to n = 1024 (complex64) or 512 (complex128,
+ * few right-hand sides), 0 when its teams are clusters and 1 when they exchange through L2.
  */
 HSWEEP_API int hsweep_sweep_plan(hsweep_t h, int nrhs, long long* out8);
 

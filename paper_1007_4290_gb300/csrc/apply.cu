@@ -453,7 +453,9 @@ int hsw_apply(hsweep_s* h, const c128* r, c128* z, int nrhs) {
   }
   if (h->opt.sweep_kernel != 1) {
     bool used = false;
-    int rc = hsw_apply_team(h, r, z, nrhs, &used);
+    int rc = hsw_apply_slab(h, r, z, nrhs, &used);
+    if (rc != HSWEEP_OK || used) return rc;
+    rc = hsw_apply_team(h, r, z, nrhs, &used);
     if (rc != HSWEEP_OK || used) return rc;
   }
   SweepConfig cfg = choose_config(h, nrhs);
@@ -533,7 +535,9 @@ int hsw_apply_scratch(hsweep_s* h, const c128* r, c128* z, int nrhs, void* scrat
   }
   if (h->opt.sweep_kernel != 1) {
     bool used = false;
-    int rc = hsw_apply_team(h, r, z, nrhs, &used, scratch, bytes);
+    int rc = hsw_apply_slab(h, r, z, nrhs, &used, scratch, bytes);
+    if (rc != HSWEEP_OK || used) return rc;
+    rc = hsw_apply_team(h, r, z, nrhs, &used, scratch, bytes);
     if (rc != HSWEEP_OK || used) return rc;
   }
   SweepConfig cfg = choose_config(h, nrhs);

@@ -91,6 +91,18 @@ struct hsweep_s {
   std::vector<int> rank_max_depth;       // per depth d = 0..L: the largest rank over all layers
   bool pack_valid = false;
 
+  // The factors as dense-diagonal slabs for the cluster sweep (sweep_slab.cu): for every
+  // layer and depth-slab_dC node one record of slab_cap entries, its column boundaries in
+  // d_slab_meta; null where the grid is too large for that sweep
+  void* d_slab = nullptr;
+  void* d_slab_meta = nullptr;
+  void* d_slab_cpl = nullptr;            // complex64: the layer couplings d_north_m in that precision
+  int slab_dC = 0, slab_rsD = 0, slab_W = 0, slab_X = 0;   // most columns / received sums of a layer
+  long long slab_cap = 0;
+  bool slab_valid = false;
+  // its launch plans already chosen: {nrhs, ok, L2 teams, G, D stages, groups, groups per launch, smem}
+  std::vector<std::array<long long, 8>> slab_plans;
+
   int* d_status = nullptr;     // [2]
   unsigned* d_bar = nullptr;   // grid barrier words [2]
 
@@ -175,6 +187,13 @@ int hsw_apply_team(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* used, vo
                    size_t scratch_bytes = 0);
 size_t hsw_apply_team_scratch_bytes(hsweep_s* h, int nrhs);
 int hsw_team_plan(hsweep_s* h, int nrhs, long long* out8);   // 1 if the team kernel would run
+// sweep_slab.cu: geometry and buffers of the dense-diagonal slabs, their packing (rk: the
+// ranks of all layers), and the sweep on them
+int hsw_slab_create(hsweep_s* h);
+int hsw_pack_slabs(hsweep_s* h, int m0, int m1, const std::vector<int>& rk);
+int hsw_apply_slab(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* used, void* scratch = nullptr,
+                   size_t scratch_bytes = 0);
+int hsw_slab_plan(hsweep_s* h, int nrhs, long long* out8);   // 1 if the slab sweep would run
 // direction.cu: reversal of the layer order (x2 -> 1 - x2)
 int hsw_flip_reserve(hsweep_s* h, size_t bytes);
 int hsw_flip_c128(hsweep_s* h, const c128* in, c128* out, int nvec);

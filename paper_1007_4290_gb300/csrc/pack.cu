@@ -108,5 +108,5 @@ int hsw_pack(hsweep_s* h, int m0, int m1) {
       h->rank_max_depth[d] = std::max(h->rank_max_depth[d], rk[(size_t)m * h->nnodes + v]);
     }
   h->pack_valid = true;
-  return HSWEEP_OK;
+  return hsw_pack_slabs(h, m0, m1, rk);
 }
