@@ -23,7 +23,8 @@
 // in complex128) are recompressed after every depth that changed them.  A small block whose factors have at least as
 // many columns as rows takes the dense path: its core is the block itself, C = F_a F_b^t,
 // and its new factors come straight from the SVD of C (no QR).  QR is classical
-// Gram-Schmidt with re-orthogonalisation; the SVD is one-sided (Hestenes) Jacobi.
+// Gram-Schmidt with re-orthogonalisation; the SVD is a column-pivoted Gram-Schmidt down to
+// the numerical rank followed by one-sided (Hestenes) Jacobi on what remains.
 // The leaf inverses are computed in FP64 with partial pivoting in both precisions.
 #include <algorithm>
 #include <cmath>
@@ -33,6 +34,12 @@
 namespace {
 
 constexpr int kBlk = 256;
+
+// Dense path of the recompression in complex64: up to this many rows the pivoted Gram-Schmidt
+// of the block itself (svd_jacobi, about 0.3 us for each of the block's 20 to 40 significant
+// columns) is shorter than the QR of its factors (3.6 us for each of up to 98 columns).  A
+// 128 x 128 core is 131 KB of shared memory.  In complex128 the QR is the cheaper.
+constexpr int kDenseRows = 128;
 
 template <typename R> struct Tiny;
 template <> struct Tiny<double> {
@@ -70,6 +77,7 @@ template <typename R> __device__ R block_sum(R v, R* red) {
 
 struct Geo {          // tree and buffer geometry passed by value to every kernel
   int n, L, leaf, nnodes, r_max, KCAP, WCAP, QCAP;
+  int dense_max;           // blocks of at most so many rows take the dense path at any rank
   const int* lo;
   const int* sz;
   const int* rowleaf;      // [n] leaf node of each row
@@ -472,8 +480,9 @@ __global__ void woodbury_append(Geo g, int d, const int* __restrict__ S_rank, co
 
 // ---------------------------------------------------------------------------------
 // Recompression, step 1, for the nodes u = list[blockIdx.x]: with w = rank(u) columns,
-// a factor with at least as many columns as rows (w >= sz(u)) takes the dense path,
-// Q = I and R = F_u (qcols = sz(u), qmode = 1); otherwise Gram-Schmidt QR (twice
+// a factor with at least as many columns as rows (w >= sz(u)), or in complex64 of at most
+// kDenseRows rows, takes the dense path, Q = I and R = F_u (qcols = sz(u), qmode = 1);
+// otherwise Gram-Schmidt QR (twice
 // orthogonalised) of F_u in place, the Q columns compacted to the independent ones and
 // R (qc x w) written out (qmode = 0).  R is row-major with leading dimension cap(u).  When
 // F_u fits the kernel's shared memory (qs_entries), the orthogonalisation runs there and
@@ -487,7 +496,7 @@ __global__ void qr_cgs2(Geo g, Cx<R>* __restrict__ G_F, const int* __restrict__ 
   const int s = g.sz[u], w = G_rank[u], ld = g.cap[u];
   Cx<R>* F = G_F + g.gfo[u];
   Cx<R>* Rm = Rb + g.rbo[u];                               // row-major qc x w, ld cap(u)
-  if (w >= s && s <= g.QCAP) {
+  if ((w >= s && s <= g.QCAP) || s <= g.dense_max) {
     for (int e = threadIdx.x; e < s * w; e += blockDim.x) {
       const int i = e % s, l = e / s;
       Rm[(long long)i * ld + l] = F[e];
@@ -729,77 +738,165 @@ template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW
   return v;
 }
 
+// Reciprocal and reciprocal square root, in complex128 by two Newton steps from the FP32
+// value (a handful of FP64 operations where the division and square root routines take
+// dozens: a warp's FP64 instruction occupies its scheduler for about 64 clocks here)
+__device__ __forceinline__ float rcp_of(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rcp_of(double x) {
+  // x in [1e-28, 4]: inside FP32's range
+  double y = (double)(1.0f / (float)x);
+  y = y * fma(-x, y, 2.0);
+  return y * fma(-x, y, 2.0);
+}
+__device__ __forceinline__ float rsqrt_of(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsqrt_of(double x) {
+  double y = (double)rsqrtf((float)x);
+  const double h = 0.5 * x;
+  y = y * fma(-h * y, y, 1.5);
+  return y * fma(-h * y, y, 1.5);
+}
+
 // Recompression, step 2b: for every sibling pair (a, b) with a = list[blockIdx.x], the
-// core C (step 2a), one-sided Jacobi C W = P Sigma, truncation, and the small transforms
-//   T_a = (P Sigma)[:, kept] (qa x k'),  T_b = conj(W)[:, kept] (qb x k').
-// qa, qb <= QCAP, the largest core of the plan (setup_alloc).
+// truncated SVD of the core C (step 2a), as the small transforms
+//   T_b = conj(P) Sigma^(1/2) (qb x k'),  T_a = C P Sigma^(-1/2) (qa x k'),
+// P the right singular vectors kept: T_a T_b^t = C P P^*, the projection of C.
+//
+// 1. Gram-Schmidt with column pivoting, C = Q R, stopped when every remaining column is
+//    below the threshold thr (relative to the largest): the block's numerical rank is a third
+//    to a half of the core's size.  Each warp picks the pivot from the column norms (no
+//    broadcast), takes its columns' inner products with the pivot column, updates them and
+//    leaves their new norms: one barrier a step.  Q is not kept: row k of R, conjugated, goes
+//    into the storage of the k-th pivot column.
+// 2. One-sided Jacobi on L = R^* (qb x kq): L W = P Sigma.  The rows of R come graded, so few
+//    sweeps do.  No rotations are accumulated: T_a takes the product with C instead, and as
+//    a projection of C it does not depend on how exactly the rotations were unitary (their
+//    angles come from FP32 reciprocal square roots in both precisions).
+// What bounds it is the latency of kq - 1 barriers a sweep (complex64) or the FP64 units of
+// one SM (complex128).  Jacobi on the whole core, with the rotations accumulated, took 683 us
+// a layer at n = 511 in complex64 and 1586 us at n = 150 in complex128.
 template <typename R>
-__global__ void svd_jacobi(Geo g, double eps, const Cx<R>* __restrict__ Cb, const int* __restrict__ qcols,
-                           const int* __restrict__ G_rank, Cx<R>* __restrict__ Wb, Cx<R>* __restrict__ Tx,
-                           int* __restrict__ newrank, int smem_entries, R frz) {
+__global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R>* __restrict__ Cb,
+                                                   const int* __restrict__ qcols, Cx<R>* __restrict__ Tx,
+                                                   int* __restrict__ newrank, int smem_entries, R thr) {
   extern __shared__ __align__(16) unsigned char sm[];
   const int a = g.list[blockIdx.x], b = a + 1, t = a >> 1;
   const int qa = qcols[a], qb = qcols[b];
-  // C (column-major qa x qb, ld qa) and, when both fit in the shared-memory plan, the
-  // accumulated rotations W (column-major qb x qb, ld qb); otherwise W stays in Wb
-  const bool w_shared = (long long)qa * qb + (long long)qb * qb <= smem_entries;
-  Cx<R>* C = reinterpret_cast<Cx<R>*>(sm);
-  Cx<R>* Wm = w_shared ? C + (size_t)qa * qb : Wb + (long long)t * g.QCAP * g.QCAP;
-  const int ldw = w_shared ? qb : g.QCAP;
-  R* sig = reinterpret_cast<R*>(reinterpret_cast<Cx<R>*>(sm) + smem_entries);   // [QCAP + 1]
-  int* order = reinterpret_cast<int*>(sig + g.QCAP + 1);                          // [QCAP]
+  const int ld = max(qa, qb);
+  Cx<R>* C = reinterpret_cast<Cx<R>*>(sm);                        // column j at j ld
+  Cx<R>* rbuf = C + smem_entries;                                  // [2][QCAP] a row of R
+  R* nrm = reinterpret_cast<R*>(rbuf + 2 * g.QCAP);                // [2][QCAP] squared column norms
+  R* sig = nrm + 2 * g.QCAP;                                       // [QCAP + 1]
+  int* slot = reinterpret_cast<int*>(sig + g.QCAP + 1);            // [QCAP] column storage of row k
+  int* order = slot + g.QCAP;                                      // [QCAP]
   __shared__ int s_rot, s_keep;
-  __shared__ R s_scale;
   if (qa == 0 || qb == 0) {
     if (threadIdx.x == 0) { newrank[a] = 0; newrank[b] = 0; }
     return;
   }
-  {
-    const Cx<R>* Cg = Cb + (long long)t * g.QCAP * g.QCAP;     // the core from step 2a
-    for (int e = threadIdx.x; e < qa * qb; e += blockDim.x) C[e] = Cg[e];
-  }
-  for (int e = threadIdx.x; e < qb * qb; e += blockDim.x) {
-    const int i = e % qb, j = e / qb;
-    Wm[(long long)j * ldw + i] = Cx<R>(i == j ? 1 : 0, 0);
-  }
-  __syncthreads();
-  // normalise by the largest column norm
+  const Cx<R>* Cg = Cb + (long long)t * g.QCAP * g.QCAP;           // the core from step 2a
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int j = warp; j < qb; j += nw) {
     R acc = 0;
-    for (int i = lane; i < qa; i += 32) acc += abs2(C[(long long)j * qa + i]);
+    for (int i = lane; i < qa; i += 32) {
+      const Cx<R> v = Cg[(long long)j * qa + i];
+      C[j * ld + i] = v;
+      acc += abs2(v);
+    }
     acc = warp_sum_r(acc);
-    if (lane == 0) sig[j] = acc;
+    if (lane == 0) nrm[j] = acc;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    R mx = 0;
-    for (int j = 0; j < qb; ++j) mx = fmax(mx, sig[j]);
-    s_scale = sqrt(mx);
-  }
-  __syncthreads();
-  const R scale = s_scale;
-  if (!(scale > 0)) {
+  // normalise by the largest column norm
+  R mx = 0;
+  for (int j = lane; j < qb; j += 32) mx = fmax(mx, nrm[j]);
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (!(mx > 0)) {
     if (threadIdx.x == 0) { newrank[a] = 0; newrank[b] = 0; }
     return;
   }
-  const R iscale = R(1) / scale;
-  for (int e = threadIdx.x; e < qa * qb; e += blockDim.x) C[e] = iscale * C[e];
+  const R scale = sqrt(mx), iscale = R(1) / scale;
   __syncthreads();
-  const int me = qb + (qb & 1);               // even number of positions (one dummy if odd)
+  for (int j = warp; j < qb; j += nw) {
+    for (int i = lane; i < qa; i += 32) C[j * ld + i] = iscale * C[j * ld + i];
+    if (lane == 0) nrm[j] = iscale * iscale * nrm[j];
+  }
+  __syncthreads();
+  // ---- 1. pivoted Gram-Schmidt -----------------------------------------------------------
+  int kq = 0;
+  const int kmax = min(qa, qb);
+  for (; kq < kmax; ++kq) {
+    const R* nr = nrm + (kq & 1) * g.QCAP;
+    R* nx = nrm + ((kq & 1) ^ 1) * g.QCAP;
+    Cx<R>* rk = rbuf + (kq & 1) * g.QCAP;
+    R best = R(-1);
+    int p = 0;
+    for (int j = lane; j < qb; j += 32)
+      if (nr[j] > best) { best = nr[j]; p = j; }
+    for (int o = 16; o > 0; o >>= 1) {
+      const R ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int op = __shfl_xor_sync(0xffffffffu, p, o);
+      if (ob > best || (ob == best && op < p)) { best = ob; p = op; }
+    }
+    if (!(best > thr)) break;
+    const R rs = rsqrt_of(best), ib = rcp_of(best);
+    const Cx<R>* cp = C + p * ld;
+    for (int j = warp; j < qb; j += nw) {
+      if (j == p || nr[j] < 0) {
+        if (lane == 0) {
+          nx[j] = R(-1);
+          rk[j] = Cx<R>(j == p ? best * rs : R(0), R(0));
+        }
+        continue;
+      }
+      Cx<R>* cj = C + j * ld;
+      Cx<R> d(0, 0);
+      for (int i = lane; i < qa; i += 32) cfma_conj(d, cp[i], cj[i]);
+      for (int o = 16; o > 0; o >>= 1) d += shfl_xor(d, o);
+      const Cx<R> be = -(ib * d);
+      R acc = 0;
+      for (int i = lane; i < qa; i += 32) {
+        Cx<R> v = cj[i];
+        cfma(v, be, cp[i]);
+        cj[i] = v;
+        acc = fma(v.re, v.re, fma(v.im, v.im, acc));
+      }
+      acc = warp_sum_r(acc);
+      if (lane == 0) {
+        nx[j] = acc;
+        rk[j] = rs * conj(d);
+      }
+    }
+    // the row of the step before into the storage of its pivot column (read by nobody now)
+    if (kq > 0 && warp == nw - 1) {
+      const Cx<R>* rp = rbuf + ((kq & 1) ^ 1) * g.QCAP;
+      Cx<R>* dst = C + slot[kq - 1] * ld;
+      for (int j = lane; j < qb; j += 32) dst[j] = rp[j];
+    }
+    if (threadIdx.x == 0) slot[kq] = p;
+    __syncthreads();
+  }
+  if (kq > 0) {
+    const Cx<R>* rp = rbuf + ((kq & 1) ^ 1) * g.QCAP;
+    Cx<R>* dst = C + slot[kq - 1] * ld;
+    for (int j = threadIdx.x; j < qb; j += blockDim.x) dst[j] = rp[j];
+  }
+  // ---- 2. one-sided Jacobi on the kq columns (length qb) of L ------------------------------
+  const int me = kq + (kq & 1);               // even number of positions (one dummy if odd)
   // one group of GW lanes per column pair: whole warps while there are at most as many
   // pairs as warps, half warps beyond (every pair of a round in one pass)
   const int GW = (me / 2 <= nw) ? 32 : 16;
   const int gpw = 32 / GW;                    // groups per warp
   for (int sweep = 0; sweep < 40; ++sweep) {
+    __syncthreads();
     if (threadIdx.x == 0) s_rot = 0;
     // squared column norms, exact at the start of every sweep and carried through its
     // rounds by the rotation's own update (a rotation by tan t of the pair (p, q) with
     // <p, q> = g maps |p|^2 to |p|^2 - t |g| and |q|^2 to |q|^2 + t |g|), so a pair's test
     // needs only the inner product
-    for (int j = warp; j < qb; j += nw) {
+    for (int j = warp; j < kq; j += nw) {
+      const Cx<R>* cj = C + slot[j] * ld;
       R acc = 0;
-      for (int i = lane; i < qa; i += 32) acc += abs2(C[(long long)j * qa + i]);
+      for (int i = lane; i < qb; i += 32) acc += abs2(cj[i]);
       acc = warp_sum_r(acc);
       if (lane == 0) sig[j] = acc;
     }
@@ -808,89 +905,112 @@ __global__ void svd_jacobi(Geo g, double eps, const Cx<R>* __restrict__ Cb, cons
       // the loop bound is uniform over the warp, so every lane reaches every shuffle
       for (int pb = warp * gpw; pb < me / 2; pb += nw * gpw) {
         const int pr = pb + lane / GW, gl = lane % GW;
-        int p0 = pr, p1 = me - 1 - pr;
-        int ip = p0 == 0 ? 0 : ((p0 - 1 + round) % (me - 1)) + 1;
-        int iq = ((p1 - 1 + round) % (me - 1)) + 1;
-        const bool live = pr < me / 2 && ip < qb && iq < qb;
-        if (ip > iq) { int tmp = ip; ip = iq; iq = tmp; }
-        Cx<R>* cp = C + (long long)(live ? ip : 0) * qa;
-        Cx<R>* cq = C + (long long)(live ? iq : 0) * qa;
-        const R al = live ? sig[ip] : R(0), be = live ? sig[iq] : R(0);
+        const int p0 = pr, p1 = me - 1 - pr;
+        int ip = p0 == 0 ? 0 : p0 - 1 + round, iq = p1 - 1 + round;
+        if (p0 != 0) ip = (ip >= me - 1 ? ip - (me - 1) : ip) + 1;
+        iq = (iq >= me - 1 ? iq - (me - 1) : iq) + 1;
+        const bool live = pr < me / 2 && ip < kq && iq < kq;
+        if (ip > iq) { const int tmp = ip; ip = iq; iq = tmp; }
+        Cx<R>* cp = C + (live ? slot[ip] : 0) * ld;
+        Cx<R>* cq = C + (live ? slot[iq] : 0) * ld;
+        const R al = live ? sig[ip] : R(1), be = live ? sig[iq] : R(1);
         Cx<R> ga(0, 0);
         if (live)
-          for (int i = gl; i < qa; i += GW) cfma_conj(ga, cp[i], cq[i]);
+          for (int i = gl; i < qb; i += GW) cfma_conj(ga, cp[i], cq[i]);
         ga = group_sum(ga, GW);
-        const R ag = sqrt(abs2(ga));
-        // a column whose squared norm is below frz (relative to the largest, 1 after the
-        // normalisation) stays below it under every rotation and is truncated in the end:
-        // it is left alone, so the sweeps stop once the significant columns are orthogonal
-        const bool rot = live && al >= frz && be >= frz && ag > Tiny<R>::jac * sqrt(al) * sqrt(be);
+        // g = <p, q> / (|p| |q|): the angle's cotangent 2 z = (|q|^2 - |p|^2) / |<p, q>|
+        const float ra = rsqrtf((float)al), rb = rsqrtf((float)be);
+        const R s = R(ra) * R(rb);
+        const Cx<R> gn = s * ga;
+        const float gg = (float)abs2(gn);
+        const bool rot = live && al >= thr && be >= thr && gg > (float)(Tiny<R>::jac * Tiny<R>::jac);
         if (rot) {
           if (gl == 0) s_rot = 1;
-          const Cx<R> e(ga.re / ag, ga.im / ag);
-          const R z = (be - al) / (R(2) * ag);
-          const R tt = fabs(z) < R(1e18) ? (z >= 0 ? R(1) : R(-1)) / (fabs(z) + sqrt(R(1) + z * z)) : R(0.5) / z;
-          const R cs = R(1) / sqrt(R(1) + tt * tt), sn = tt * cs;
-          const Cx<R> snc = sn * conj(e), sne = sn * e;
+          const float ig = rsqrtf(gg);
+          const float z = 0.5f * (float)((be - al) * s) * ig;
+          // (z reaches 1e29 in complex128, where its square would overflow)
+          const float za = fabsf(z), tt = copysignf(1.0f, z) / (za + (za < 1e9f ? sqrtf(fmaf(z, z, 1.0f)) : za));
+          const R tr = (R)tt;
+          const R cs = rsqrt_of(fma(tr, tr, R(1))), sn = tr * cs;
+          R igr = (R)ig;
+          if (sizeof(R) == 8) igr = igr * fma(R(-0.5) * abs2(gn) * igr, igr, R(1.5));
+          const Cx<R> sne = (sn * igr) * gn, snc = conj(sne);
           if (gl == 0) {
-            sig[ip] = fmax(R(0), al - tt * ag);
-            sig[iq] = be + tt * ag;
+            const R ag = tr * (abs2(gn) * igr * rcp_of(s));
+            sig[ip] = fmax(R(0), al - ag);
+            sig[iq] = be + ag;
           }
-          for (int i = gl; i < qa; i += GW) {
-            const Cx<R> x = cp[i], y = cq[i];
-            cp[i] = cs * x - snc * y;
-            cq[i] = sne * x + cs * y;
-          }
-          Cx<R>* wp = Wm + (long long)ip * ldw;
-          Cx<R>* wq = Wm + (long long)iq * ldw;
           for (int i = gl; i < qb; i += GW) {
-            const Cx<R> x = wp[i], y = wq[i];
-            wp[i] = cs * x - snc * y;
-            wq[i] = sne * x + cs * y;
+            const Cx<R> x = cp[i], y = cq[i];
+            Cx<R> nx = cs * x, ny = cs * y;
+            cfma(nx, -snc, y);
+            cfma(ny, sne, x);
+            cp[i] = nx;
+            cq[i] = ny;
           }
         }
       }
       __syncthreads();
     }
     if (s_rot == 0) break;
-    __syncthreads();
   }
   // singular values, ordering, truncation
-  for (int j = warp; j < qb; j += nw) {
+  for (int j = warp; j < kq; j += nw) {
+    const Cx<R>* cj = C + slot[j] * ld;
     R acc = 0;
-    for (int i = lane; i < qa; i += 32) acc += abs2(C[(long long)j * qa + i]);
+    for (int i = lane; i < qb; i += 32) acc += abs2(cj[i]);
     acc = warp_sum_r(acc);
     if (lane == 0) sig[j] = sqrt(acc);
   }
+  if (threadIdx.x == 0) s_keep = 0;
   __syncthreads();
-  for (int j = threadIdx.x; j < qb; j += blockDim.x) {
+  for (int j = threadIdx.x; j < kq; j += blockDim.x) {
     int rk = 0;
-    for (int l = 0; l < qb; ++l) rk += (sig[l] > sig[j] || (sig[l] == sig[j] && l < j)) ? 1 : 0;
+    R smax = 0;
+    for (int l = 0; l < kq; ++l) {
+      rk += (sig[l] > sig[j] || (sig[l] == sig[j] && l < j)) ? 1 : 0;
+      smax = fmax(smax, sig[l]);
+    }
     order[rk] = j;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const R smax = sig[order[0]];
-    int keep = 0;
-    while (keep < qb && keep < g.r_max && smax > 0 && sig[order[keep]] > R(eps) * smax && sig[order[keep]] > 0) ++keep;
-    s_keep = keep;
-    newrank[a] = keep;
-    newrank[b] = keep;
+    // (a column below thr may have been left unrotated: only those clear of it are orthogonal
+    // to the others; at eps below the rounding noise this is what ends the expansion)
+    if (rk < g.r_max && sig[j] > R(eps) * smax && sig[j] * sig[j] > R(4) * thr) atomicMax(&s_keep, rk + 1);
   }
   __syncthreads();
   const int keep = s_keep;
+  if (threadIdx.x == 0) {
+    newrank[a] = keep;
+    newrank[b] = keep;
+  }
   Cx<R>* Ta = Tx + (long long)a * g.QCAP * g.r_max;   // column-major (ld QCAP)
   Cx<R>* Tb = Tx + (long long)b * g.QCAP * g.r_max;
-  // balanced split: T_a = P_j sigma_j^(1/2), T_b = conj(W_j) sigma_j^(1/2)
-  for (int e = threadIdx.x; e < qa * keep; e += blockDim.x) {
-    const int i = e % qa, j = e / qa;
-    const R f = sqrt(scale / sig[order[j]]);
-    Ta[(long long)j * g.QCAP + i] = f * C[(long long)order[j] * qa + i];
+  // balanced split, four columns of T_a per thread and pass over a row of C
+  for (int e = threadIdx.x; e < qa * ((keep + 3) / 4); e += blockDim.x) {
+    const int i = e % qa, j0 = (e / qa) * 4;
+    Cx<R> acc[4];
+    const Cx<R>* l[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      acc[u] = Cx<R>(0, 0);
+      l[u] = C + slot[order[min(j0 + u, keep - 1)]] * ld;
+    }
+#pragma unroll 4
+    for (int j = 0; j < qb; ++j) {
+      const Cx<R> c = Cg[(long long)j * qa + i];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cfma(acc[u], c, l[u][j]);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j0 + u < keep) {
+        const R sg = sig[order[j0 + u]];
+        Ta[(long long)(j0 + u) * g.QCAP + i] = (R(1) / (sg * sqrt(scale * sg))) * acc[u];
+      }
   }
   for (int e = threadIdx.x; e < qb * keep; e += blockDim.x) {
     const int i = e % qb, j = e / qb;
-    const R f = sqrt(scale * sig[order[j]]);
-    Tb[(long long)j * g.QCAP + i] = f * conj(Wm[(long long)order[j] * ldw + i]);
+    const R f = sqrt(scale / sig[order[j]]);
+    Tb[(long long)j * g.QCAP + i] = f * conj(C[slot[order[j]] * ld + i]);
   }
 }
 
@@ -991,7 +1111,7 @@ __global__ void store_layer(Geo g, const Cx<R>* __restrict__ G_leaf, const Cx<R>
 
 // ---------------------------------------------------------------------------------------
 struct SetupWork {
-  int KCAP = 0, WCAP = 0, QCAP = 0;
+  int KCAP = 0, WCAP = 0, QCAP = 0, dense_max = 0;
   long long gfo_total = 0;   // entries of one G factor buffer
   std::vector<long long> sfo, gfo, qro, rbo;
   std::vector<int> rowleaf, cap;
@@ -1011,7 +1131,7 @@ struct SetupWork {
   int* d_lists = nullptr;
   void *S_leaf = nullptr, *S_F = nullptr, *G_leaf = nullptr, *G_F = nullptr, *G_F2 = nullptr;
   void *Y = nullptr, *W = nullptr, *Qr = nullptr, *PQ = nullptr, *M = nullptr, *Rb = nullptr;
-  void *Wb = nullptr, *Tx = nullptr, *Cb = nullptr;
+  void *Tx = nullptr, *Cb = nullptr;
   int *S_rank = nullptr, *G_rank = nullptr, *qcols = nullptr, *qmode = nullptr, *newrank = nullptr;
 };
 
@@ -1019,7 +1139,7 @@ void hsw_setup_free(hsweep_s* h) {
   if (!h->sw) return;
   SetupWork* w = h->sw;
   void* ptrs[] = {w->d_sfo, w->d_gfo, w->d_qro, w->d_rbo, w->d_rowleaf, w->d_cap, w->d_lists, w->S_leaf, w->S_F,
-                  w->G_leaf, w->G_F, w->G_F2, w->Y, w->W, w->Qr, w->PQ, w->M, w->Rb, w->Wb, w->Tx, w->Cb, w->S_rank,
+                  w->G_leaf, w->G_F, w->G_F2, w->Y, w->W, w->Qr, w->PQ, w->M, w->Rb, w->Tx, w->Cb, w->S_rank,
                   w->G_rank, w->qcols, w->qmode, w->newrank};
   for (void* p : ptrs) hsw_release(h, p);
   delete w;
@@ -1040,13 +1160,16 @@ static int setup_alloc(hsweep_s* h) {
   // min(rows, depth x KCAP) (every depth step above appends at most KCAP columns), fits the
   // Jacobi SVD's shared memory; its blocks are recompressed once per layer.  The other
   // depths are recompressed after every depth step (at most WCAP columns).
-  const size_t smem_cap = 227 * 1024 - 4096;
+  const size_t smem_cap = 227 * 1024 - 8192;
   const int qlim = (int)std::sqrt((double)(smem_cap / es));
   auto deferred_core = [&](int d) { return std::min(h->tree.maxsz(d), d * w->KCAP); };
   auto small_depth = [&](int d) { return deferred_core(d) <= qlim; };
   w->QCAP = w->WCAP;
-  for (int d = 1; d <= L; ++d)
+  w->dense_max = es == sizeof(c64) ? kDenseRows : 0;
+  for (int d = 1; d <= L; ++d) {
     if (small_depth(d)) w->QCAP = std::max(w->QCAP, deferred_core(d));
+    if (h->tree.maxsz(d) <= w->dense_max) w->QCAP = std::max(w->QCAP, h->tree.maxsz(d));
+  }
   w->sfo.assign(nn, 0);
   w->gfo.assign(nn, 0);
   w->qro.assign(nn, 0);
@@ -1060,7 +1183,7 @@ static int setup_alloc(hsweep_s* h) {
     w->sfo[v] = so; so += (long long)sv * w->KCAP;
     w->gfo[v] = go; go += (long long)sv * cv;
     w->qro[v] = qo; qo += (long long)cv * w->KCAP;
-    w->rbo[v] = ro; ro += (long long)std::min(sv, cv) * cv;
+    w->rbo[v] = ro; ro += (long long)(sv <= w->dense_max ? sv : std::min(sv, cv)) * cv;
   }
   // recompression lists
   w->lists.clear();
@@ -1119,7 +1242,6 @@ static int setup_alloc(hsweep_s* h) {
   A(w->PQ, ntau * 2 * w->KCAP * w->KCAP * es);
   A(w->M, ntau * 4 * w->KCAP * w->KCAP * es);
   A(w->Rb, std::max(ro, 1LL) * es);
-  A(w->Wb, (long long)nn * w->QCAP * w->QCAP * es);
   A(w->Tx, (long long)nn * w->QCAP * h->r_max * es);
   A(w->Cb, (long long)(nn / 2) * w->QCAP * w->QCAP * es);
   A(w->S_rank, nn * sizeof(int));
@@ -1149,7 +1271,7 @@ static int factor_impl(hsweep_s* h) {
   const size_t es = sizeof(Cx<R>);
   Geo g;
   g.n = h->n; g.L = h->L; g.leaf = h->leaf; g.nnodes = h->nnodes; g.r_max = h->r_max;
-  g.KCAP = w->KCAP; g.WCAP = w->WCAP; g.QCAP = w->QCAP;
+  g.KCAP = w->KCAP; g.WCAP = w->WCAP; g.QCAP = w->QCAP; g.dense_max = w->dense_max;
   g.lo = h->d_lo; g.sz = h->d_sz; g.rowleaf = w->d_rowleaf; g.sfo = w->d_sfo; g.gfo = w->d_gfo;
   g.cap = w->d_cap; g.qro = w->d_qro; g.rbo = w->d_rbo; g.list = w->d_lists;
   cudaStream_t st = h->stream;
@@ -1165,7 +1287,6 @@ static int factor_impl(hsweep_s* h) {
   Cx<R>* PQ = (Cx<R>*)w->PQ;
   Cx<R>* M = (Cx<R>*)w->M;
   Cx<R>* Rb = (Cx<R>*)w->Rb;
-  Cx<R>* Wb = (Cx<R>*)w->Wb;
   Cx<R>* Tx = (Cx<R>*)w->Tx;
   const int L = h->L, nn = h->nnodes, KCAP = w->KCAP, QCAP = w->QCAP;
   const size_t core_smem = (size_t)(2 * KCAP) * (2 * KCAP) * es + 32 * sizeof(R) + (2 * KCAP + 1) * sizeof(int) + 16;
@@ -1173,11 +1294,9 @@ static int factor_impl(hsweep_s* h) {
   const size_t qr_base = ((size_t)(h->tree.maxsz(1) + QCAP) * es + 32 * sizeof(R) + 15) & ~size_t(15);
   const int qs_entries = qr_base < 226 * 1024 ? (int)((226 * 1024 - qr_base) / es) : 0;
   const size_t qr_smem = qr_base + (size_t)qs_entries * es;
-  // the Jacobi SVD's shared memory: C and, where it fits, the rotations W (up to 2 QCAP^2
-  // entries; for large cores W stays in global memory)
-  const size_t svd_tail = (size_t)(QCAP + 1) * sizeof(R) + (size_t)QCAP * sizeof(int) + 64;
-  // (1 KB of the 227 KB per block stays free for the kernel's static shared variables)
-  const int svd_entries = (int)std::min<size_t>((size_t)2 * QCAP * QCAP, (226 * 1024 - svd_tail) / es);
+  // the SVD's shared memory: C, two rows of R, norms, singular values and index tables
+  const size_t svd_tail = (size_t)2 * QCAP * es + (size_t)(3 * QCAP + 1) * sizeof(R) + (size_t)2 * QCAP * sizeof(int) + 16;
+  const int svd_entries = QCAP * QCAP;
   const size_t svd_smem = (size_t)svd_entries * es + svd_tail;
   // one shared-memory carveout for every kernel of the layer loop, so that consecutive
   // launches do not reconfigure the SMs' L1/shared split
@@ -1193,7 +1312,7 @@ static int factor_impl(hsweep_s* h) {
   HSW_CUDA(cudaFuncSetAttribute(core_inverse<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)core_smem));
   HSW_CUDA(cudaFuncSetAttribute(qr_cgs2<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qr_smem));
   HSW_CUDA(cudaFuncSetAttribute(svd_jacobi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)svd_smem));
-  if (core_smem > 227 * 1024 || qr_smem > 227 * 1024 || svd_smem > 227 * 1024 || svd_entries < QCAP * QCAP)
+  if (core_smem > 227 * 1024 || qr_smem > 227 * 1024 || svd_smem > 227 * 1024)
     return HSWEEP_ERR_ARG;
 
   // Autotuning of the core products (step 2a), complex64 only: on layer tune_m, the first
@@ -1201,8 +1320,9 @@ static int factor_impl(hsweep_s* h) {
   // recompression) runs both kernels, timed with CUDA events, and the faster one serves that
   // kind of launch from then on; before it, and in complex128, the CUDA-core kernel runs.
   const int tune_m = h->n / 2;
-  // Jacobi: columns below a tenth of the truncation threshold (squared, relative) are frozen
-  const R frz = (R)std::max((double)Tiny<R>::neg, 0.01 * h->eps_H * h->eps_H);
+  // SVD: columns below a fraction of the truncation threshold (squared, relative) are left out:
+  // a quarter in complex64 (rounding noise lies just below), a twentieth in complex128
+  const R thr = (R)std::max((double)Tiny<R>::neg, (sizeof(R) == 4 ? 0.0625 : 0.0025) * h->eps_H * h->eps_H);
   const int core_tiles = ((QCAP + kCT - 1) / kCT) * ((QCAP + kCT - 1) / kCT);
   const int gemm_tiles = ((h->tree.maxsz(1) + kCT - 1) / kCT) * ((h->r_max + kCT - 1) / kCT);
   Cx<R>* Cb = (Cx<R>*)w->Cb;
@@ -1259,8 +1379,7 @@ static int factor_impl(hsweep_s* h) {
     gp.list = w->d_lists + pair_off;
     int rc = core_product(gp, np_list, kind);
     if (rc) return rc;
-    svd_jacobi<R><<<np_list, 1024, svd_smem, st>>>(gp, h->eps_H, Cb, w->qcols, w->G_rank, Wb, Tx, w->newrank,
-                                                   svd_entries, frz);
+    svd_jacobi<R><<<np_list, 1024, svd_smem, st>>>(gp, h->eps_H, Cb, w->qcols, Tx, w->newrank, svd_entries, thr);
     recompress_gemm<R><<<dim3(gemm_tiles, nn_list), 256, 0, st>>>(gl, G_F, w->qcols, w->qmode, Tx, w->newrank, G_F2);
     recompress_copy<R><<<nn_list, kBlk, 0, st>>>(gl, G_F2, w->newrank, G_F, w->G_rank);
     h->nlaunch += 4;
