@@ -38,7 +38,33 @@ template <typename R> __host__ __device__ __forceinline__ void cfma_conj(Cx<R>& 
   acc.re = fma(a.re, b.re, fma(a.im, b.im, acc.re));
   acc.im = fma(a.re, b.im, fma(-a.im, b.re, acc.im));
 }
+// ---- double <-> float by integer arithmetic ------------------------------------------------
+// The FP64 unit of this GPU (half a lane a clock and scheduler) also serves the conversions:
+// in the sweeps, those of r and z took longer than the multiply-adds.  Values in FP32's normal
+// range (and zeros) are converted with integer operations, to the same bits.
+__device__ __forceinline__ float to_float(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+  if (e - 897u <= 253u) {               // 2^-126 <= |v| < 2^128: round to nearest even
+    unsigned b = __funnelshift_l(lo, hi, 3) - 0xc0000000u;     // exponent bias 1023 -> 127
+    b += ((lo & 0x1fffffffu) + 0x0fffffffu + (b & 1u)) >> 29;
+    return __uint_as_float(b | sign);
+  }
+  if (e < 873u) return __uint_as_float(sign);                  // below half of the least subnormal
+  return (float)v;
+}
+__device__ __forceinline__ double to_double(float v) {
+  const unsigned b = __float_as_uint(v);
+  if (((b >> 23) & 0xffu) - 1u <= 253u)
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+  if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
+  return (double)v;
+}
 template <typename To, typename From> __host__ __device__ __forceinline__ Cx<To> cvt(Cx<From> a) {
+#ifdef __CUDA_ARCH__
+  if constexpr (sizeof(To) == 4 && sizeof(From) == 8) return Cx<To>(to_float(a.re), to_float(a.im));
+  if constexpr (sizeof(To) == 8 && sizeof(From) == 4) return Cx<To>(to_double(a.re), to_double(a.im));
+#endif
   return Cx<To>(To(a.re), To(a.im));
 }
 // 1 / a
@@ -57,6 +83,36 @@ template <typename R> __host__ __device__ __forceinline__ Cx<R> csqrt(Cx<R> a) {
 
 template <typename R> __device__ __forceinline__ Cx<R> shfl_xor(Cx<R> v, int off) {
   return Cx<R>(__shfl_xor_sync(0xffffffffu, v.re, off), __shfl_xor_sync(0xffffffffu, v.im, off));
+}
+
+// Sum of v[0..G) over the NL lanes that differ in the lane bits UNIT, 2 UNIT, ... NL/2 UNIT,
+// scattered: each step a lane keeps half of its right-hand sides and hands the other half to
+// its partner, so a lane ends with CNT = max(1, G / NL) sums, right-hand sides g .. g+CNT-1.
+// With fewer right-hand sides than lanes the last steps are plain sums (every lane of such a
+// group holds the same value; `first` marks one of them).
+template <typename R, int G, int NL, int UNIT>
+__device__ __forceinline__ void scatter_sum(Cx<R> (&v)[G], int lane, int& g, bool& first) {
+  g = 0;
+  first = true;
+  int cnt = G;
+#pragma unroll
+  for (int o = NL / 2; o > 0; o >>= 1) {
+    const bool up = (lane & (o * UNIT)) != 0;
+    if (cnt > 1) {
+      cnt >>= 1;
+#pragma unroll
+      for (int j = 0; j < G / 2; ++j)
+        if (j < cnt) {
+          const Cx<R> send = up ? v[j] : v[j + cnt];
+          const Cx<R> keep = up ? v[j + cnt] : v[j];
+          v[j] = keep + shfl_xor(send, o * UNIT);
+        }
+      if (up) g += cnt;
+    } else {
+      v[0] += shfl_xor(v[0], o * UNIT);
+      first = first && !up;
+    }
+  }
 }
 
 // L2-only loads/stores for data exchanged between CTAs of one sweep team.

@@ -47,11 +47,15 @@ template <> struct Tiny<double> {
   static constexpr double jac = 1e-15;    // Jacobi: orthogonality tolerance (about 8 ulp)
   static constexpr double neg = 1e-28;    // Jacobi: squared norm of a rounding-noise column
                                           // (normalised: below 1e-14 of the largest column)
+  static constexpr float quad = 1e-16f;   // Jacobi: squared cosine from which one more sweep
+                                          // is needed (the convergence is quadratic: a sweep
+                                          // whose cosines were below 1e-8 leaves 1e-16)
 };
 template <> struct Tiny<float> {
   static constexpr float dep = 2e-6f;
   static constexpr float jac = 4e-7f;     // about 7 ulp: tighter only rotates rounding noise
   static constexpr float neg = 1e-14f;    // below 1e-7 of the largest column: FP32 noise
+  static constexpr float quad = 1e-8f;
 };
 
 template <typename R> __device__ __forceinline__ Cx<R> warp_sum(Cx<R> v) {
@@ -75,8 +79,69 @@ template <typename R> __device__ R block_sum(R v, R* red) {
   return t;
 }
 
+// Reciprocal and reciprocal square root, in complex128 by two Newton steps from the FP32
+// value (a handful of FP64 operations where the division and square root routines take
+// dozens: a warp's FP64 instruction occupies its scheduler for about 64 clocks here)
+__device__ __forceinline__ float rcp_of(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rcp_of(double x) {
+  // for x well inside FP32's range
+  double y = (double)(1.0f / (float)x);
+  y = y * fma(-x, y, 2.0);
+  return y * fma(-x, y, 2.0);
+}
+__device__ __forceinline__ float rsqrt_of(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsqrt_of(double x) {
+  double y = (double)rsqrtf((float)x);
+  const double h = 0.5 * x;
+  y = y * fma(-h * y, y, 1.5);
+  return y * fma(-h * y, y, 1.5);
+}
+
+// the same for any positive normal x: its exponent is taken out first
+__device__ __forceinline__ float rcp_any(float x) { return 1.0f / x; }
+__device__ __forceinline__ float rsqrt_any(float x) { return 1.0f / sqrtf(x); }
+__device__ __forceinline__ double rcp_any(double x) {
+  const int e = ((__double2hiint(x) >> 20) & 0x7ff) - 1023;
+  const double s = __hiloint2double((1023 - e) << 20, 0);       // 2^-e
+  return rcp_of(x * s) * s;
+}
+__device__ __forceinline__ double rsqrt_any(double x) {
+  const int q = (((__double2hiint(x) >> 20) & 0x7ff) - 1023) >> 1;
+  const double s = __hiloint2double((1023 - q) << 20, 0);       // 2^-q
+  return rsqrt_of(x * s * s) * s;
+}
+// 1 / a, by the Newton reciprocal where |a|^2 is well inside FP32's range
+__device__ __forceinline__ c128 cinv_fast(c128 a) {
+  const double d = abs2(a);
+  const double s = (d > 1e-30 && d < 1e30) ? rcp_of(d) : 1.0 / d;
+  return c128(a.re * s, -a.im * s);
+}
+
+// Programmatic dependent launch: a kernel lets its successor's CTAs start (they wait here for
+// its end), so that the launch latency between the layer's forty short kernels is hidden
+// (about 1 us each; no effect on kernels launched without the attribute).
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... KA, typename... A>
+static cudaError_t pdl_launch(void (*kern)(KA...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = dim3(block);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kern, KA(args)...);
+}
+
 struct Geo {          // tree and buffer geometry passed by value to every kernel
   int n, L, leaf, nnodes, r_max, KCAP, WCAP, QCAP;
+  int cap_max;             // the largest cap
   int dense_max;           // blocks of at most so many rows take the dense path at any rank
   const int* lo;
   const int* sz;
@@ -92,123 +157,133 @@ struct Geo {          // tree and buffer geometry passed by value to every kerne
 __device__ __forceinline__ int depth_of(int v) { return 31 - __clz(v); }
 
 // ---------------------------------------------------------------------------------
-// S~_m: leaves A_mm[leaf] - D T_leaf D, factors [-D F_a, a e_last] / [D F_b, e_first].
+// S~_m, one launch: blocks 0 .. nleaves - 1 (of slice 0) form a leaf A_mm[leaf] - D T_leaf D
+// and invert it, FP64 Gauss-Jordan with partial pivoting in both precisions (a serial chain
+// of FP64 instructions, 15 us, with the factors beside it); the others form the factors
+// [-D F_a, a e_last] / [D F_b, e_first] of node v = 2 + blockIdx.x - nleaves, in gridDim.y slices.
 template <typename R>
-__global__ void schur_leaves(Geo g, int m, const c128* __restrict__ diag, const c128* __restrict__ east,
-                             const c128* __restrict__ north, const Cx<R>* __restrict__ Tprev,
-                             Cx<R>* __restrict__ S_leaf) {
-  const int lam = (1 << g.L) + blockIdx.x;
-  const int lo = g.lo[lam], s = g.sz[lam], lf = g.leaf;
-  for (int e = threadIdx.x; e < lf * lf; e += blockDim.x) {
-    const int a = e % lf, b = e / lf;     // column-major: entry (a, b) at b*leaf + a
-    Cx<R> v(0, 0);
-    if (a < s && b < s) {
-      const int i = lo + a, j = lo + b;
-      c128 av(0, 0);
-      if (a == b) av = diag[(long long)m * g.n + i];
-      else if (j == i + 1) av = east[(long long)m * (g.n + 1) + j];
-      else if (i == j + 1) av = east[(long long)m * (g.n + 1) + i];
-      v = cvt<R>(av);
-      if (Tprev) {
-        Cx<R> di = cvt<R>(north[(long long)m * g.n + i]), dj = cvt<R>(north[(long long)m * g.n + j]);
-        v -= di * (Tprev[(long long)blockIdx.x * lf * lf + e] * dj);
+__global__ void __launch_bounds__(kBlk) schur_layer(Geo g, int m, const c128* __restrict__ diag,
+                                                    const c128* __restrict__ east, const c128* __restrict__ north,
+                                                    const Cx<R>* __restrict__ Tprev, const long long* __restrict__ toff,
+                                                    const int* __restrict__ trank, Cx<R>* __restrict__ S_F,
+                                                    int* __restrict__ S_rank, Cx<R>* __restrict__ G_leaf,
+                                                    int* __restrict__ G_rank, int* status) {
+  pdl_begin();
+  const int nleaves = 1 << g.L;
+  if ((int)blockIdx.x >= nleaves) {
+    const int v = 2 + (int)blockIdx.x - nleaves;
+    const int lo = g.lo[v], s = g.sz[v];
+    const bool left = (v & 1) == 0;
+    const int r0 = Tprev ? trank[v] : 0;
+    const int k = r0 + 1;
+    Cx<R>* dst = S_F + g.sfo[v];
+    const int edge = g.lo[v | 1];     // the coupling edge joins rows edge-1 and edge
+    for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < s * k; e += gridDim.y * blockDim.x) {
+      const int i = e % s, col = e / s;
+      Cx<R> val(0, 0);
+      if (col < r0) {
+        Cx<R> dv = cvt<R>(north[(long long)m * g.n + lo + i]);
+        val = dv * Tprev[toff[v] + (long long)col * s + i];
+        if (left) val = -val;
+      } else if (i == (left ? s - 1 : 0)) {
+        // the rank-one coupling a e_last e_first^t, split as sqrt(a) on both sides so
+        // that the two factors carry the same scale
+        val = cvt<R>(csqrt(east[(long long)m * (g.n + 1) + edge]));
       }
-    } else if (a == b) {
-      v = Cx<R>(1, 0);    // identity padding keeps the padded leaf invertible
+      dst[(long long)col * s + i] = val;
     }
-    S_leaf[(long long)blockIdx.x * lf * lf + e] = v;
-  }
-}
-
-template <typename R>
-__global__ void schur_factors(Geo g, int m, const c128* __restrict__ east, const c128* __restrict__ north,
-                              const Cx<R>* __restrict__ Tprev, const long long* __restrict__ toff,
-                              const int* __restrict__ trank, Cx<R>* __restrict__ S_F, int* __restrict__ S_rank) {
-  const int v = 2 + blockIdx.x;
-  const int lo = g.lo[v], s = g.sz[v];
-  const bool left = (v & 1) == 0;
-  const int r0 = Tprev ? trank[v] : 0;
-  const int k = r0 + 1;
-  Cx<R>* dst = S_F + g.sfo[v];
-  const int edge = g.lo[v | 1];     // the coupling edge joins rows edge-1 and edge
-  for (int e = threadIdx.x; e < s * k; e += blockDim.x) {
-    const int i = e % s, col = e / s;
-    Cx<R> val(0, 0);
-    if (col < r0) {
-      Cx<R> dv = cvt<R>(north[(long long)m * g.n + lo + i]);
-      val = dv * Tprev[toff[v] + (long long)col * s + i];
-      if (left) val = -val;
-    } else {
-      // the rank-one coupling a e_last e_first^t, split as sqrt(a) on both sides so
-      // that the two factors carry the same scale
-      const c128 ra = csqrt(east[(long long)m * (g.n + 1) + edge]);
-      if (left) { if (i == s - 1) val = cvt<R>(ra); }
-      else if (i == 0) val = cvt<R>(ra);
+    if (blockIdx.y == 0 && threadIdx.x == 0) {
+      S_rank[v] = k;
+      G_rank[v] = 0;
     }
-    dst[(long long)col * s + i] = val;
+    return;
   }
-  if (threadIdx.x == 0) S_rank[v] = k;
-}
-
-// ---------------------------------------------------------------------------------
-// Leaf inverses, FP64 Gauss-Jordan with partial pivoting (one block per leaf).
-template <typename R>
-__global__ void leaf_inverse(Geo g, int m, const Cx<R>* __restrict__ S_leaf, Cx<R>* __restrict__ G_leaf,
-                             int* status) {
+  if (blockIdx.y > 0) return;
   __shared__ c128 A[8][16];
   __shared__ c128 colk[8];
   __shared__ int piv;
-  const int lf = g.leaf;
-  const Cx<R>* src = S_leaf + (long long)blockIdx.x * lf * lf;
-  for (int e = threadIdx.x; e < lf * 2 * lf; e += blockDim.x) {
-    int a = e / (2 * lf), b = e % (2 * lf);
-    A[a][b] = b < lf ? cvt<double>(src[b * lf + a]) : c128(a == b - lf ? 1.0 : 0.0, 0.0);
-  }
   __shared__ double s_red[4];
+  const int lf = g.leaf, lam = nleaves + blockIdx.x, tid = threadIdx.x;
+  const int lo = g.lo[lam], s = g.sz[lam];
+  const bool act = tid < 128;         // four warps, one a scheduler (FP64)
+  for (int e = tid; e < lf * 2 * lf; e += blockDim.x) {
+    const int a = e / (2 * lf), b = e % (2 * lf);
+    c128 v(0.0, 0.0);
+    if (b >= lf) {
+      v = c128(a == b - lf ? 1.0 : 0.0, 0.0);
+    } else {
+      Cx<R> x(0, 0);
+      if (a < s && b < s) {
+        const int i = lo + a, j = lo + b;
+        c128 av(0, 0);
+        if (a == b) av = diag[(long long)m * g.n + i];
+        else if (j == i + 1) av = east[(long long)m * (g.n + 1) + j];
+        else if (i == j + 1) av = east[(long long)m * (g.n + 1) + i];
+        x = cvt<R>(av);
+        if (Tprev) {
+          const Cx<R> di = cvt<R>(north[(long long)m * g.n + i]), dj = cvt<R>(north[(long long)m * g.n + j]);
+          x -= di * (Tprev[(long long)blockIdx.x * lf * lf + b * lf + a] * dj);
+        }
+      } else if (a == b) {
+        x = Cx<R>(1, 0);    // identity padding keeps the padded leaf invertible
+      }
+      v = cvt<double>(x);
+    }
+    A[a][b] = v;
+  }
   __syncthreads();
   // the largest squared modulus of the leaf's entries (one entry per thread, then warps)
   double scale2 = 0;
-  for (int e = threadIdx.x; e < lf * lf; e += blockDim.x) scale2 = fmax(scale2, abs2(A[e / lf][e % lf]));
-  for (int o = 16; o > 0; o >>= 1) scale2 = fmax(scale2, __shfl_xor_sync(0xffffffffu, scale2, o));
-  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = scale2;
+  if (act) {
+    for (int e = tid; e < lf * lf; e += 128) scale2 = fmax(scale2, abs2(A[e / lf][e % lf]));
+    for (int o = 16; o > 0; o >>= 1) scale2 = fmax(scale2, __shfl_xor_sync(0xffffffffu, scale2, o));
+    if ((tid & 31) == 0) s_red[tid >> 5] = scale2;
+  }
   __syncthreads();
-  scale2 = 0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) scale2 = fmax(scale2, s_red[i]);
+  if (!act) return;
+  // (from here on the first 128 threads, on their own barrier)
+  auto sync = []() { asm volatile("bar.sync 1, 128;" ::: "memory"); };
+  scale2 = fmax(fmax(s_red[0], s_red[1]), fmax(s_red[2], s_red[3]));
   bool bad = false;
   for (int k = 0; k < lf; ++k) {
-    if (threadIdx.x == 0) {
-      int p = k;
-      double best = abs2(A[k][k]);
-      for (int a = k + 1; a < lf; ++a)
-        if (abs2(A[a][k]) > best) { best = abs2(A[a][k]); p = a; }
-      piv = p;
+    if (tid < 32) {
+      // the first warp's lanes compare the candidates (ties: the smallest row)
+      const int a = k + tid;
+      double best = a < lf ? abs2(A[a][k]) : -1.0;
+      int p = a < lf ? a : lf;
+      for (int o = 4; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int op = __shfl_xor_sync(0xffffffffu, p, o);
+        if (ob > best || (ob == best && op < p)) { best = ob; p = op; }
+      }
+      if (tid == 0) piv = p;
     }
-    __syncthreads();
+    sync();
     const int p = piv;
-    if (p != k && threadIdx.x < 2 * lf) {
-      c128 t = A[k][threadIdx.x]; A[k][threadIdx.x] = A[p][threadIdx.x]; A[p][threadIdx.x] = t;
+    if (p != k && tid < 2 * lf) {
+      c128 t = A[k][tid]; A[k][tid] = A[p][tid]; A[p][tid] = t;
     }
-    __syncthreads();
+    sync();
     const c128 pv = A[k][k];
     if (!(abs2(pv) > 1e-28 * scale2)) { bad = true; break; }   // |pivot| <= 1e-14 max |entry|
-    const c128 ip = cinv(pv);
-    __syncthreads();
-    if (threadIdx.x < 2 * lf) A[k][threadIdx.x] = A[k][threadIdx.x] * ip;
-    if (threadIdx.x < lf) colk[threadIdx.x] = A[threadIdx.x][k];
-    __syncthreads();
-    for (int e = threadIdx.x; e < lf * 2 * lf; e += blockDim.x) {
-      int a = e / (2 * lf), b = e % (2 * lf);
+    const c128 ip = cinv_fast(pv);
+    sync();
+    if (tid < 2 * lf) A[k][tid] = A[k][tid] * ip;
+    if (tid < lf) colk[tid] = A[tid][k];
+    sync();
+    for (int e = tid; e < lf * 2 * lf; e += 128) {
+      const int a = e / (2 * lf), b = e % (2 * lf);
       if (a != k) A[a][b] = A[a][b] - colk[a] * A[k][b];
     }
-    __syncthreads();
+    sync();
   }
   if (bad) {
-    if (threadIdx.x == 0) report_error(status, HSWEEP_ERR_NUMERIC, m);
+    if (tid == 0) report_error(status, HSWEEP_ERR_NUMERIC, m);
     return;
   }
   Cx<R>* dst = G_leaf + (long long)blockIdx.x * lf * lf;
-  for (int e = threadIdx.x; e < lf * lf; e += blockDim.x) {
-    int a = e % lf, b = e / lf;
+  for (int e = tid; e < lf * lf; e += 128) {
+    const int a = e % lf, b = e / lf;
     dst[e] = cvt<R>(A[a][lf + b]);
   }
 }
@@ -216,67 +291,98 @@ __global__ void leaf_inverse(Geo g, int m, const Cx<R>* __restrict__ S_leaf, Cx<
 // ---------------------------------------------------------------------------------
 // Y_v = G_v X_v for every node v at depth d+1 (X_v = S factor of v, k_v columns):
 // an H-matrix times a tall-skinny block, as reductions (per node u below depth d+1:
-// Qr_u = F_u^t X restricted to u) followed by an expansion.
+// Qr_u = F_u^t X restricted to u) followed by an expansion.  Both are chains of dependent
+// loads; they are cut short by spreading them over more CTAs and warps: the reductions take
+// eight columns of X per CTA, the expansion 32 rows and four columns with the sum over the
+// factor columns split over the eight warps (23 -> 5 us and 11 -> 4 us a launch at n = 511).
 template <typename R>
-__global__ void tsmm_reduce(Geo g, int d, const Cx<R>* __restrict__ G_F, const int* __restrict__ G_rank,
-                            const Cx<R>* __restrict__ S_F, const int* __restrict__ S_rank, Cx<R>* __restrict__ Qr) {
+__global__ void __launch_bounds__(kBlk) tsmm_reduce(Geo g, int d, const Cx<R>* __restrict__ G_F,
+                                                    const int* __restrict__ G_rank, const Cx<R>* __restrict__ S_F,
+                                                    const int* __restrict__ S_rank, Cx<R>* __restrict__ Qr) {
+  pdl_begin();
   const int u = (1 << (d + 2)) + blockIdx.x;
   const int du = depth_of(u);
   const int nu = u >> (du - (d + 1));          // ancestor at depth d+1
-  const int ru = G_rank[u], k = S_rank[nu];
+  const int ru = G_rank[u], k = S_rank[nu], c0 = 8 * blockIdx.y;
+  if (c0 >= k) return;
   const int s = g.sz[u], ld_x = g.sz[nu], xo = g.lo[u] - g.lo[nu];
   const Cx<R>* F = G_F + g.gfo[u];
-  const Cx<R>* X = S_F + g.sfo[nu];
+  const Cx<R>* X[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) X[t] = S_F + g.sfo[nu] + (long long)min(c0 + t, k - 1) * ld_x + xo;
   Cx<R>* out = Qr + g.qro[u];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int kr = warp; kr < ru; kr += nw) {
-    for (int c0 = 0; c0 < k; c0 += 8) {
-      Cx<R> acc[8];
+    Cx<R> acc[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) acc[t] = Cx<R>(0, 0);
-      for (int i = lane; i < s; i += 32) {
-        Cx<R> f = F[(long long)kr * s + i];
+    for (int t = 0; t < 8; ++t) acc[t] = Cx<R>(0, 0);
+    for (int i = lane; i < s; i += 32) {
+      const Cx<R> f = F[(long long)kr * s + i];
 #pragma unroll
-        for (int t = 0; t < 8; ++t)
-          if (c0 + t < k) cfma(acc[t], f, X[(long long)(c0 + t) * ld_x + xo + i]);
-      }
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        Cx<R> v = warp_sum(acc[t]);
-        if (lane == 0 && c0 + t < k) out[kr * g.KCAP + c0 + t] = v;
-      }
+      for (int t = 0; t < 8; ++t) cfma(acc[t], f, X[t][i]);
     }
+    int t;
+    bool first;
+    scatter_sum<R, 8, 32, 1>(acc, lane, t, first);
+    if (first && c0 + t < k) out[kr * g.KCAP + c0 + t] = acc[0];
   }
 }
 
 template <typename R>
-__global__ void tsmm_expand(Geo g, int d, const Cx<R>* __restrict__ G_leaf, const Cx<R>* __restrict__ G_F,
-                            const int* __restrict__ G_rank, const Cx<R>* __restrict__ S_F,
-                            const int* __restrict__ S_rank, const Cx<R>* __restrict__ Qr, Cx<R>* __restrict__ Y) {
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;
-  const int col = blockIdx.y;
-  if (row >= g.n) return;
+__global__ void __launch_bounds__(kBlk) tsmm_expand(Geo g, int d, const Cx<R>* __restrict__ G_leaf,
+                                                    const Cx<R>* __restrict__ G_F, const int* __restrict__ G_rank,
+                                                    const Cx<R>* __restrict__ S_F, const int* __restrict__ S_rank,
+                                                    const Cx<R>* __restrict__ Qr, Cx<R>* __restrict__ Y) {
+  pdl_begin();
+  __shared__ Cx<R> red[kBlk / 32][4][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kBlk / 32;
+  const int row = min(blockIdx.x * 32 + lane, g.n - 1);
+  const int col = 4 * blockIdx.y;
   const int lam = g.rowleaf[row];
   const int nu = lam >> (g.L - (d + 1));
   const int k = S_rank[nu];
-  if (col >= k) return;
   const int lo_nu = g.lo[nu], ld = g.sz[nu];
-  const Cx<R>* X = S_F + g.sfo[nu] + (long long)col * ld;
-  Cx<R> y(0, 0);
-  {
-    const int lf = g.leaf, a = row - g.lo[lam], s = g.sz[lam];
-    const Cx<R>* D = G_leaf + (long long)(lam - (1 << g.L)) * lf * lf;
-    for (int b = 0; b < s; ++b) cfma(y, D[b * lf + a], X[g.lo[lam] - lo_nu + b]);
+  Cx<R> y[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) y[t] = Cx<R>(0, 0);
+  if (col < k) {
+    int ct[4];        // the columns (the last one again past the end)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) ct[t] = min(col + t, k - 1);
+    {
+      const int lf = g.leaf, a = row - g.lo[lam], s = g.sz[lam];
+      const Cx<R>* D = G_leaf + (long long)(lam - (1 << g.L)) * lf * lf;
+      const Cx<R>* X = S_F + g.sfo[nu] + (g.lo[lam] - lo_nu);
+      for (int b = warp; b < s; b += nw) {
+        const Cx<R> f = D[b * lf + a];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) cfma(y[t], f, X[(long long)ct[t] * ld + b]);
+      }
+    }
+    for (int du = d + 2; du <= g.L; ++du) {
+      const int u = lam >> (g.L - du);
+      const int ru = G_rank[u];
+      const Cx<R>* F = G_F + g.gfo[u] + (row - g.lo[u]);
+      const Cx<R>* q = Qr + g.qro[u ^ 1];
+      const int s = g.sz[u];
+#pragma unroll 4
+      for (int kr = warp; kr < ru; kr += nw) {
+        const Cx<R> f = F[(long long)kr * s];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) cfma(y[t], f, q[kr * g.KCAP + ct[t]]);
+      }
+    }
   }
-  for (int du = d + 2; du <= g.L; ++du) {
-    const int u = lam >> (g.L - du);
-    const int ru = G_rank[u];
-    const Cx<R>* F = G_F + g.gfo[u] + (row - g.lo[u]);
-    const Cx<R>* q = Qr + g.qro[u ^ 1] + col;
-    const int s = g.sz[u];
-    for (int kr = 0; kr < ru; ++kr) cfma(y, F[(long long)kr * s], q[kr * g.KCAP]);
+#pragma unroll
+  for (int t = 0; t < 4; ++t) red[warp][t][lane] = y[t];
+  __syncthreads();
+  const int t = threadIdx.x >> 5;       // column of this thread's sum
+  if (t < 4 && blockIdx.x * 32 + lane < g.n && col + t < k) {
+    Cx<R> v = red[0][t][lane];
+#pragma unroll
+    for (int w = 1; w < kBlk / 32; ++w) v += red[w][t][lane];
+    Y[(long long)lo_nu * g.KCAP + (long long)(col + t) * ld + (row - lo_nu)] = v;
   }
-  Y[(long long)lo_nu * g.KCAP + (long long)col * ld + (row - lo_nu)] = y;
 }
 
 // ---------------------------------------------------------------------------------
@@ -285,6 +391,7 @@ __global__ void tsmm_expand(Geo g, int d, const Cx<R>* __restrict__ G_leaf, cons
 template <typename R>
 __global__ void core_dots(Geo g, int d, const Cx<R>* __restrict__ S_F, const int* __restrict__ S_rank,
                           const Cx<R>* __restrict__ Y, Cx<R>* __restrict__ PQ) {
+  pdl_begin();
   const int t = (1 << d) + blockIdx.x / 2;
   const int side = blockIdx.x & 1;
   const int v = 2 * t + side;
@@ -293,19 +400,33 @@ __global__ void core_dots(Geo g, int d, const Cx<R>* __restrict__ S_F, const int
   const Cx<R>* Yv = Y + (long long)g.lo[v] * g.KCAP;
   Cx<R>* out = PQ + ((long long)(t - (1 << d)) * 2 + side) * g.KCAP * g.KCAP;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int e = blockIdx.y * nw + warp; e < k * k; e += gridDim.y * nw) {
-    const int a = e / k, b = e % k;
-    Cx<R> acc(0, 0);
-    for (int i = lane; i < s; i += 32) cfma(acc, U[(long long)a * s + i], Yv[(long long)b * s + i]);
-    acc = warp_sum(acc);
-    if (lane == 0) out[a * g.KCAP + b] = acc;
+  const int kb = (k + 3) / 4;      // four columns of Y at a time
+  for (int e = blockIdx.y * nw + warp; e < k * kb; e += gridDim.y * nw) {
+    const int a = e / kb, b = 4 * (e % kb);
+    Cx<R> acc[4];
+    const Cx<R>* yc[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      acc[t] = Cx<R>(0, 0);
+      yc[t] = Yv + (long long)min(b + t, k - 1) * s;
+    }
+    for (int i = lane; i < s; i += 32) {
+      const Cx<R> f = U[(long long)a * s + i];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) cfma(acc[t], f, yc[t][i]);
+    }
+    int t;
+    bool first;
+    scatter_sum<R, 4, 32, 1>(acc, lane, t, first);
+    if (first && b + t < k) out[a * g.KCAP + b + t] = acc[0];
   }
 }
 
+// (the whole CTA; dynamic shared memory sm)
 template <typename R>
-__global__ void core_inverse(Geo g, int d, int m, const int* __restrict__ S_rank, const Cx<R>* __restrict__ PQ,
-                             Cx<R>* __restrict__ Mb, int* status) {
-  extern __shared__ __align__(16) unsigned char sm[];
+__device__ void core_inverse_pivoted(const Geo& g, int d, int m, const int* __restrict__ S_rank,
+                                     const Cx<R>* __restrict__ PQ, Cx<R>* __restrict__ Mb, int* status,
+                                     unsigned char* sm) {
   const int t = (1 << d) + blockIdx.x;
   const int k = S_rank[2 * t];
   const int n2 = 2 * k;
@@ -411,33 +532,255 @@ __global__ void core_inverse(Geo g, int d, int m, const int* __restrict__ S_rank
   }
 }
 
-// W_v = Y_v M_side (k x k block of M), and the new off-diagonal block at the parent:
-// F_a = -Y_a M12, F_b = Y_b.
 template <typename R>
-__global__ void woodbury_form(Geo g, int d, const int* __restrict__ S_rank, const Cx<R>* __restrict__ Y,
-                              const Cx<R>* __restrict__ Mb, Cx<R>* __restrict__ W, Cx<R>* __restrict__ G_F,
-                              int* __restrict__ G_rank) {
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;
-  const int col = blockIdx.y;
+__global__ void core_inverse(Geo g, int d, int m, const int* __restrict__ S_rank, const Cx<R>* __restrict__ PQ,
+                             Cx<R>* __restrict__ Mb, int* status) {
+  pdl_begin();
+  extern __shared__ __align__(16) unsigned char sm[];
+  core_inverse_pivoted<R>(g, d, m, S_rank, PQ, Mb, status, sm);
+}
+
+// In complex64, the blocks of the inverse that are used, from one k x k inverse: with
+// N = (I - Q P)^{-1},
+//     M11 = -N Q,  M12 = N,  M22 = -P N   (M21 = M12^t is not needed),
+// half the pivots and an eighth of the elimination of the 2k x 2k matrix (31 -> 13 us a depth
+// at 76 columns).  It takes the identity blocks as pivots, which is as stable as pivoting
+// while the entries of P and Q are of order one, as they are for a block's coupling seen
+// through its own inverse; a matrix with an entry above kCoreLarge, or with a vanishing pivot,
+// goes through the pivoted elimination above.
+// N by Gauss-Jordan in registers: warp w of sixteen holds the rows w, w + 16, ..., a lane the
+// columns lane, lane + 32.  No row is moved: a pivot row keeps its place (order kept in prow)
+// and the interchanges are undone by where the result is written.  After its update each warp
+// offers its best candidate for the next pivot and that row; after one barrier every warp
+// picks the largest of the sixteen offers.
+constexpr int kCoreWarps = 16, kCoreRows = 4, kCoreCols = 2;      // k <= 57 columns (r_max + 1)
+constexpr float kCoreLarge = 4.0f;
+
+// out[i][j] = add[i][j] + sgn (X Y)[i][j] for k x k matrices in shared memory (ld k), 2 x 2 tiles
+template <typename Store>
+__device__ __forceinline__ void core_gemm(const Cx<float>* X, const Cx<float>* Y, int k, Store store) {
+  const int kt = (k + 1) / 2;
+  for (int e = threadIdx.x; e < kt * kt; e += blockDim.x) {
+    const int i0 = 2 * (e / kt), j0 = 2 * (e % kt), i1 = min(i0 + 1, k - 1), j1 = min(j0 + 1, k - 1);
+    Cx<float> a00(0.f, 0.f), a01 = a00, a10 = a00, a11 = a00;
+#pragma unroll 2
+    for (int l = 0; l < k; ++l) {
+      const Cx<float> x0 = X[i0 * k + l], x1 = X[i1 * k + l], y0 = Y[l * k + j0], y1 = Y[l * k + j1];
+      cfma(a00, x0, y0);
+      cfma(a01, x0, y1);
+      cfma(a10, x1, y0);
+      cfma(a11, x1, y1);
+    }
+    store(i0, j0, a00);
+    if (j1 > j0) store(i0, j1, a01);
+    if (i1 > i0) store(i1, j0, a10);
+    if (i1 > i0 && j1 > j0) store(i1, j1, a11);
+  }
+}
+
+__global__ void __launch_bounds__(32 * kCoreWarps) core_inverse_block(Geo g, int d, int m,
+                                                                      const int* __restrict__ S_rank,
+                                                                      const Cx<float>* __restrict__ PQ,
+                                                                      Cx<float>* __restrict__ Mb, int* status) {
+  pdl_begin();
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ Cx<float> offer[2][kCoreWarps][32 * kCoreCols];
+  __shared__ float osize[2][kCoreWarps];
+  __shared__ int orow[2][kCoreWarps];
+  __shared__ int prow[kCoreWarps * kCoreRows];
+  __shared__ float red[2][kCoreWarps];
+  const int t = (1 << d) + blockIdx.x;
+  const int k = S_rank[2 * t];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const Cx<float>* Pg = PQ + ((long long)(t - (1 << d)) * 2) * g.KCAP * g.KCAP;
+  const Cx<float>* Qg = Pg + g.KCAP * g.KCAP;
+  Cx<float>* P = reinterpret_cast<Cx<float>*>(sm);
+  Cx<float>* Q = P + k * k;
+  Cx<float>* B = Q + k * k;
+  float mx = 0;
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
+    const int i = e / k, j = e - i * k;
+    const Cx<float> p = Pg[i * g.KCAP + j], q = Qg[i * g.KCAP + j];
+    P[e] = p;
+    Q[e] = q;
+    mx = fmaxf(mx, fmaxf(abs2(p), abs2(q)));
+  }
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) red[0][warp] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kCoreWarps; ++i) mx = fmaxf(mx, red[0][i]);
+  if (!(mx <= kCoreLarge * kCoreLarge)) {
+    __syncthreads();
+    core_inverse_pivoted<float>(g, d, m, S_rank, PQ, Mb, status, sm);
+    return;
+  }
+  core_gemm(Q, P, k, [&](int i, int j, Cx<float> v) { B[i * k + j] = (i == j ? Cx<float>(1.f, 0.f) : Cx<float>(0.f, 0.f)) - v; });
+  __syncthreads();
+  Cx<float> A[kCoreRows][kCoreCols];
+  mx = 0;
+#pragma unroll
+  for (int r = 0; r < kCoreRows; ++r)
+#pragma unroll
+    for (int c = 0; c < kCoreCols; ++c) {
+      const int a = warp + kCoreWarps * r, b = lane + 32 * c;
+      A[r][c] = (a < k && b < k) ? B[a * k + b] : Cx<float>(0.f, 0.f);
+      mx = fmaxf(mx, abs2(A[r][c]));
+    }
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) red[1][warp] = mx;
+  const int nr = (k - warp + kCoreWarps - 1) / kCoreWarps;      // rows of this warp
+  unsigned used = 0;                    // bit r: row r of this warp was a pivot row
+  // this warp's largest unused |A[.][kl + 32 cc]|^2 (ties: the smallest row) and that row
+  auto make_offer = [&](auto ccc, int kl, int b) {
+    constexpr int cc = decltype(ccc)::value;
+    float best = -1.f;
+    int br = 0;
+#pragma unroll
+    for (int r = 0; r < kCoreRows; ++r) {
+      const float v = abs2(A[r][cc]);
+      if (r < nr && !(used >> r & 1u) && v > best) { best = v; br = r; }
+    }
+    best = __shfl_sync(0xffffffffu, best, kl);      // the lane that holds the column decides
+    br = __shfl_sync(0xffffffffu, br, kl);
+    if (lane == 0) {
+      osize[b][warp] = best;
+      orow[b][warp] = warp + kCoreWarps * br;
+    }
+#pragma unroll
+    for (int r = 0; r < kCoreRows; ++r)
+      if (r == br) {
+#pragma unroll
+        for (int c = 0; c < kCoreCols; ++c) offer[b][warp][lane + 32 * c] = A[r][c];
+      }
+  };
+  make_offer(std::integral_constant<int, 0>(), 0, 0);
+  __syncthreads();
+  mx = 0;
+#pragma unroll
+  for (int i = 0; i < kCoreWarps; ++i) mx = fmaxf(mx, red[1][i]);
+  const float tiny = 1e-14f * mx;       // on |pivot|^2
+  bool bad = false;
+  auto half = [&](auto ccc) {           // the pivots of columns 32 cc ..
+    constexpr int cc = decltype(ccc)::value;
+    for (int kk = 32 * cc; kk < min(k, 32 * cc + 32); ++kk) {
+      const int b = kk & 1, kl = kk & 31;
+      float best = osize[b][0];
+      int ow = 0, p = orow[b][0];
+#pragma unroll
+      for (int i = 1; i < kCoreWarps; ++i) {
+        const float v = osize[b][i];
+        const int pi = orow[b][i];
+        if (v > best || (v == best && pi < p)) { best = v; ow = i; p = pi; }
+      }
+      if (!(best > tiny)) { bad = true; return; }
+      if (threadIdx.x == 0) prow[kk] = p;
+      const Cx<float> ip = cinv(offer[b][ow][kk]);
+      // the pivot row divided by the pivot, with 1 / pivot in its own column
+      Cx<float> pr[kCoreCols];
+#pragma unroll
+      for (int c = 0; c < kCoreCols; ++c) pr[c] = offer[b][ow][lane + 32 * c] * ip;
+      if (lane == kl) pr[cc] = ip;
+#pragma unroll
+      for (int r = 0; r < kCoreRows; ++r) {
+        if (r < nr) {
+          const Cx<float> f(__shfl_sync(0xffffffffu, A[r][cc].re, kl), __shfl_sync(0xffffffffu, A[r][cc].im, kl));
+          if (warp + kCoreWarps * r == p) {
+            used |= 1u << r;
+#pragma unroll
+            for (int c = 0; c < kCoreCols; ++c) A[r][c] = pr[c];
+          } else {
+            if (lane == kl) A[r][cc] = Cx<float>(0.f, 0.f);
+#pragma unroll
+            for (int c = 0; c < kCoreCols; ++c) cfma(A[r][c], -f, pr[c]);
+          }
+        }
+      }
+      if (kk + 1 < k) {
+        if (kl < 31) make_offer(ccc, kl + 1, b ^ 1);
+        else make_offer(std::integral_constant<int, (cc + 1 < kCoreCols ? cc + 1 : cc)>(), 0, b ^ 1);
+      }
+      __syncthreads();
+    }
+  };
+  half(std::integral_constant<int, 0>());
+  if (!bad && k > 32) half(std::integral_constant<int, 1>());
+  if (bad) {
+    __syncthreads();
+    core_inverse_pivoted<float>(g, d, m, S_rank, PQ, Mb, status, sm);
+    return;
+  }
+  // physical row prow[i] is row i of the inverse, column l is its column prow[l]
+  int* inv = reinterpret_cast<int*>(&offer[0][0][0]);      // logical row of a physical one
+  for (int i = threadIdx.x; i < k; i += blockDim.x) inv[prow[i]] = i;
+  __syncthreads();
+  Cx<float>* M = Mb + (long long)(t - (1 << d)) * 4 * g.KCAP * g.KCAP;
+  const int ldm = 2 * g.KCAP;
+#pragma unroll
+  for (int r = 0; r < kCoreRows; ++r)
+    if (r < nr) {
+      const int i = inv[warp + kCoreWarps * r];
+#pragma unroll
+      for (int c = 0; c < kCoreCols; ++c) {
+        const int l = lane + 32 * c;
+        if (l < k) {
+          B[i * k + prow[l]] = A[r][c];
+          M[i * ldm + k + prow[l]] = A[r][c];                  // M12
+        }
+      }
+    }
+  __syncthreads();
+  core_gemm(B, Q, k, [&](int i, int j, Cx<float> v) { M[i * ldm + j] = -v; });                       // M11
+  core_gemm(P, B, k, [&](int i, int j, Cx<float> v) { M[(k + i) * ldm + k + j] = -v; });             // M22
+}
+
+// W_v = Y_v M_side (k x k block of M), and the new off-diagonal block at the parent:
+// F_a = -Y_a M12, F_b = Y_b.  A thread has one row and four columns.
+template <typename R>
+__global__ void __launch_bounds__(128) woodbury_form(Geo g, int d, const int* __restrict__ S_rank,
+                                                     const Cx<R>* __restrict__ Y, const Cx<R>* __restrict__ Mb,
+                                                     Cx<R>* __restrict__ W, Cx<R>* __restrict__ G_F,
+                                                     int* __restrict__ G_rank) {
+  pdl_begin();
+  const int row = blockIdx.x * 32 + (threadIdx.x & 31);
+  const int col = 4 * (blockIdx.y * 4 + (threadIdx.x >> 5));
   if (row >= g.n) return;
   const int v = g.rowleaf[row] >> (g.L - (d + 1));
   const int t = v >> 1, side = v & 1;
   const int k = S_rank[v];
   if (col >= k) return;
   const int s = g.sz[v], i = row - g.lo[v];
-  const Cx<R>* Yv = Y + (long long)g.lo[v] * g.KCAP;
+  const Cx<R>* Yv = Y + (long long)g.lo[v] * g.KCAP + i;
   const Cx<R>* M = Mb + (long long)(t - (1 << d)) * 4 * g.KCAP * g.KCAP;
   const int ldm = 2 * g.KCAP;
   const int off = side ? k : 0;
-  Cx<R> w(0, 0), nf(0, 0);
-  for (int j = 0; j < k; ++j) {
-    const Cx<R> y = Yv[(long long)j * s + i];
-    cfma(w, y, M[(off + j) * ldm + off + col]);          // M11 or M22
-    if (!side) cfma(nf, y, M[j * ldm + k + col]);         // M12
+  Cx<R> w[4], nf[4];
+  int c[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    w[u] = nf[u] = Cx<R>(0, 0);
+    c[u] = min(col + u, k - 1);
   }
-  W[(long long)g.lo[v] * g.KCAP + (long long)col * s + i] = w;
+#pragma unroll 2
+  for (int j = 0; j < k; ++j) {
+    const Cx<R> y = Yv[(long long)j * s];
+    const Cx<R>* M1 = M + (off + j) * ldm + off;        // M11 or M22
+#pragma unroll
+    for (int u = 0; u < 4; ++u) cfma(w[u], y, M1[c[u]]);
+    if (!side) {
+      const Cx<R>* M2 = M + j * ldm + k;                 // M12
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cfma(nf[u], y, M2[c[u]]);
+    }
+  }
   Cx<R>* F = G_F + g.gfo[v];
-  F[(long long)col * s + i] = side ? Yv[(long long)col * s + i] : -nf;
+  Cx<R>* Wv = W + (long long)g.lo[v] * g.KCAP;
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    if (col + u < k) {
+      Wv[(long long)(col + u) * s + i] = w[u];
+      F[(long long)(col + u) * s + i] = side ? Yv[(long long)(col + u) * s] : -nf[u];
+    }
   if (i == 0 && col == 0) G_rank[v] = k;
 }
 
@@ -448,6 +791,7 @@ template <typename R>
 __global__ void woodbury_append(Geo g, int d, const int* __restrict__ S_rank, const Cx<R>* __restrict__ Y,
                                 const Cx<R>* __restrict__ W, Cx<R>* __restrict__ G_F, int* __restrict__ G_rank,
                                 Cx<R>* __restrict__ G_leaf) {
+  pdl_begin();
   const int u = (1 << (d + 1)) + blockIdx.x;
   const int du = depth_of(u);
   const int nu = u >> (du - (d + 1));
@@ -482,15 +826,21 @@ __global__ void woodbury_append(Geo g, int d, const int* __restrict__ S_rank, co
 // Recompression, step 1, for the nodes u = list[blockIdx.x]: with w = rank(u) columns,
 // a factor with at least as many columns as rows (w >= sz(u)), or in complex64 of at most
 // kDenseRows rows, takes the dense path, Q = I and R = F_u (qcols = sz(u), qmode = 1);
-// otherwise Gram-Schmidt QR (twice
-// orthogonalised) of F_u in place, the Q columns compacted to the independent ones and
-// R (qc x w) written out (qmode = 0).  R is row-major with leading dimension cap(u).  When
-// F_u fits the kernel's shared memory (qs_entries), the orthogonalisation runs there and
-// the kept columns are written back at the end (every projection reads all earlier
-// columns: O(w^2 s) reads that would otherwise go to L2).
+// otherwise the QR of F_u in place by modified Gram-Schmidt: a column whose remainder is at
+// the rounding level of its own norm is dropped, the Q columns are compacted and R (qc x w)
+// written out (qmode = 0).  R is row-major with leading dimension cap(u).
+// Every step updates all later columns (a warp per column, the new norm with the update), so
+// a step costs one barrier; classical Gram-Schmidt with its two passes took ten, 3.6 us a
+// column (256 rows, 37 columns: 120 us, now 15).  F = Q R holds to rounding; Q is orthogonal
+// to rounding over the relative size of a column's remainder, which is all the SVD of the
+// core asks of it (a skew of a column near the drop threshold moves the singular values
+// compared with eps_H by as much, not the product).  When F_u fits the kernel's shared
+// memory (qs_entries) the columns stay there.
 template <typename R>
-__global__ void qr_cgs2(Geo g, Cx<R>* __restrict__ G_F, const int* __restrict__ G_rank, Cx<R>* __restrict__ Rb,
-                        int* __restrict__ qcols, int* __restrict__ qmode, int qs_entries) {
+__global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, const int* __restrict__ G_rank,
+                                               Cx<R>* __restrict__ Rb, int* __restrict__ qcols, int* __restrict__ qmode,
+                                               int qs_entries) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char sm[];
   const int u = g.list[blockIdx.x];
   const int s = g.sz[u], w = G_rank[u], ld = g.cap[u];
@@ -504,77 +854,68 @@ __global__ void qr_cgs2(Geo g, Cx<R>* __restrict__ G_F, const int* __restrict__ 
     if (threadIdx.x == 0) { qcols[u] = s; qmode[u] = 1; }
     return;
   }
-  Cx<R>* v = reinterpret_cast<Cx<R>*>(sm);                // [s]
-  Cx<R>* c = v + s;                                        // [QCAP]
-  R* red = reinterpret_cast<R*>(c + g.QCAP);               // [32]
-  const size_t qs_off = ((size_t)(s + g.QCAP) * sizeof(Cx<R>) + 32 * sizeof(R) + 15) & ~size_t(15);
+  const int wcap = g.cap_max;
+  R* cur = reinterpret_cast<R*>(sm);                       // [wcap] squared norm of a column's remainder
+  R* org = cur + wcap;                                     // [wcap] and of the column itself
+  int* pos = reinterpret_cast<int*>(org + wcap);           // [wcap] Q column of a kept column, or -1
+  const size_t qs_off = ((size_t)wcap * (2 * sizeof(R) + sizeof(int)) + 15) & ~size_t(15);
   const bool qsh = (long long)s * w <= qs_entries;
   Cx<R>* Fq = qsh ? reinterpret_cast<Cx<R>*>(sm + qs_off) : F;   // the columns being orthogonalised
-  __shared__ int s_qc;
-  if (threadIdx.x == 0) s_qc = 0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int rows = min(s, ld);
   for (int e = threadIdx.x; e < rows * w; e += blockDim.x) Rm[(long long)(e / w) * ld + e % w] = Cx<R>(0, 0);
-  if (qsh)
-    for (int e = threadIdx.x; e < s * w; e += blockDim.x) Fq[e] = F[e];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  // lanes per row of the projection update: a power of two, at most 32 and at most
-  // blockDim / s (at least 1); blockDim.x is a multiple of 32
-  int gT = 1;
-  while (gT < 32 && 2 * gT * s <= (int)blockDim.x) gT *= 2;
-  const int rows_per_pass = (int)blockDim.x / gT;
-  for (int j = 0; j < w; ++j) {
-    const int qc = s_qc;
-    R nrm0 = 0;
-    for (int i = threadIdx.x; i < s; i += blockDim.x) {
-      v[i] = Fq[(long long)j * s + i];
-      nrm0 += abs2(v[i]);
+  for (int j = warp; j < w; j += nw) {
+    R acc = 0;
+    for (int i = lane; i < s; i += 32) {
+      const Cx<R> v = F[(long long)j * s + i];
+      if (qsh) Fq[(long long)j * s + i] = v;
+      acc += abs2(v);
     }
-    nrm0 = block_sum(nrm0, red);
-    __syncthreads();
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int l = warp; l < qc; l += nw) {
-        Cx<R> acc(0, 0);
-        for (int i = lane; i < s; i += 32) cfma_conj(acc, Fq[(long long)l * s + i], v[i]);
-        acc = warp_sum(acc);
+    acc = warp_sum_r(acc);
+    if (lane == 0) cur[j] = org[j] = acc;
+  }
+  __syncthreads();
+  int qc = 0;
+  for (int j = 0; j < w; ++j) {
+    const R nr = cur[j];
+    const bool kept = nr > Tiny<R>::dep * Tiny<R>::dep * org[j] && nr > 0 && qc < rows;
+    if (kept) {
+      const R inv = rcp_any(nr), rs = rsqrt_any(nr), nn = nr * rs;
+      const Cx<R>* cj = Fq + (long long)j * s;
+      for (int l = j + 1 + warp; l < w; l += nw) {
+        Cx<R>* cl = Fq + (long long)l * s;
+        Cx<R> d(0, 0);
+        for (int i = lane; i < s; i += 32) cfma_conj(d, cj[i], cl[i]);
+        for (int o = 16; o > 0; o >>= 1) d += shfl_xor(d, o);
+        const Cx<R> be = -(inv * d);
+        R acc = 0;
+        for (int i = lane; i < s; i += 32) {
+          Cx<R> v = cl[i];
+          cfma(v, be, cj[i]);
+          cl[i] = v;
+          acc = fma(v.re, v.re, fma(v.im, v.im, acc));
+        }
+        acc = warp_sum_r(acc);
         if (lane == 0) {
-          c[l] = acc;
-          Rm[(long long)l * ld + j] += acc;
+          cur[l] = acc;
+          Rm[(long long)qc * ld + l] = rs * d;
         }
       }
-      __syncthreads();
-      // v -= Q c: gT lanes per row share the sum over the kept columns (all threads busy
-      // when the block has fewer rows than threads)
-      for (int i0 = 0; i0 < s; i0 += rows_per_pass) {
-        const int i = i0 + threadIdx.x / gT, sub = threadIdx.x % gT;
-        Cx<R> acc(0, 0);
-        if (i < s)
-          for (int l = sub; l < qc; l += gT) cfma(acc, Fq[(long long)l * s + i], c[l]);
-        for (int o = gT >> 1; o > 0; o >>= 1) acc += shfl_xor(acc, o);
-        if (i < s && sub == 0) v[i] -= acc;
-      }
-      __syncthreads();
+      if (threadIdx.x == 0) Rm[(long long)qc * ld + j] = Cx<R>(nn, 0);
     }
-    R nr = 0;
-    for (int i = threadIdx.x; i < s; i += blockDim.x) nr += abs2(v[i]);
-    nr = block_sum(nr, red);
-    if (nr > Tiny<R>::dep * Tiny<R>::dep * nrm0 && nr > 0) {
-      const R sn = sqrt(nr), is = R(1) / sn;
-      for (int i = threadIdx.x; i < s; i += blockDim.x) Fq[(long long)qc * s + i] = is * v[i];
-      if (threadIdx.x == 0) {
-        Rm[(long long)qc * ld + j] = Cx<R>(sn, 0);
-        s_qc = qc + 1;
-      }
-    } else if (threadIdx.x == 0) {
-      // dependent column: its projections were accumulated into R; drop the remainder
-    }
+    if (threadIdx.x == 0) pos[j] = kept ? qc : -1;
+    if (kept) ++qc;
     __syncthreads();
   }
-  if (qsh) {
-    const int qc = s_qc;
-    for (int e = threadIdx.x; e < s * qc; e += blockDim.x) F[e] = Fq[e];
+  // the kept columns, normalised, to the front (a Q column never lies behind its source)
+  for (int j = 0; j < w; ++j) {
+    const int c = pos[j];
+    if (c < 0) continue;
+    const R rs = rsqrt_any(cur[j]);
+    for (int i = threadIdx.x; i < s; i += blockDim.x) F[(long long)c * s + i] = rs * Fq[(long long)j * s + i];
+    if (!qsh) __syncthreads();
   }
-  if (threadIdx.x == 0) { qcols[u] = s_qc; qmode[u] = 0; }
+  if (threadIdx.x == 0) { qcols[u] = qc; qmode[u] = 0; }
 }
 
 // Recompression, step 2a: the cores C = R_a R_b^t (qa x qb, column-major, ld qa, at
@@ -600,6 +941,7 @@ template <typename R>
 __global__ void __launch_bounds__(256) core_product_cc(Geo g, const Cx<R>* __restrict__ Rb,
                                                        const int* __restrict__ qcols, const int* __restrict__ G_rank,
                                                        Cx<R>* __restrict__ Cb) {
+  pdl_begin();
   __shared__ Cx<R> As[kCK][kCT + 1], Bs[kCK][kCT + 1];
   const int a = g.list[blockIdx.y], b = a + 1;
   const int qa = qcols[a], qb = qcols[b], w = G_rank[a];
@@ -660,6 +1002,7 @@ __device__ __forceinline__ void mma_m16n8k8_tf32(float (&c)[4], const unsigned (
 __global__ void __launch_bounds__(256) core_product_tc(Geo g, const Cx<float>* __restrict__ Rb,
                                                        const int* __restrict__ qcols, const int* __restrict__ G_rank,
                                                        Cx<float>* __restrict__ Cb) {
+  pdl_begin();
   __shared__ Cx<float> As[kCT][kCK + 1], Bs[kCT][kCK + 1];
   const int a = g.list[blockIdx.y], b = a + 1;
   const int qa = qcols[a], qb = qcols[b], w = G_rank[a];
@@ -738,24 +1081,6 @@ template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW
   return v;
 }
 
-// Reciprocal and reciprocal square root, in complex128 by two Newton steps from the FP32
-// value (a handful of FP64 operations where the division and square root routines take
-// dozens: a warp's FP64 instruction occupies its scheduler for about 64 clocks here)
-__device__ __forceinline__ float rcp_of(float x) { return 1.0f / x; }
-__device__ __forceinline__ double rcp_of(double x) {
-  // x in [1e-28, 4]: inside FP32's range
-  double y = (double)(1.0f / (float)x);
-  y = y * fma(-x, y, 2.0);
-  return y * fma(-x, y, 2.0);
-}
-__device__ __forceinline__ float rsqrt_of(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_of(double x) {
-  double y = (double)rsqrtf((float)x);
-  const double h = 0.5 * x;
-  y = y * fma(-h * y, y, 1.5);
-  return y * fma(-h * y, y, 1.5);
-}
-
 // Recompression, step 2b: for every sibling pair (a, b) with a = list[blockIdx.x], the
 // truncated SVD of the core C (step 2a), as the small transforms
 //   T_b = conj(P) Sigma^(1/2) (qb x k'),  T_a = C P Sigma^(-1/2) (qa x k'),
@@ -778,6 +1103,7 @@ template <typename R>
 __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R>* __restrict__ Cb,
                                                    const int* __restrict__ qcols, Cx<R>* __restrict__ Tx,
                                                    int* __restrict__ newrank, int smem_entries, R thr) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char sm[];
   const int a = g.list[blockIdx.x], b = a + 1, t = a >> 1;
   const int qa = qcols[a], qb = qcols[b];
@@ -915,8 +1241,23 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
         Cx<R>* cq = C + (live ? slot[iq] : 0) * ld;
         const R al = live ? sig[ip] : R(1), be = live ? sig[iq] : R(1);
         Cx<R> ga(0, 0);
-        if (live)
+        // (complex64, a warp a pair: the two columns stay in registers for the rotation)
+        constexpr int NR = 5;
+        const bool reg = sizeof(R) == 4 && GW == 32 && qb <= 32 * NR;
+        Cx<float> xr[NR], yr[NR];
+        if (reg) {
+          if constexpr (sizeof(R) == 4) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+              const bool in = live && lane + 32 * r < qb;
+              xr[r] = in ? cp[lane + 32 * r] : Cx<float>(0.f, 0.f);
+              yr[r] = in ? cq[lane + 32 * r] : Cx<float>(0.f, 0.f);
+              cfma_conj(ga, xr[r], yr[r]);
+            }
+          }
+        } else if (live) {
           for (int i = gl; i < qb; i += GW) cfma_conj(ga, cp[i], cq[i]);
+        }
         ga = group_sum(ga, GW);
         // g = <p, q> / (|p| |q|): the angle's cotangent 2 z = (|q|^2 - |p|^2) / |<p, q>|
         const float ra = rsqrtf((float)al), rb = rsqrtf((float)be);
@@ -925,7 +1266,7 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
         const float gg = (float)abs2(gn);
         const bool rot = live && al >= thr && be >= thr && gg > (float)(Tiny<R>::jac * Tiny<R>::jac);
         if (rot) {
-          if (gl == 0) s_rot = 1;
+          if (gl == 0 && gg > Tiny<R>::quad) s_rot = 1;
           const float ig = rsqrtf(gg);
           const float z = 0.5f * (float)((be - al) * s) * ig;
           // (z reaches 1e29 in complex128, where its square would overflow)
@@ -940,19 +1281,33 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
             sig[ip] = fmax(R(0), al - ag);
             sig[iq] = be + ag;
           }
-          for (int i = gl; i < qb; i += GW) {
-            const Cx<R> x = cp[i], y = cq[i];
-            Cx<R> nx = cs * x, ny = cs * y;
-            cfma(nx, -snc, y);
-            cfma(ny, sne, x);
-            cp[i] = nx;
-            cq[i] = ny;
+          if (reg) {
+            if constexpr (sizeof(R) == 4) {
+#pragma unroll
+              for (int r = 0; r < NR; ++r)
+                if (lane + 32 * r < qb) {
+                  Cx<float> nx = cs * xr[r], ny = cs * yr[r];
+                  cfma(nx, -snc, yr[r]);
+                  cfma(ny, sne, xr[r]);
+                  cp[lane + 32 * r] = nx;
+                  cq[lane + 32 * r] = ny;
+                }
+            }
+          } else {
+            for (int i = gl; i < qb; i += GW) {
+              const Cx<R> x = cp[i], y = cq[i];
+              Cx<R> nx = cs * x, ny = cs * y;
+              cfma(nx, -snc, y);
+              cfma(ny, sne, x);
+              cp[i] = nx;
+              cq[i] = ny;
+            }
           }
         }
       }
       __syncthreads();
     }
-    if (s_rot == 0) break;
+    if (s_rot == 0) break;       // every cosine of this sweep was rounding noise or nearly so
   }
   // singular values, ordering, truncation
   for (int j = warp; j < kq; j += nw) {
@@ -1018,21 +1373,25 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
 // column-major; T_u itself on the dense path) into the node's region of the scratch
 // buffer Fs, one kCT x kCT tile per CTA (blockIdx.x), the k chunks of Q_u and T_u staged
 // with coalesced loads; recompress_copy then moves it into G_F (Q_u is read from G_F
-// until every tile is done).
+// until every tile is done).  The layer's last recompression, when it covers every node,
+// writes the factor store and its ranks directly (Fs, off, rank_out).
 template <typename R>
 __global__ void __launch_bounds__(256) recompress_gemm(Geo g, const Cx<R>* __restrict__ G_F,
                                                        const int* __restrict__ qcols, const int* __restrict__ qmode,
                                                        const Cx<R>* __restrict__ Tx, const int* __restrict__ newrank,
-                                                       Cx<R>* __restrict__ Fs) {
+                                                       Cx<R>* __restrict__ Fs, const long long* __restrict__ off,
+                                                       int* __restrict__ rank_out) {
+  pdl_begin();
   __shared__ Cx<R> Qs[kCK][kCT + 1], Ts[kCK][kCT + 1];
   const int u = g.list[blockIdx.y];
   const int s = g.sz[u], qc = qcols[u], kr = newrank[u];
+  if (rank_out && blockIdx.x == 0 && threadIdx.x == 0) rank_out[u] = kr;
   const int ni = (s + kCT - 1) / kCT, nj = (kr + kCT - 1) / kCT;
   if ((int)blockIdx.x >= ni * nj) return;
   const int ti = blockIdx.x % ni, tj = blockIdx.x / ni;
   const Cx<R>* Qu = G_F + g.gfo[u];
   const Cx<R>* T = Tx + (long long)u * g.QCAP * g.r_max;
-  Cx<R>* S = Fs + g.gfo[u];
+  Cx<R>* S = Fs + off[u];
   if (qmode[u]) {
     for (int e = threadIdx.x; e < kCT * kCT; e += blockDim.x) {
       const int i = ti * kCT + e % kCT, j = tj * kCT + e / kCT;
@@ -1074,6 +1433,7 @@ __global__ void __launch_bounds__(256) recompress_gemm(Geo g, const Cx<R>* __res
 template <typename R>
 __global__ void recompress_copy(Geo g, const Cx<R>* __restrict__ Fs, const int* __restrict__ newrank,
                                 Cx<R>* __restrict__ G_F, int* __restrict__ G_rank) {
+  pdl_begin();
   const int u = g.list[blockIdx.x];
   const int s = g.sz[u], kr = newrank[u];
   const Cx<R>* S = Fs + g.gfo[u];
@@ -1082,25 +1442,27 @@ __global__ void recompress_copy(Geo g, const Cx<R>* __restrict__ Fs, const int* 
   if (threadIdx.x == 0) G_rank[u] = kr;
 }
 
-// T~_m into the factor store (leaf padding zeroed, factors truncated to r_max columns).
+// T~_m into the factor store (leaf padding zeroed, factors truncated to r_max columns): the
+// first nlb blocks store the leaves, the others the factor of node 2 + blockIdx.x - nlb (none
+// of them when the recompression has stored the factors).
 template <typename R>
-__global__ void store_layer(Geo g, const Cx<R>* __restrict__ G_leaf, const Cx<R>* __restrict__ G_F,
+__global__ void store_layer(Geo g, int nlb, const Cx<R>* __restrict__ G_leaf, const Cx<R>* __restrict__ G_F,
                             const int* __restrict__ G_rank, Cx<R>* __restrict__ dst, const long long* __restrict__ off,
                             int* __restrict__ rank_dst) {
-  const int v = blockIdx.x;   // 0: leaves, v >= 2: factors
-  if (v == 0) {
+  pdl_begin();
+  if ((int)blockIdx.x < nlb) {
     const int lf = g.leaf;
-    const long long tot = (long long)(1 << g.L) * lf * lf;
-    for (long long e = threadIdx.x; e < tot; e += blockDim.x) {
-      const int lam = (1 << g.L) + (int)(e / (lf * lf));
-      const int r = (int)(e % (lf * lf));
+    const int tot = (1 << g.L) * lf * lf;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += nlb * blockDim.x) {
+      const int lam = (1 << g.L) + e / (lf * lf);
+      const int r = e % (lf * lf);
       const int a = r % lf, b = r / lf, s = g.sz[lam];
       dst[e] = (a < s && b < s) ? G_leaf[e] : Cx<R>(0, 0);
     }
-    if (threadIdx.x == 0) { rank_dst[0] = 0; rank_dst[1] = 0; }
+    if (blockIdx.x == 0 && threadIdx.x == 0) { rank_dst[0] = 0; rank_dst[1] = 0; }
     return;
   }
-  if (v < 2) return;
+  const int v = 2 + (int)blockIdx.x - nlb;
   const int s = g.sz[v], r = G_rank[v];
   const Cx<R>* F = G_F + g.gfo[v];
   for (int e = threadIdx.x; e < s * r; e += blockDim.x) dst[off[v] + e] = F[e];
@@ -1129,7 +1491,7 @@ struct SetupWork {
   int* d_rowleaf = nullptr;
   int* d_cap = nullptr;
   int* d_lists = nullptr;
-  void *S_leaf = nullptr, *S_F = nullptr, *G_leaf = nullptr, *G_F = nullptr, *G_F2 = nullptr;
+  void *S_F = nullptr, *G_leaf = nullptr, *G_F = nullptr, *G_F2 = nullptr;
   void *Y = nullptr, *W = nullptr, *Qr = nullptr, *PQ = nullptr, *M = nullptr, *Rb = nullptr;
   void *Tx = nullptr, *Cb = nullptr;
   int *S_rank = nullptr, *G_rank = nullptr, *qcols = nullptr, *qmode = nullptr, *newrank = nullptr;
@@ -1138,7 +1500,7 @@ struct SetupWork {
 void hsw_setup_free(hsweep_s* h) {
   if (!h->sw) return;
   SetupWork* w = h->sw;
-  void* ptrs[] = {w->d_sfo, w->d_gfo, w->d_qro, w->d_rbo, w->d_rowleaf, w->d_cap, w->d_lists, w->S_leaf, w->S_F,
+  void* ptrs[] = {w->d_sfo, w->d_gfo, w->d_qro, w->d_rbo, w->d_rowleaf, w->d_cap, w->d_lists, w->S_F,
                   w->G_leaf, w->G_F, w->G_F2, w->Y, w->W, w->Qr, w->PQ, w->M, w->Rb, w->Tx, w->Cb, w->S_rank,
                   w->G_rank, w->qcols, w->qmode, w->newrank};
   for (void* p : ptrs) hsw_release(h, p);
@@ -1230,7 +1592,6 @@ static int setup_alloc(hsweep_s* h) {
   A(w->d_rowleaf, h->n * sizeof(int));
   A(w->d_cap, nn * sizeof(int));
   A(w->d_lists, std::max<size_t>(1, w->lists.size()) * sizeof(int));
-  A(w->S_leaf, lf2 * es);
   A(w->G_leaf, lf2 * es);
   A(w->S_F, std::max(so, 1LL) * es);
   A(w->G_F, std::max(go, 1LL) * es);
@@ -1260,6 +1621,7 @@ static int setup_alloc(hsweep_s* h) {
     HSW_CUDA(cudaMemcpyAsync(w->d_lists, w->lists.data(), w->lists.size() * sizeof(int), cudaMemcpyHostToDevice,
                              h->stream));
   HSW_CUDA(cudaMemsetAsync(w->S_rank, 0, nn * sizeof(int), h->stream));
+  HSW_CUDA(cudaMemsetAsync(w->G_rank, 0, nn * sizeof(int), h->stream));
   // the host vectors above are read by the asynchronous copies: keep them until the copies ran
   HSW_CUDA(cudaStreamSynchronize(h->stream));
   return HSWEEP_OK;
@@ -1272,11 +1634,11 @@ static int factor_impl(hsweep_s* h) {
   Geo g;
   g.n = h->n; g.L = h->L; g.leaf = h->leaf; g.nnodes = h->nnodes; g.r_max = h->r_max;
   g.KCAP = w->KCAP; g.WCAP = w->WCAP; g.QCAP = w->QCAP; g.dense_max = w->dense_max;
+  g.cap_max = *std::max_element(w->cap.begin(), w->cap.end());
   g.lo = h->d_lo; g.sz = h->d_sz; g.rowleaf = w->d_rowleaf; g.sfo = w->d_sfo; g.gfo = w->d_gfo;
   g.cap = w->d_cap; g.qro = w->d_qro; g.rbo = w->d_rbo; g.list = w->d_lists;
   cudaStream_t st = h->stream;
   Cx<R>* fac = reinterpret_cast<Cx<R>*>(h->d_fac);
-  Cx<R>* S_leaf = (Cx<R>*)w->S_leaf;
   Cx<R>* S_F = (Cx<R>*)w->S_F;
   Cx<R>* G_leaf = (Cx<R>*)w->G_leaf;
   Cx<R>* G_F = (Cx<R>*)w->G_F;
@@ -1290,8 +1652,8 @@ static int factor_impl(hsweep_s* h) {
   Cx<R>* Tx = (Cx<R>*)w->Tx;
   const int L = h->L, nn = h->nnodes, KCAP = w->KCAP, QCAP = w->QCAP;
   const size_t core_smem = (size_t)(2 * KCAP) * (2 * KCAP) * es + 32 * sizeof(R) + (2 * KCAP + 1) * sizeof(int) + 16;
-  // QR: v, c and the reduction scratch, then as many entries of F_u as fit (226 KB in all)
-  const size_t qr_base = ((size_t)(h->tree.maxsz(1) + QCAP) * es + 32 * sizeof(R) + 15) & ~size_t(15);
+  // QR: norms and positions, then as many entries of F_u as fit (226 KB in all)
+  const size_t qr_base = ((size_t)g.cap_max * (2 * sizeof(R) + sizeof(int)) + 15) & ~size_t(15);
   const int qs_entries = qr_base < 226 * 1024 ? (int)((226 * 1024 - qr_base) / es) : 0;
   const size_t qr_smem = qr_base + (size_t)qs_entries * es;
   // the SVD's shared memory: C, two rows of R, norms, singular values and index tables
@@ -1301,16 +1663,19 @@ static int factor_impl(hsweep_s* h) {
   // one shared-memory carveout for every kernel of the layer loop, so that consecutive
   // launches do not reconfigure the SMs' L1/shared split
   {
-    const void* ks[] = {(const void*)schur_leaves<R>, (const void*)schur_factors<R>, (const void*)leaf_inverse<R>,
+    const void* ks[] = {(const void*)schur_layer<R>,
                         (const void*)tsmm_reduce<R>, (const void*)tsmm_expand<R>, (const void*)core_dots<R>,
                         (const void*)core_inverse<R>, (const void*)woodbury_form<R>, (const void*)woodbury_append<R>,
-                        (const void*)qr_cgs2<R>, (const void*)svd_jacobi<R>, (const void*)recompress_gemm<R>,
+                        (const void*)qr_mgs<R>, (const void*)svd_jacobi<R>, (const void*)recompress_gemm<R>,
                         (const void*)recompress_copy<R>, (const void*)store_layer<R>, (const void*)core_product_cc<R>};
     for (const void* k : ks)
       HSW_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   }
+  // (four KCAP x KCAP blocks and tables: also holds the three blocks of core_inverse_block)
   HSW_CUDA(cudaFuncSetAttribute(core_inverse<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)core_smem));
-  HSW_CUDA(cudaFuncSetAttribute(qr_cgs2<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qr_smem));
+  HSW_CUDA(cudaFuncSetAttribute(core_inverse_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)core_smem));
+  HSW_CUDA(cudaFuncSetAttribute(core_inverse_block, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+  HSW_CUDA(cudaFuncSetAttribute(qr_mgs<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qr_smem));
   HSW_CUDA(cudaFuncSetAttribute(svd_jacobi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)svd_smem));
   if (core_smem > 227 * 1024 || qr_smem > 227 * 1024 || svd_smem > 227 * 1024)
     return HSWEEP_ERR_ARG;
@@ -1330,17 +1695,17 @@ static int factor_impl(hsweep_s* h) {
   auto core_product = [&](const Geo& gp, int np_list, int kind) -> int {
     const dim3 grid(core_tiles, np_list);
     const bool f32 = sizeof(R) == 4;
-    auto run = [&](int mode) {
+    auto run = [&](int mode) -> cudaError_t {
       if constexpr (sizeof(R) == 4) {
         if (mode == 1) {
-          core_product_tc<<<grid, 256, 0, st>>>(gp, (const Cx<float>*)Rb, w->qcols, w->G_rank, (Cx<float>*)Cb);
-          return;
+          return pdl_launch(core_product_tc, grid, 256, 0, st, gp, (const Cx<float>*)Rb, w->qcols, w->G_rank,
+                            (Cx<float>*)Cb);
         }
       }
-      core_product_cc<R><<<grid, 256, 0, st>>>(gp, Rb, w->qcols, w->G_rank, Cb);
+      return pdl_launch(core_product_cc<R>, grid, 256, 0, st, gp, Rb, w->qcols, w->G_rank, Cb);
     };
     if (h->opt.core_kernel > 0) {          // fixed by the caller
-      run(f32 && h->opt.core_kernel == 2 ? 1 : 0);
+      HSW_CUDA(run(f32 && h->opt.core_kernel == 2 ? 1 : 0));
       h->nlaunch += 1;
       return HSWEEP_OK;
     }
@@ -1348,9 +1713,9 @@ static int factor_impl(hsweep_s* h) {
       cudaEvent_t ev[3];
       for (auto& e : ev) HSW_CUDA(cudaEventCreate(&e));
       HSW_CUDA(cudaEventRecord(ev[0], st));
-      run(0);
+      HSW_CUDA(run(0));
       HSW_CUDA(cudaEventRecord(ev[1], st));
-      run(1);
+      HSW_CUDA(run(1));
       HSW_CUDA(cudaEventRecord(ev[2], st));
       HSW_CUDA(cudaEventSynchronize(ev[2]));
       float t0 = 0, t1 = 0;
@@ -1363,25 +1728,31 @@ static int factor_impl(hsweep_s* h) {
       h->nlaunch += 2;
       return HSWEEP_OK;
     }
-    run(f32 && h->core_mode[kind] == 1 ? 1 : 0);
+    HSW_CUDA(run(f32 && h->core_mode[kind] == 1 ? 1 : 0));
     h->nlaunch += 1;
     return HSWEEP_OK;
   };
 
   // QR (or the dense path), the cores, their SVD and the new factors, for nn_list nodes
   // whose list starts at node_off and their np_list left siblings at pair_off
-  auto recompress = [&](int node_off, int nn_list, int pair_off, int np_list, int kind) -> int {
+  auto recompress = [&](int node_off, int nn_list, int pair_off, int np_list, int kind, Cx<R>* store = nullptr,
+                        int* store_rank = nullptr) -> int {
     if (nn_list <= 0) return HSWEEP_OK;
     Geo gl = g;
     gl.list = w->d_lists + node_off;
-    qr_cgs2<R><<<nn_list, 1024, qr_smem, st>>>(gl, G_F, w->G_rank, Rb, w->qcols, w->qmode, qs_entries);
+    HSW_CUDA(pdl_launch(qr_mgs<R>, dim3(nn_list), 1024, qr_smem, st, gl, G_F, w->G_rank, Rb, w->qcols, w->qmode, qs_entries));
     Geo gp = g;
     gp.list = w->d_lists + pair_off;
     int rc = core_product(gp, np_list, kind);
     if (rc) return rc;
-    svd_jacobi<R><<<np_list, 1024, svd_smem, st>>>(gp, h->eps_H, Cb, w->qcols, Tx, w->newrank, svd_entries, thr);
-    recompress_gemm<R><<<dim3(gemm_tiles, nn_list), 256, 0, st>>>(gl, G_F, w->qcols, w->qmode, Tx, w->newrank, G_F2);
-    recompress_copy<R><<<nn_list, kBlk, 0, st>>>(gl, G_F2, w->newrank, G_F, w->G_rank);
+    HSW_CUDA(pdl_launch(svd_jacobi<R>, dim3(np_list), 1024, svd_smem, st, gp, h->eps_H, Cb, w->qcols, Tx, w->newrank, svd_entries, thr));
+    if (store) {
+      HSW_CUDA(pdl_launch(recompress_gemm<R>, dim3(gemm_tiles, nn_list), 256, 0, st, gl, G_F, w->qcols, w->qmode, Tx, w->newrank, store, h->d_off, store_rank));
+      h->nlaunch += 3;
+      return HSWEEP_OK;
+    }
+    HSW_CUDA(pdl_launch(recompress_gemm<R>, dim3(gemm_tiles, nn_list), 256, 0, st, gl, G_F, w->qcols, w->qmode, Tx, w->newrank, G_F2, w->d_gfo, (int*)nullptr));
+    HSW_CUDA(pdl_launch(recompress_copy<R>, dim3(nn_list), kBlk, 0, st, gl, G_F2, w->newrank, G_F, w->G_rank));
     h->nlaunch += 4;
     return HSWEEP_OK;
   };
@@ -1391,34 +1762,32 @@ static int factor_impl(hsweep_s* h) {
     m_cur = m;
     const Cx<R>* Tprev = m > 0 ? fac + (long long)(m - 1) * h->layer_stride : nullptr;
     const int* rprev = m > 0 ? h->d_rank + (long long)(m - 1) * nn : nullptr;
-    schur_leaves<R><<<h->nleaves, 64, 0, st>>>(g, m, h->d_diag_m, h->d_east_m, h->d_north_m, Tprev, S_leaf);
-    h->nlaunch += 1;
-    if (nn > 2) {
-      schur_factors<R><<<nn - 2, kBlk, 0, st>>>(g, m, h->d_east_m, h->d_north_m, Tprev, h->d_off, rprev, S_F,
-                                                 w->S_rank);
-      h->nlaunch += 1;
-    }
-    HSW_CUDA(cudaMemsetAsync(w->G_rank, 0, nn * sizeof(int), st));
-    leaf_inverse<R><<<h->nleaves, 128, 0, st>>>(g, m, S_leaf, G_leaf, h->d_status);
+    HSW_CUDA(pdl_launch(schur_layer<R>, dim3(h->nleaves + nn - 2, nn > 2 ? 8 : 1), kBlk, 0, st, g, m, h->d_diag_m,
+                        h->d_east_m, h->d_north_m, Tprev, h->d_off, rprev, S_F, w->S_rank, G_leaf, w->G_rank,
+                        h->d_status));
     h->nlaunch += 1;
     for (int d = L - 1; d >= 0; --d) {
       const int n_below2 = (d + 2 <= L) ? (1 << (L + 1)) - (1 << (d + 2)) : 0;
       const int n_below1 = (1 << (L + 1)) - (1 << (d + 1));
       const int ntau_d = 1 << d;
       if (n_below2 > 0) {
-        tsmm_reduce<R><<<n_below2, kBlk, 0, st>>>(g, d, G_F, w->G_rank, S_F, w->S_rank, Qr);
+        HSW_CUDA(pdl_launch(tsmm_reduce<R>, dim3(n_below2, (KCAP + 7) / 8), kBlk, 0, st, g, d, G_F, w->G_rank, S_F, w->S_rank, Qr));
         h->nlaunch += 1;
       }
-      tsmm_expand<R><<<dim3(div_up(h->n, 128), KCAP), 128, 0, st>>>(g, d, G_leaf, G_F, w->G_rank, S_F,
-                                                                     w->S_rank, Qr, Y);
+      HSW_CUDA(pdl_launch(tsmm_expand<R>, dim3(div_up(h->n, 32), (KCAP + 3) / 4), kBlk, 0, st, g, d, G_leaf, G_F,
+                          w->G_rank, S_F, w->S_rank, Qr, Y));
       h->nlaunch += 1;
-      core_dots<R><<<dim3(2 * ntau_d, 8), kBlk, 0, st>>>(g, d, S_F, w->S_rank, Y, PQ);
+      HSW_CUDA(pdl_launch(core_dots<R>, dim3(2 * ntau_d, std::max(8, 64 / (2 * ntau_d))), kBlk, 0, st, g, d, S_F, w->S_rank, Y, PQ));
       h->nlaunch += 1;
-      core_inverse<R><<<ntau_d, 1024, core_smem, st>>>(g, d, m, w->S_rank, PQ, M, h->d_status);
+      if constexpr (sizeof(R) == 4)
+        HSW_CUDA(pdl_launch(core_inverse_block, dim3(ntau_d), 32 * kCoreWarps, core_smem, st, g, d, m, w->S_rank, PQ, M, h->d_status));
+      else
+        HSW_CUDA(pdl_launch(core_inverse<R>, dim3(ntau_d), 1024, core_smem, st, g, d, m, w->S_rank, PQ, M, h->d_status));
       h->nlaunch += 1;
-      woodbury_form<R><<<dim3(div_up(h->n, 128), KCAP), 128, 0, st>>>(g, d, w->S_rank, Y, M, Wv, G_F, w->G_rank);
+      HSW_CUDA(pdl_launch(woodbury_form<R>, dim3(div_up(h->n, 32), (KCAP + 15) / 16), 128, 0, st, g, d, w->S_rank, Y, M, Wv,
+                          G_F, w->G_rank));
       h->nlaunch += 1;
-      woodbury_append<R><<<n_below1, kBlk, 0, st>>>(g, d, w->S_rank, Y, Wv, G_F, w->G_rank, G_leaf);
+      HSW_CUDA(pdl_launch(woodbury_append<R>, dim3(n_below1), kBlk, 0, st, g, d, w->S_rank, Y, Wv, G_F, w->G_rank, G_leaf));
       h->nlaunch += 1;
       // the blocks of the non-deferred depths that this depth step changed
       int rc = recompress(w->big_nodes_off[d], w->big_nodes_off[d + 1] - w->big_nodes_off[d], w->big_pairs_off[d],
@@ -1426,8 +1795,13 @@ static int factor_impl(hsweep_s* h) {
       if (rc) return rc;
     }
     // the blocks of the deferred depths, once per layer, in their final form
+    Cx<R>* store = fac + (long long)m * h->layer_stride;
+    int* store_rank = h->d_rank + (long long)m * nn;
+    const bool direct = nn > 2 && (h->strong_R > 0 || w->small_nodes == nn - 2);   // the last one covers every node
     {
-      int rc = recompress(w->small_nodes_off, w->small_nodes, w->small_pairs_off, w->small_pairs, 1);
+      const bool last = direct && h->strong_R == 0;
+      int rc = recompress(w->small_nodes_off, w->small_nodes, w->small_pairs_off, w->small_pairs, 1,
+                          last ? store : nullptr, store_rank);
       if (rc) return rc;
     }
     if (h->strong_R > 0) {
@@ -1441,11 +1815,13 @@ static int factor_impl(hsweep_s* h) {
       // the records of the strong sweep, from the exact strongly admissible factors
       rc = hsw_spack_layer(h, m, G_F, G_leaf, w->d_gfo);
       if (rc) return rc;
-      rc = recompress(w->all_nodes_off, w->all_nodes, w->all_pairs_off, w->all_pairs, 1);
+      rc = recompress(w->all_nodes_off, w->all_nodes, w->all_pairs_off, w->all_pairs, 1, direct ? store : nullptr,
+                      store_rank);
       if (rc) return rc;
     }
-    store_layer<R><<<nn, kBlk, 0, st>>>(g, G_leaf, G_F, w->G_rank, fac + (long long)m * h->layer_stride,
-                                        h->d_off, h->d_rank + (long long)m * nn);
+    const int nlb = (int)std::min<long long>(64, div_up(h->leaf_entries, kBlk));
+    HSW_CUDA(pdl_launch(store_layer<R>, dim3(direct ? nlb : nlb + nn - 2), kBlk, 0, st, g, nlb, G_leaf, G_F, w->G_rank, store,
+                        h->d_off, store_rank));
     h->nlaunch += 1;
     HSW_CUDA(cudaGetLastError());
   }

@@ -111,34 +111,6 @@ __host__ __device__ constexpr int slab_stride(int w) {
   return u == 0 ? 0 : (u | 1) * U;
 }
 
-// ---- double <-> float by integer arithmetic ------------------------------------------------
-// The FP64 unit of this GPU also serves the conversions (two lanes a clock and SM): a step's
-// conversions of the coupling row, r and z took longer than its multiply-adds.  Values in
-// FP32's normal range (and zeros) are converted with integer operations, to the same bits.
-__device__ __forceinline__ float to_float(double v) {
-  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-  const unsigned e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
-  if (e - 897u <= 253u) {               // 2^-126 <= |v| < 2^128: round to nearest even
-    unsigned b = __funnelshift_l(lo, hi, 3) - 0xc0000000u;     // exponent bias 1023 -> 127
-    b += ((lo & 0x1fffffffu) + 0x0fffffffu + (b & 1u)) >> 29;
-    return __uint_as_float(b | sign);
-  }
-  if (e < 873u) return __uint_as_float(sign);                  // below half of the least subnormal
-  return (float)v;
-}
-__device__ __forceinline__ double to_double(float v) {
-  const unsigned b = __float_as_uint(v);
-  if (((b >> 23) & 0xffu) - 1u <= 253u)
-    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
-  if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
-  return (double)v;
-}
-template <typename R> __device__ __forceinline__ Cx<R> from_c128(c128 v);
-template <> __device__ __forceinline__ Cx<float> from_c128<float>(c128 v) { return Cx<float>(to_float(v.re), to_float(v.im)); }
-template <> __device__ __forceinline__ Cx<double> from_c128<double>(c128 v) { return v; }
-__device__ __forceinline__ c128 to_c128(Cx<float> v) { return c128(to_double(v.re), to_double(v.im)); }
-__device__ __forceinline__ c128 to_c128(Cx<double> v) { return v; }
-
 // ---- cluster primitives ------------------------------------------------------------------
 __device__ __forceinline__ unsigned mapa(unsigned addr, unsigned rank) {
   unsigned r;
@@ -174,36 +146,6 @@ __device__ __forceinline__ void send2(unsigned addr, Cx<float> v, Cx<float> w, u
 __device__ __forceinline__ void send2(unsigned addr, Cx<double> v, Cx<double> w, unsigned bar) {
   send(addr, v, bar);
   send(addr + 16, w, bar);
-}
-
-// Sum of v[0..G) over the NL lanes that differ in the lane bits UNIT, 2 UNIT, ... NL/2 UNIT,
-// scattered: each step a lane keeps half of its right-hand sides and hands the other half to
-// its partner, so a lane ends with CNT = max(1, G / NL) sums, right-hand sides g .. g+CNT-1.
-// With fewer right-hand sides than lanes the last steps are plain sums (every lane of such a
-// group holds the same value; `first` marks one of them).
-template <typename R, int G, int NL, int UNIT>
-__device__ __forceinline__ void scatter_sum(Cx<R> (&v)[G], int lane, int& g, bool& first) {
-  g = 0;
-  first = true;
-  int cnt = G;
-#pragma unroll
-  for (int o = NL / 2; o > 0; o >>= 1) {
-    const bool up = (lane & (o * UNIT)) != 0;
-    if (cnt > 1) {
-      cnt >>= 1;
-#pragma unroll
-      for (int j = 0; j < G / 2; ++j)
-        if (j < cnt) {
-          const Cx<R> send = up ? v[j] : v[j + cnt];
-          const Cx<R> keep = up ? v[j + cnt] : v[j];
-          v[j] = keep + shfl_xor(send, o * UNIT);
-        }
-      if (up) g += cnt;
-    } else {
-      v[0] += shfl_xor(v[0], o * UNIT);
-      first = first && !up;
-    }
-  }
 }
 
 // V tagged words (16 bytes)
@@ -635,14 +577,14 @@ __global__ void __launch_bounds__(NT, 1) sweep_slab_kernel(SlabArgs<R> a) {
         if (fwd) {
           if (m < n - 1) {
             if (uown) a.w[pos] = y;
-            xn = from_c128<R>(in_r) - cpl * y;
+            xn = cvt<R>(in_r) - cpl * y;
           } else {
-            if (uown) a.z[pos] = to_c128(y);
+            if (uown) a.z[pos] = cvt<double>(y);
             xn = cpl * y;
           }
         } else {
           const Cx<R> uu = uown ? in_w - y : Cx<R>(0, 0);
-          if (uown) a.z[pos] = to_c128(uu);
+          if (uown) a.z[pos] = cvt<double>(uu);
           xn = cpl * uu;
         }
         x[urow * GS + ug] = xn;
