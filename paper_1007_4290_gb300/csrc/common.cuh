@@ -115,6 +115,72 @@ __device__ __forceinline__ void scatter_sum(Cx<R> (&v)[G], int lane, int& g, boo
   }
 }
 
+// Reciprocal and reciprocal square root, in complex128 by two Newton steps from the FP32
+// value (a handful of FP64 operations where the division and square root routines take
+// dozens: a warp's FP64 instruction occupies its scheduler for about 64 clocks here)
+__device__ __forceinline__ float rcp_of(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rcp_of(double x) {
+  // for x well inside FP32's range
+  double y = (double)(1.0f / (float)x);
+  y = y * fma(-x, y, 2.0);
+  return y * fma(-x, y, 2.0);
+}
+__device__ __forceinline__ float rsqrt_of(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsqrt_of(double x) {
+  double y = (double)rsqrtf((float)x);
+  const double h = 0.5 * x;
+  y = y * fma(-h * y, y, 1.5);
+  return y * fma(-h * y, y, 1.5);
+}
+
+// the same for any positive normal x: its exponent is taken out first
+__device__ __forceinline__ float rcp_any(float x) { return 1.0f / x; }
+__device__ __forceinline__ float rsqrt_any(float x) { return 1.0f / sqrtf(x); }
+__device__ __forceinline__ double rcp_any(double x) {
+  const int e = ((__double2hiint(x) >> 20) & 0x7ff) - 1023;
+  const double s = __hiloint2double((1023 - e) << 20, 0);       // 2^-e
+  return rcp_of(x * s) * s;
+}
+__device__ __forceinline__ double rsqrt_any(double x) {
+  const int q = (((__double2hiint(x) >> 20) & 0x7ff) - 1023) >> 1;
+  const double s = __hiloint2double((1023 - q) << 20, 0);       // 2^-q
+  return rsqrt_of(x * s * s) * s;
+}
+// The rotation of one-sided Jacobi for columns p, q with squared norms al, be (at least about
+// 1e-28 of the largest column's) and inner product ga = <p, q>:
+//     p' = cs p - conj(sne) q,  q' = cs q + sne p,  |p'|^2 = al - dn, |q'|^2 = be + dn.
+// gg = |ga|^2 / (al be).  The angle comes from FP32 reciprocal square roots in both precisions
+// (its error only leaves an inner product smaller by 1e-7, and the convergence does the rest);
+// cs and the phase are refined to the storage precision.
+template <typename R>
+struct JacobiRotation {
+  float gg;
+  R cs, dn;
+  Cx<R> sne;
+  __device__ __forceinline__ bool needed(R al, R be, Cx<R> ga, float tol2) {
+    s = R(rsqrtf((float)al)) * R(rsqrtf((float)be));
+    gn = s * ga;
+    gg = (float)abs2(gn);
+    return gg > tol2;
+  }
+  __device__ __forceinline__ void angle(R al, R be) {
+    const float ig = rsqrtf(gg);
+    const float z = 0.5f * (float)((be - al) * s) * ig;
+    // (z reaches 1e29 in complex128, where its square would overflow)
+    const float za = fabsf(z), tt = copysignf(1.0f, z) / (za + (za < 1e9f ? sqrtf(fmaf(z, z, 1.0f)) : za));
+    const R tr = (R)tt;
+    cs = rsqrt_of(fma(tr, tr, R(1)));
+    R igr = (R)ig;
+    if (sizeof(R) == 8) igr = igr * fma(R(-0.5) * abs2(gn) * igr, igr, R(1.5));
+    sne = (tr * cs * igr) * gn;
+    dn = tr * (abs2(gn) * igr * rcp_of(s));
+  }
+
+ private:
+  R s;
+  Cx<R> gn;
+};
+
 // L2-only loads/stores for data exchanged between CTAs of one sweep team.
 template <typename R> __device__ __forceinline__ Cx<R> ld_cg(const Cx<R>* p);
 template <> __device__ __forceinline__ Cx<float> ld_cg(const Cx<float>* p) {

@@ -44,7 +44,7 @@ constexpr int kDenseRows = 128;
 template <typename R> struct Tiny;
 template <> struct Tiny<double> {
   static constexpr double dep = 1e-13;    // Gram-Schmidt: dependent-column threshold
-  static constexpr double jac = 1e-15;    // Jacobi: orthogonality tolerance (about 8 ulp)
+  static constexpr float jac2 = 1e-30f;   // Jacobi: orthogonality tolerance 1e-15 (about 8 ulp), squared
   static constexpr double neg = 1e-28;    // Jacobi: squared norm of a rounding-noise column
                                           // (normalised: below 1e-14 of the largest column)
   static constexpr float quad = 1e-16f;   // Jacobi: squared cosine from which one more sweep
@@ -53,7 +53,7 @@ template <> struct Tiny<double> {
 };
 template <> struct Tiny<float> {
   static constexpr float dep = 2e-6f;
-  static constexpr float jac = 4e-7f;     // about 7 ulp: tighter only rotates rounding noise
+  static constexpr float jac2 = 1.6e-13f; // (4e-7)^2, about 7 ulp: tighter only rotates rounding noise
   static constexpr float neg = 1e-14f;    // below 1e-7 of the largest column: FP32 noise
   static constexpr float quad = 1e-8f;
 };
@@ -79,37 +79,6 @@ template <typename R> __device__ R block_sum(R v, R* red) {
   return t;
 }
 
-// Reciprocal and reciprocal square root, in complex128 by two Newton steps from the FP32
-// value (a handful of FP64 operations where the division and square root routines take
-// dozens: a warp's FP64 instruction occupies its scheduler for about 64 clocks here)
-__device__ __forceinline__ float rcp_of(float x) { return 1.0f / x; }
-__device__ __forceinline__ double rcp_of(double x) {
-  // for x well inside FP32's range
-  double y = (double)(1.0f / (float)x);
-  y = y * fma(-x, y, 2.0);
-  return y * fma(-x, y, 2.0);
-}
-__device__ __forceinline__ float rsqrt_of(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_of(double x) {
-  double y = (double)rsqrtf((float)x);
-  const double h = 0.5 * x;
-  y = y * fma(-h * y, y, 1.5);
-  return y * fma(-h * y, y, 1.5);
-}
-
-// the same for any positive normal x: its exponent is taken out first
-__device__ __forceinline__ float rcp_any(float x) { return 1.0f / x; }
-__device__ __forceinline__ float rsqrt_any(float x) { return 1.0f / sqrtf(x); }
-__device__ __forceinline__ double rcp_any(double x) {
-  const int e = ((__double2hiint(x) >> 20) & 0x7ff) - 1023;
-  const double s = __hiloint2double((1023 - e) << 20, 0);       // 2^-e
-  return rcp_of(x * s) * s;
-}
-__device__ __forceinline__ double rsqrt_any(double x) {
-  const int q = (((__double2hiint(x) >> 20) & 0x7ff) - 1023) >> 1;
-  const double s = __hiloint2double((1023 - q) << 20, 0);       // 2^-q
-  return rsqrt_of(x * s * s) * s;
-}
 // 1 / a, by the Newton reciprocal where |a|^2 is well inside FP32's range
 __device__ __forceinline__ c128 cinv_fast(c128 a) {
   const double d = abs2(a);
@@ -823,6 +792,9 @@ __global__ void woodbury_append(Geo g, int d, const int* __restrict__ S_rank, co
 }
 
 // ---------------------------------------------------------------------------------
+// lanes per column of the Gram-Schmidt steps
+template <typename R> __host__ __device__ constexpr int group_lanes() { return sizeof(R) == 8 ? 8 : 32; }
+
 // Recompression, step 1, for the nodes u = list[blockIdx.x]: with w = rank(u) columns,
 // a factor with at least as many columns as rows (w >= sz(u)), or in complex64 of at most
 // kDenseRows rows, takes the dense path, Q = I and R = F_u (qcols = sz(u), qmode = 1);
@@ -875,6 +847,7 @@ __global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, c
     if (lane == 0) cur[j] = org[j] = acc;
   }
   __syncthreads();
+  constexpr int kGL = group_lanes<R>(), kCPW = 32 / kGL;
   int qc = 0;
   for (int j = 0; j < w; ++j) {
     const R nr = cur[j];
@@ -882,21 +855,25 @@ __global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, c
     if (kept) {
       const R inv = rcp_any(nr), rs = rsqrt_any(nr), nn = nr * rs;
       const Cx<R>* cj = Fq + (long long)j * s;
-      for (int l = j + 1 + warp; l < w; l += nw) {
-        Cx<R>* cl = Fq + (long long)l * s;
+      for (int lb = j + 1 + warp * kCPW; lb < w; lb += nw * kCPW) {
+        const int l = lb + lane / kGL, gl = lane % kGL;
+        const bool act = l < w;
+        Cx<R>* cl = Fq + (long long)(act ? l : j) * s;
         Cx<R> d(0, 0);
-        for (int i = lane; i < s; i += 32) cfma_conj(d, cj[i], cl[i]);
-        for (int o = 16; o > 0; o >>= 1) d += shfl_xor(d, o);
+        if (act)
+          for (int i = gl; i < s; i += kGL) cfma_conj(d, cj[i], cl[i]);
+        for (int o = kGL / 2; o > 0; o >>= 1) d += shfl_xor(d, o);
         const Cx<R> be = -(inv * d);
         R acc = 0;
-        for (int i = lane; i < s; i += 32) {
-          Cx<R> v = cl[i];
-          cfma(v, be, cj[i]);
-          cl[i] = v;
-          acc = fma(v.re, v.re, fma(v.im, v.im, acc));
-        }
-        acc = warp_sum_r(acc);
-        if (lane == 0) {
+        if (act)
+          for (int i = gl; i < s; i += kGL) {
+            Cx<R> v = cl[i];
+            cfma(v, be, cj[i]);
+            cl[i] = v;
+            acc = fma(v.re, v.re, fma(v.im, v.im, acc));
+          }
+        for (int o = kGL / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (act && gl == 0) {
           cur[l] = acc;
           Rm[(long long)qc * ld + l] = rs * d;
         }
@@ -924,9 +901,11 @@ __global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, c
 // precision) and, in complex64, core_product_tc on tensor cores; the setup times both on
 // a layer of representative ranks and keeps the faster for each kind of recompression
 // launch (factor_impl).
-constexpr int kCT = 32;    // tile edge in complex entries
+// tile edge in complex entries; in complex128 a quarter of the tile per CTA (FP64 units)
+template <typename R> __host__ __device__ constexpr int core_tile_edge() { return sizeof(R) == 8 ? 16 : 32; }
 constexpr int kCK = 16;    // complex k chunk staged in shared memory
 
+template <int kCT>
 __device__ __forceinline__ bool core_tile(int qa, int qb, int tile, int& ti, int& tj) {
   const int ni = (qa + kCT - 1) / kCT, nj = (qb + kCT - 1) / kCT;
   if (tile >= ni * nj) return false;
@@ -935,25 +914,26 @@ __device__ __forceinline__ bool core_tile(int qa, int qb, int tile, int& ti, int
   return true;
 }
 
-// 256 threads: thread (tx, ty) of a 16 x 16 grid owns rows ty, ty + 16 and columns tx,
-// tx + 16 of the tile; the k chunks of R_a and R_b are staged with coalesced loads
+// 256 threads: thread (tx, ty) of a 16 x 16 grid owns rows ty (+ 16) and columns tx (+ 16)
+// of the tile; the k chunks of R_a and R_b are staged with coalesced loads
 template <typename R>
 __global__ void __launch_bounds__(256) core_product_cc(Geo g, const Cx<R>* __restrict__ Rb,
                                                        const int* __restrict__ qcols, const int* __restrict__ G_rank,
                                                        Cx<R>* __restrict__ Cb) {
   pdl_begin();
+  constexpr int kCT = core_tile_edge<R>(), U = kCT / 16;
   __shared__ Cx<R> As[kCK][kCT + 1], Bs[kCK][kCT + 1];
   const int a = g.list[blockIdx.y], b = a + 1;
   const int qa = qcols[a], qb = qcols[b], w = G_rank[a];
   int ti, tj;
-  if (!core_tile(qa, qb, blockIdx.x, ti, tj)) return;
+  if (!core_tile<kCT>(qa, qb, blockIdx.x, ti, tj)) return;
   const Cx<R>* Ra = Rb + g.rbo[a];
   const Cx<R>* Rbb = Rb + g.rbo[b];
   const int lda = g.cap[a], ldb = g.cap[b];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  Cx<R> acc[2][2];
-  for (int u = 0; u < 2; ++u)
-    for (int v = 0; v < 2; ++v) acc[u][v] = Cx<R>(0, 0);
+  Cx<R> acc[U][U];
+  for (int u = 0; u < U; ++u)
+    for (int v = 0; v < U; ++v) acc[u][v] = Cx<R>(0, 0);
   for (int k0 = 0; k0 < w; k0 += kCK) {
     for (int e = threadIdx.x; e < kCK * kCT; e += blockDim.x) {
       const int kk = e % kCK, r = e / kCK;
@@ -963,18 +943,16 @@ __global__ void __launch_bounds__(256) core_product_cc(Geo g, const Cx<R>* __res
     }
     __syncthreads();
 #pragma unroll 4
-    for (int kk = 0; kk < kCK; ++kk) {
-      const Cx<R> a0 = As[kk][ty], a1 = As[kk][ty + 16], b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-      cfma(acc[0][0], a0, b0);
-      cfma(acc[0][1], a0, b1);
-      cfma(acc[1][0], a1, b0);
-      cfma(acc[1][1], a1, b1);
-    }
+    for (int kk = 0; kk < kCK; ++kk)
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < U; ++v) cfma(acc[u][v], As[kk][ty + 16 * u], Bs[kk][tx + 16 * v]);
     __syncthreads();
   }
   Cx<R>* C = Cb + (long long)(a >> 1) * g.QCAP * g.QCAP;
-  for (int u = 0; u < 2; ++u)
-    for (int v = 0; v < 2; ++v) {
+  for (int u = 0; u < U; ++u)
+    for (int v = 0; v < U; ++v) {
       const int i = ti * kCT + ty + 16 * u, j = tj * kCT + tx + 16 * v;
       if (i < qa && j < qb) C[(long long)j * qa + i] = acc[u][v];
     }
@@ -1003,11 +981,12 @@ __global__ void __launch_bounds__(256) core_product_tc(Geo g, const Cx<float>* _
                                                        const int* __restrict__ qcols, const int* __restrict__ G_rank,
                                                        Cx<float>* __restrict__ Cb) {
   pdl_begin();
+  constexpr int kCT = core_tile_edge<float>();
   __shared__ Cx<float> As[kCT][kCK + 1], Bs[kCT][kCK + 1];
   const int a = g.list[blockIdx.y], b = a + 1;
   const int qa = qcols[a], qb = qcols[b], w = G_rank[a];
   int ti, tj;
-  if (!core_tile(qa, qb, blockIdx.x, ti, tj)) return;
+  if (!core_tile<kCT>(qa, qb, blockIdx.x, ti, tj)) return;
   const Cx<float>* Ra = Rb + g.rbo[a];
   const Cx<float>* Rbb = Rb + g.rbo[b];
   const int lda = g.cap[a], ldb = g.cap[b];
@@ -1147,6 +1126,7 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
     if (lane == 0) nrm[j] = iscale * iscale * nrm[j];
   }
   __syncthreads();
+  constexpr int kGL = group_lanes<R>(), kCPW = 32 / kGL;
   // ---- 1. pivoted Gram-Schmidt -----------------------------------------------------------
   int kq = 0;
   const int kmax = min(qa, qb);
@@ -1166,30 +1146,29 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
     if (!(best > thr)) break;
     const R rs = rsqrt_of(best), ib = rcp_of(best);
     const Cx<R>* cp = C + p * ld;
-    for (int j = warp; j < qb; j += nw) {
-      if (j == p || nr[j] < 0) {
-        if (lane == 0) {
-          nx[j] = R(-1);
-          rk[j] = Cx<R>(j == p ? best * rs : R(0), R(0));
-        }
-        continue;
-      }
-      Cx<R>* cj = C + j * ld;
+    // kGL lanes a column: a warp in complex64, eight lanes in complex128 (an FP64 instruction
+    // costs the same whatever the number of columns it serves)
+    for (int jb = warp * kCPW; jb < qb; jb += nw * kCPW) {
+      const int j = jb + lane / kGL, gl = lane % kGL;
+      const bool in = j < qb, act = in && j != p && nr[in ? j : 0] >= 0;
+      Cx<R>* cj = C + (act ? j : 0) * ld;
       Cx<R> d(0, 0);
-      for (int i = lane; i < qa; i += 32) cfma_conj(d, cp[i], cj[i]);
-      for (int o = 16; o > 0; o >>= 1) d += shfl_xor(d, o);
+      if (act)
+        for (int i = gl; i < qa; i += kGL) cfma_conj(d, cp[i], cj[i]);
+      for (int o = kGL / 2; o > 0; o >>= 1) d += shfl_xor(d, o);
       const Cx<R> be = -(ib * d);
       R acc = 0;
-      for (int i = lane; i < qa; i += 32) {
-        Cx<R> v = cj[i];
-        cfma(v, be, cp[i]);
-        cj[i] = v;
-        acc = fma(v.re, v.re, fma(v.im, v.im, acc));
-      }
-      acc = warp_sum_r(acc);
-      if (lane == 0) {
-        nx[j] = acc;
-        rk[j] = rs * conj(d);
+      if (act)
+        for (int i = gl; i < qa; i += kGL) {
+          Cx<R> v = cj[i];
+          cfma(v, be, cp[i]);
+          cj[i] = v;
+          acc = fma(v.re, v.re, fma(v.im, v.im, acc));
+        }
+      for (int o = kGL / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (in && gl == 0) {
+        nx[j] = act ? acc : R(-1);
+        rk[j] = act ? rs * conj(d) : Cx<R>(j == p ? best * rs : R(0), R(0));
       }
     }
     // the row of the step before into the storage of its pivot column (read by nobody now)
@@ -1209,8 +1188,11 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
   // ---- 2. one-sided Jacobi on the kq columns (length qb) of L ------------------------------
   const int me = kq + (kq & 1);               // even number of positions (one dummy if odd)
   // one group of GW lanes per column pair: whole warps while there are at most as many
-  // pairs as warps, half warps beyond (every pair of a round in one pass)
-  const int GW = (me / 2 <= nw) ? 32 : 16;
+  // pairs as warps, half warps beyond (every pair of a round in one pass); in complex128 as
+  // many pairs to a warp as keep four warps busy, one a scheduler's FP64 unit
+  int GW = (me / 2 <= nw) ? 32 : 16;
+  if (sizeof(R) == 8)
+    while (GW > 4 && me / 2 * GW > 128) GW >>= 1;
   const int gpw = 32 / GW;                    // groups per warp
   for (int sweep = 0; sweep < 40; ++sweep) {
     __syncthreads();
@@ -1259,27 +1241,15 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
           for (int i = gl; i < qb; i += GW) cfma_conj(ga, cp[i], cq[i]);
         }
         ga = group_sum(ga, GW);
-        // g = <p, q> / (|p| |q|): the angle's cotangent 2 z = (|q|^2 - |p|^2) / |<p, q>|
-        const float ra = rsqrtf((float)al), rb = rsqrtf((float)be);
-        const R s = R(ra) * R(rb);
-        const Cx<R> gn = s * ga;
-        const float gg = (float)abs2(gn);
-        const bool rot = live && al >= thr && be >= thr && gg > (float)(Tiny<R>::jac * Tiny<R>::jac);
-        if (rot) {
-          if (gl == 0 && gg > Tiny<R>::quad) s_rot = 1;
-          const float ig = rsqrtf(gg);
-          const float z = 0.5f * (float)((be - al) * s) * ig;
-          // (z reaches 1e29 in complex128, where its square would overflow)
-          const float za = fabsf(z), tt = copysignf(1.0f, z) / (za + (za < 1e9f ? sqrtf(fmaf(z, z, 1.0f)) : za));
-          const R tr = (R)tt;
-          const R cs = rsqrt_of(fma(tr, tr, R(1))), sn = tr * cs;
-          R igr = (R)ig;
-          if (sizeof(R) == 8) igr = igr * fma(R(-0.5) * abs2(gn) * igr, igr, R(1.5));
-          const Cx<R> sne = (sn * igr) * gn, snc = conj(sne);
+        JacobiRotation<R> rot;
+        if (rot.needed(al, be, ga, Tiny<R>::jac2) && live && al >= thr && be >= thr) {
+          rot.angle(al, be);
+          const R cs = rot.cs;
+          const Cx<R> sne = rot.sne, snc = conj(sne);
           if (gl == 0) {
-            const R ag = tr * (abs2(gn) * igr * rcp_of(s));
-            sig[ip] = fmax(R(0), al - ag);
-            sig[iq] = be + ag;
+            if (rot.gg > Tiny<R>::quad) s_rot = 1;
+            sig[ip] = fmax(R(0), al - rot.dn);
+            sig[iq] = be + rot.dn;
           }
           if (reg) {
             if constexpr (sizeof(R) == 4) {
@@ -1382,6 +1352,7 @@ __global__ void __launch_bounds__(256) recompress_gemm(Geo g, const Cx<R>* __res
                                                        Cx<R>* __restrict__ Fs, const long long* __restrict__ off,
                                                        int* __restrict__ rank_out) {
   pdl_begin();
+  constexpr int kCT = core_tile_edge<R>(), U = kCT / 16;
   __shared__ Cx<R> Qs[kCK][kCT + 1], Ts[kCK][kCT + 1];
   const int u = g.list[blockIdx.y];
   const int s = g.sz[u], qc = qcols[u], kr = newrank[u];
@@ -1400,9 +1371,9 @@ __global__ void __launch_bounds__(256) recompress_gemm(Geo g, const Cx<R>* __res
     return;
   }
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  Cx<R> acc[2][2];
-  for (int a = 0; a < 2; ++a)
-    for (int b = 0; b < 2; ++b) acc[a][b] = Cx<R>(0, 0);
+  Cx<R> acc[U][U];
+  for (int a = 0; a < U; ++a)
+    for (int b = 0; b < U; ++b) acc[a][b] = Cx<R>(0, 0);
   for (int k0 = 0; k0 < qc; k0 += kCK) {
     for (int e = threadIdx.x; e < kCK * kCT; e += blockDim.x) {
       const int r = e % kCT, kq = e / kCT;          // Q: consecutive threads, consecutive rows
@@ -1414,17 +1385,15 @@ __global__ void __launch_bounds__(256) recompress_gemm(Geo g, const Cx<R>* __res
     }
     __syncthreads();
 #pragma unroll 4
-    for (int kk = 0; kk < kCK; ++kk) {
-      const Cx<R> a0 = Qs[kk][ty], a1 = Qs[kk][ty + 16], b0 = Ts[kk][tx], b1 = Ts[kk][tx + 16];
-      cfma(acc[0][0], a0, b0);
-      cfma(acc[0][1], a0, b1);
-      cfma(acc[1][0], a1, b0);
-      cfma(acc[1][1], a1, b1);
-    }
+    for (int kk = 0; kk < kCK; ++kk)
+#pragma unroll
+      for (int a = 0; a < U; ++a)
+#pragma unroll
+        for (int b = 0; b < U; ++b) cfma(acc[a][b], Qs[kk][ty + 16 * a], Ts[kk][tx + 16 * b]);
     __syncthreads();
   }
-  for (int a = 0; a < 2; ++a)
-    for (int b = 0; b < 2; ++b) {
+  for (int a = 0; a < U; ++a)
+    for (int b = 0; b < U; ++b) {
       const int i = ti * kCT + ty + 16 * a, j = tj * kCT + tx + 16 * b;
       if (i < s && j < kr) S[(long long)j * s + i] = acc[a][b];
     }
@@ -1688,6 +1657,7 @@ static int factor_impl(hsweep_s* h) {
   // SVD: columns below a fraction of the truncation threshold (squared, relative) are left out:
   // a quarter in complex64 (rounding noise lies just below), a twentieth in complex128
   const R thr = (R)std::max((double)Tiny<R>::neg, (sizeof(R) == 4 ? 0.0625 : 0.0025) * h->eps_H * h->eps_H);
+  constexpr int kCT = core_tile_edge<R>();
   const int core_tiles = ((QCAP + kCT - 1) / kCT) * ((QCAP + kCT - 1) / kCT);
   const int gemm_tiles = ((h->tree.maxsz(1) + kCT - 1) / kCT) * ((h->r_max + kCT - 1) / kCT);
   Cx<R>* Cb = (Cx<R>*)w->Cb;

@@ -10,8 +10,8 @@
 //     the weak form, S(u, w) = F_a[rows u] F_b[rows w]^t; its rank-R approximation comes
 //     from the randomized SVD (Halko, Martinsson and Tropp; the paper uses it for
 //     F = H . H): Y = S Omega with P = R + 8 Gaussian test vectors, Q = orth(Y),
-//     B = Q^* S, and the dominant R-dimensional left singular subspace of B (Hermitian
-//     Jacobi on B B^*) gives S ~ (Q V) (V^* B).  The near-field blocks (neighbouring
+//     B = Q^* S, and the dominant right singular vectors P of B (one-sided Jacobi) give
+//     S ~ S P P^*.  The near-field blocks (neighbouring
 //     leaves) are formed densely;
 //   expansion: the strong matrix is written back into the sibling-pair factor store
 //     without approximation.  Inside a sibling block (a, b) the well-separated blocks
@@ -60,7 +60,8 @@ __host__ __device__ void hsw_philox4x32_10(const uint32_t ctr[4], const uint32_t
 namespace {
 
 // Two complex standard normals (real and imaginary parts independent N(0, 1)) from one
-// Philox block, by the Box-Muller transform.
+// Philox block, by the Box-Muller transform, in the precision that stores them (the FP64
+// logarithms and sines took longer than the products with the test vectors).
 template <typename R>
 __device__ inline void gauss2(uint32_t row, uint32_t pair, uint32_t blk, uint32_t m, uint32_t seed, Cx<R>& z0,
                               Cx<R>& z1) {
@@ -68,15 +69,20 @@ __device__ inline void gauss2(uint32_t row, uint32_t pair, uint32_t blk, uint32_
   const uint32_t key[2] = {seed, 0x5EEDu};
   uint32_t x[4];
   hsw_philox4x32_10(ctr, key, x);
-  const double s = 2.3283064365386963e-10;   // 2^-32
-  const double u0 = ((double)x[0] + 0.5) * s, u1 = (double)x[1] * s;
-  const double u2 = ((double)x[2] + 0.5) * s, u3 = (double)x[3] * s;
-  const double r0 = sqrt(-2.0 * log(u0)), r1 = sqrt(-2.0 * log(u2));
-  double s0, c0, s1, c1;
-  sincospi(2.0 * u1, &s0, &c0);
-  sincospi(2.0 * u3, &s1, &c1);
-  z0 = Cx<R>(R(r0 * c0), R(r0 * s0));
-  z1 = Cx<R>(R(r1 * c1), R(r1 * s1));
+  const R s = R(2.3283064365386963e-10);   // 2^-32
+  const R u0 = (R(x[0]) + R(0.5)) * s, u1 = R(x[1]) * s;
+  const R u2 = (R(x[2]) + R(0.5)) * s, u3 = R(x[3]) * s;
+  const R r0 = sqrt(R(-2) * log(u0)), r1 = sqrt(R(-2) * log(u2));
+  R s0, c0, s1, c1;
+  if constexpr (sizeof(R) == 4) {
+    sincospif(2.0f * u1, &s0, &c0);
+    sincospif(2.0f * u3, &s1, &c1);
+  } else {
+    sincospi(2.0 * u1, &s0, &c0);
+    sincospi(2.0 * u3, &s1, &c1);
+  }
+  z0 = Cx<R>(r0 * c0, r0 * s0);
+  z1 = Cx<R>(r1 * c1, r1 * s1);
 }
 
 struct FarArgs {
@@ -86,34 +92,76 @@ struct FarArgs {
   const long long* soff;    // [nblk] scratch offset (entries): Omega/Bt (sw x P), then Y/Q (su x P)
   const long long* gfo;     // factor offsets per node
   const int* sz;            // node sizes
+  int shared;               // the scratch of every block fits in dynamic shared memory
 };
 
-template <typename R>
-__device__ inline R block_sum(R v, R* red) {
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  R t = 0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-  return t;
+// Z[p][c] (ld kKMax) = sum_r F[r, c] v_p[r] (CONJ: conj(v_p[r])), c < k, p < np: a warp per
+// column c and eight vectors
+template <bool CONJ, typename R>
+__device__ __forceinline__ void columns_dot(const Cx<R>* __restrict__ F, int ldf, int k, const Cx<R>* V, int rows, int np,
+                                            Cx<R>* Z) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int pg = (np + 7) / 8;
+  for (int e = warp; e < k * pg; e += nw) {
+    const int c = e / pg, p0 = 8 * (e % pg);
+    Cx<R> acc[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc[u] = Cx<R>(0, 0);
+    for (int r = lane; r < rows; r += 32) {
+      const Cx<R> f = F[(long long)c * ldf + r];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const Cx<R> v = V[min(p0 + u, np - 1) * rows + r];
+        if (CONJ) cfma_conj(acc[u], v, f);
+        else cfma(acc[u], v, f);
+      }
+    }
+    int u;
+    bool first;
+    scatter_sum<R, 8, 32, 1>(acc, lane, u, first);
+    if (first && p0 + u < np) Z[(p0 + u) * kKMax + c] = acc[0];
+  }
+}
+
+// put(r, p, sum_c F[r, c] Z[p][c]) for r < rows, p < np: a thread per row and four vectors
+template <typename R, typename Put>
+__device__ __forceinline__ void rows_times(const Cx<R>* __restrict__ F, int ldf, int k, const Cx<R>* Z, int rows, int np,
+                                           Put put) {
+  const int pg = (np + 3) / 4;
+  for (int e = threadIdx.x; e < rows * pg; e += blockDim.x) {
+    const int r = e % rows, p0 = 4 * (e / rows);
+    Cx<R> acc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u] = Cx<R>(0, 0);
+#pragma unroll 4
+    for (int c = 0; c < k; ++c) {
+      const Cx<R> f = F[(long long)c * ldf + r];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cfma(acc[u], f, Z[min(p0 + u, np - 1) * kKMax + c]);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (p0 + u < np) put(r, p0 + u, acc[u]);
+  }
 }
 
 // One CTA per well-separated block: randomized rank-R projection, written into the
-// expanded factors of the sibling pair (a, b) that contains it.
+// expanded factors of the sibling pair (a, b) that contains it.  The basis of the sampled
+// range comes from two rounds of right-looking Gram-Schmidt (a warp per later column, one
+// barrier a step); the dominant right singular vectors of B = Q^* S from one-sided Jacobi on
+// the columns of B^t (a warp per pair); and the left factor from the product of S with them,
+// so that the result is the projection S P P^* whatever the basis.  What bounds it is the
+// latency of these short chains; with classical Gram-Schmidt (a block-wide sum per inner
+// product) and FP64 Jacobi on the Gram matrix by one warp it took 850 us a layer at n = 255.
 template <typename R>
-__global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, int m, double eps, const Cx<R>* __restrict__ F,
+__global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, int m, R eps, const Cx<R>* __restrict__ F,
                                                        const int* __restrict__ rank, Cx<R>* __restrict__ Fout,
                                                        Cx<R>* __restrict__ scratch) {
+  extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ Cx<R> Z[kKMax * kPMax];
-  __shared__ double Gre[kPMax * kPMax], Gim[kPMax * kPMax];
-  __shared__ double Vre[kPMax * kPMax], Vim[kPMax * kPMax];
-  __shared__ double lam[kPMax], scl[kPMax];
-  __shared__ int order[kPMax];
-  __shared__ Cx<R> coef[kPMax];
-  __shared__ R red[32];
-  __shared__ int s_q, s_keep;
+  __shared__ R cur[kPMax], org[kPMax], sig[kPMax];
+  __shared__ int kept[kPMax], order[kPMax];
+  __shared__ int s_rot, s_keep;
 
   const int bi = blockIdx.x;
   const int* inf = fa.info + 8 * bi;
@@ -121,201 +169,192 @@ __global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, int m, double
   const int k = rank[a];
   if (k <= 0) return;
   const int P = fa.P, tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31, nw = kThreads / 32;
   const int lda = fa.sz[a], ldb = fa.sz[b];
   const Cx<R>* Fa = F + fa.gfo[a] + ru0;
   const Cx<R>* Fb = F + fa.gfo[b] + rw0;
-  Cx<R>* Om = scratch + fa.soff[bi];          // sw x P (Omega, later Bt), column-major
-  Cx<R>* Y = Om + (long long)sw * P;          // su x P (Y, then Q), column-major
+  Cx<R>* Om = fa.shared ? reinterpret_cast<Cx<R>*>(dyn) : scratch + fa.soff[bi];   // sw x P (Omega, later Bt)
+  Cx<R>* Y = Om + sw * P;                                                            // su x P (Y, then Q)
 
   // Omega: complex Gaussian test vectors
   for (int e = tid; e < sw * (P / 2); e += blockDim.x) {
     const int row = e % sw, pr = e / sw;
     Cx<R> z0, z1;
     gauss2<R>((uint32_t)row, (uint32_t)pr, (uint32_t)bi, (uint32_t)m, fa.seed, z0, z1);
-    Om[(long long)(2 * pr) * sw + row] = z0;
-    Om[(long long)(2 * pr + 1) * sw + row] = z1;
+    Om[(2 * pr) * sw + row] = z0;
+    Om[(2 * pr + 1) * sw + row] = z1;
   }
   __syncthreads();
-  // Z = F_b[rows w]^t Omega  (k x P)
-  for (int e = tid; e < k * P; e += blockDim.x) {
-    const int c = e % k, p = e / k;
-    Cx<R> acc(0, 0);
-    for (int r = 0; r < sw; ++r) cfma(acc, Fb[(long long)c * ldb + r], Om[(long long)p * sw + r]);
-    Z[p * kKMax + c] = acc;
-  }
+  // Y = S Omega = F_a[rows u] (F_b[rows w]^t Omega)
+  columns_dot<false>(Fb, ldb, k, Om, sw, P, Z);
   __syncthreads();
-  // Y = F_a[rows u] Z  (su x P)
-  for (int e = tid; e < su * P; e += blockDim.x) {
-    const int r = e % su, p = e / su;
-    Cx<R> acc(0, 0);
-    for (int c = 0; c < k; ++c) cfma(acc, Fa[(long long)c * lda + r], Z[p * kKMax + c]);
-    Y[(long long)p * su + r] = acc;
-  }
+  rows_times(Fa, lda, k, Z, su, P, [&](int r, int p, Cx<R> v) { Y[p * su + r] = v; });
   __syncthreads();
-  // Q = orth(Y): classical Gram-Schmidt applied twice, dependent columns dropped
+  // Q = orth(Y), dependent columns dropped; the second round restores the orthogonality the
+  // first one lost on columns with small remainders
   const R keep_tol = sizeof(R) == 4 ? R(1e-5) : R(1e-12);
-  if (tid == 0) s_q = 0;
-  __syncthreads();
-  for (int j = 0; j < P; ++j) {
-    const int q = s_q;
-    Cx<R>* y = Y + (long long)j * su;
-    R n0 = 0;
-    for (int r = tid; r < su; r += blockDim.x) n0 += abs2(y[r]);
-    n0 = block_sum(n0, red);
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int i = 0; i < q; ++i) {
-        Cx<R> acc(0, 0);
-        for (int r = tid; r < su; r += blockDim.x) cfma_conj(acc, Y[(long long)i * su + r], y[r]);
-        const R re = block_sum(acc.re, red);
-        const R im = block_sum(acc.im, red);
-        if (tid == 0) coef[i] = Cx<R>(re, im);
-      }
-      __syncthreads();
-      for (int r = tid; r < su; r += blockDim.x) {
-        Cx<R> v = y[r];
-        for (int i = 0; i < q; ++i) v -= coef[i] * Y[(long long)i * su + r];
-        y[r] = v;
-      }
-      __syncthreads();
+  int q = 0;
+  for (int round = 0; round < 2; ++round) {
+    const int nc = round == 0 ? P : q;
+    for (int j = warp; j < nc; j += nw) {
+      const Cx<R>* y = Y + (round == 0 ? j : kept[j]) * su;
+      R acc = 0;
+      for (int r = lane; r < su; r += 32) acc += abs2(y[r]);
+      for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) cur[j] = org[j] = acc;
     }
-    R n1 = 0;
-    for (int r = tid; r < su; r += blockDim.x) n1 += abs2(y[r]);
-    n1 = block_sum(n1, red);
-    if (n1 > keep_tol * keep_tol * n0 && n1 > R(0)) {
-      const R inv = R(1) / sqrt(n1);
-      Cx<R>* dst = Y + (long long)q * su;
-      for (int r = tid; r < su; r += blockDim.x) dst[r] = inv * y[r];
+    __syncthreads();
+    int qn = 0;
+    for (int j = 0; j < nc; ++j) {
+      const R nr = cur[j];
+      const bool keep = round == 1 || (nr > keep_tol * keep_tol * org[j] && nr > R(0));
+      const int src = round == 0 ? j : kept[j];
+      if (keep) {
+        const Cx<R>* yj = Y + src * su;
+        const R inv = rcp_any(nr);
+        for (int l = j + 1 + warp; l < nc; l += nw) {
+          Cx<R>* yl = Y + (round == 0 ? l : kept[l]) * su;
+          Cx<R> d(0, 0);
+          for (int r = lane; r < su; r += 32) cfma_conj(d, yj[r], yl[r]);
+          for (int o = 16; o; o >>= 1) d += shfl_xor(d, o);
+          const Cx<R> be = -(inv * d);
+          R acc = 0;
+          for (int r = lane; r < su; r += 32) {
+            Cx<R> v = yl[r];
+            cfma(v, be, yj[r]);
+            yl[r] = v;
+            acc += abs2(v);
+          }
+          for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+          if (lane == 0) cur[l] = acc;
+        }
+      }
       __syncthreads();
-      if (tid == 0) s_q = q + 1;
+      if (keep) {
+        if (round == 0 && tid == 0) kept[qn] = j;
+        ++qn;
+      }
+    }
+    q = qn;
+    __syncthreads();
+    // normalise (after the first round, the kept columns' norms again)
+    for (int j = warp; j < q; j += nw) {
+      Cx<R>* y = Y + kept[j] * su;
+      const R rs = rsqrt_any(cur[round == 0 ? kept[j] : j]);
+      for (int r = lane; r < su; r += 32) y[r] = rs * y[r];
     }
     __syncthreads();
   }
-  const int q = s_q;
   if (q == 0) return;
-  // Z2 = F_a[rows u]^t conj(Q)  (k x q)
-  for (int e = tid; e < k * q; e += blockDim.x) {
-    const int c = e % k, p = e / k;
-    Cx<R> acc(0, 0);
-    for (int r = 0; r < su; ++r) cfma_conj(acc, Y[(long long)p * su + r], Fa[(long long)c * lda + r]);
-    Z[p * kKMax + c] = acc;
+  // the kept columns side by side (a column never lies before its place)
+  for (int j = 0; j < q; ++j) {
+    const int src = kept[j];
+    if (src != j)
+      for (int r = tid; r < su; r += blockDim.x) Y[j * su + r] = Y[src * su + r];
+    __syncthreads();
+  }
+  // Bt = (Q^* S)^t = F_b[rows w] (F_a[rows u]^t conj(Q))  (sw x q), over Omega
+  columns_dot<true>(Fa, lda, k, Y, su, q, Z);
+  __syncthreads();
+  rows_times(Fb, ldb, k, Z, sw, q, [&](int r, int p, Cx<R> v) { Om[p * sw + r] = v; });
+  __syncthreads();
+  // one-sided Jacobi on the q columns of Bt, scaled by the largest: Bt W = P Sigma
+  for (int j = warp; j < q; j += nw) {
+    R acc = 0;
+    for (int r = lane; r < sw; r += 32) acc += abs2(Om[j * sw + r]);
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) sig[j] = acc;
   }
   __syncthreads();
-  // Bt = F_b[rows w] Z2 = (Q^* S)^t  (sw x q), over Omega
-  for (int e = tid; e < sw * q; e += blockDim.x) {
-    const int r = e % sw, p = e / sw;
-    Cx<R> acc(0, 0);
-    for (int c = 0; c < k; ++c) cfma(acc, Fb[(long long)c * ldb + r], Z[p * kKMax + c]);
-    Om[(long long)p * sw + r] = acc;
-  }
+  R scale2 = 0;
+  for (int j = 0; j < q; ++j) scale2 = fmax(scale2, sig[j]);
+  if (!(scale2 > R(0))) return;
+  const R iscale = rsqrt_any(scale2);
+  const R floor2 = sizeof(R) == 4 ? R(1e-14) : R(1e-28);
+  const float tol2 = sizeof(R) == 4 ? 1.6e-13f : 1e-30f, quad = sizeof(R) == 4 ? 1e-8f : 1e-16f;
   __syncthreads();
-  // Gram matrix B B^* (q x q, Hermitian), FP64
-  for (int e = tid; e < q * q; e += blockDim.x) {
-    const int p = e % q, r = e / q;
-    double re = 0, im = 0;
-    for (int x = 0; x < sw; ++x) {
-      const Cx<R> u = Om[(long long)p * sw + x], v = Om[(long long)r * sw + x];
-      re += (double)u.re * v.re + (double)u.im * v.im;
-      im += (double)u.im * v.re - (double)u.re * v.im;
-    }
-    Gre[p * kPMax + r] = re;
-    Gim[p * kPMax + r] = im;
-    Vre[p * kPMax + r] = p == r ? 1.0 : 0.0;
-    Vim[p * kPMax + r] = 0.0;
-  }
-  __syncthreads();
-  // cyclic Jacobi on the Hermitian Gram matrix, one warp: U = diag(1, e^{-i phi}) J with the
-  // real symmetric Schur rotation J, G <- U^* G U, V <- V U
-  if (tid < 32) {
-    const int x = tid;
-    for (int sweep = 0; sweep < 30; ++sweep) {
-      double off = 0, dia = 0;
-      for (int e = x; e < q * q; e += 32) {
-        const int p = e % q, r = e / q;
-        const double v2 = Gre[p * kPMax + r] * Gre[p * kPMax + r] + Gim[p * kPMax + r] * Gim[p * kPMax + r];
-        if (p == r) dia += v2; else off += v2;
-      }
-      for (int o = 16; o; o >>= 1) {
-        off += __shfl_xor_sync(0xffffffffu, off, o);
-        dia += __shfl_xor_sync(0xffffffffu, dia, o);
-      }
-      if (!(off > 1e-30 * dia)) break;
-      for (int p = 0; p < q - 1; ++p)
-        for (int r = p + 1; r < q; ++r) {
-          const double gr = Gre[p * kPMax + r], gi = Gim[p * kPMax + r];
-          const double ag = sqrt(gr * gr + gi * gi);
-          const double ap = Gre[p * kPMax + p], ar = Gre[r * kPMax + r];
-          if (!(ag > 1e-18 * sqrt(fabs(ap * ar)) && ag > 1e-300)) continue;
-          const double tau = (ar - ap) / (2.0 * ag);
-          const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-          const double c = 1.0 / sqrt(1.0 + t * t), s = t * c;
-          const double er = gr / ag, ei = gi / ag;           // e^{i phi}
-          __syncwarp();
-          if (x < q) {     // columns p, r: col_p' = c col_p - s e^{-i phi} col_r, col_r' = s col_p + c e^{-i phi} col_r
-            const double pr_ = Gre[x * kPMax + p], pi_ = Gim[x * kPMax + p];
-            const double rr_ = Gre[x * kPMax + r], ri_ = Gim[x * kPMax + r];
-            const double er_r = rr_ * er + ri_ * ei, er_i = ri_ * er - rr_ * ei;   // e^{-i phi} col_r
-            Gre[x * kPMax + p] = c * pr_ - s * er_r; Gim[x * kPMax + p] = c * pi_ - s * er_i;
-            Gre[x * kPMax + r] = s * pr_ + c * er_r; Gim[x * kPMax + r] = s * pi_ + c * er_i;
-            const double vpr = Vre[x * kPMax + p], vpi = Vim[x * kPMax + p];
-            const double vrr = Vre[x * kPMax + r], vri = Vim[x * kPMax + r];
-            const double vr_r = vrr * er + vri * ei, vr_i = vri * er - vrr * ei;
-            Vre[x * kPMax + p] = c * vpr - s * vr_r; Vim[x * kPMax + p] = c * vpi - s * vr_i;
-            Vre[x * kPMax + r] = s * vpr + c * vr_r; Vim[x * kPMax + r] = s * vpi + c * vr_i;
-          }
-          __syncwarp();
-          if (x < q) {     // rows p, r: row_p' = c row_p - s e^{i phi} row_r, row_r' = s row_p + c e^{i phi} row_r
-            const double pr_ = Gre[p * kPMax + x], pi_ = Gim[p * kPMax + x];
-            const double rr_ = Gre[r * kPMax + x], ri_ = Gim[r * kPMax + x];
-            const double er_r = rr_ * er - ri_ * ei, er_i = ri_ * er + rr_ * ei;   // e^{i phi} row_r
-            Gre[p * kPMax + x] = c * pr_ - s * er_r; Gim[p * kPMax + x] = c * pi_ - s * er_i;
-            Gre[r * kPMax + x] = s * pr_ + c * er_r; Gim[r * kPMax + x] = s * pi_ + c * er_i;
-          }
-          __syncwarp();
+  for (int e = tid; e < sw * q; e += blockDim.x) Om[e] = iscale * Om[e];
+  const int me = q + (q & 1);
+  for (int sweep = 0; sweep < 30; ++sweep) {
+    __syncthreads();
+    if (tid == 0) s_rot = 0;
+    __syncthreads();
+    for (int round = 0; round < me - 1; ++round) {
+      for (int pr = warp; pr < me / 2; pr += nw) {
+        const int p1 = me - 1 - pr;
+        const int ip = pr == 0 ? 0 : (pr - 1 + round) % (me - 1) + 1, iq = (p1 - 1 + round) % (me - 1) + 1;
+        if (ip >= q || iq >= q) continue;
+        Cx<R>* cp = Om + min(ip, iq) * sw;
+        Cx<R>* cq = Om + max(ip, iq) * sw;
+        R al = 0, be = 0;
+        Cx<R> ga(0, 0);
+        for (int r = lane; r < sw; r += 32) {
+          const Cx<R> x = cp[r], y = cq[r];
+          al += abs2(x);
+          be += abs2(y);
+          cfma_conj(ga, x, y);
         }
-    }
-    if (x == 0) {
-      for (int p = 0; p < q; ++p) { lam[p] = Gre[p * kPMax + p]; order[p] = p; }
-      for (int p = 1; p < q; ++p)
-        for (int r = p; r > 0 && lam[order[r]] > lam[order[r - 1]]; --r) {
-          const int t = order[r]; order[r] = order[r - 1]; order[r - 1] = t;
+        for (int o = 16; o; o >>= 1) {
+          al += __shfl_xor_sync(0xffffffffu, al, o);
+          be += __shfl_xor_sync(0xffffffffu, be, o);
+          ga += shfl_xor(ga, o);
         }
-      const double floor_rel = sizeof(R) == 4 ? 1e-12 : 1e-28;
-      const double thr = lam[order[0]] * fmax(eps * eps, floor_rel);
-      int keep = 0;
-      while (keep < fa.R && keep < q && lam[order[keep]] > thr && lam[order[keep]] > 0) {
-        scl[keep] = sqrt(sqrt(lam[order[keep]]));     // sigma^(1/2): balanced factors
-        ++keep;
+        if (!(al >= floor2 && be >= floor2)) continue;
+        JacobiRotation<R> rot;
+        if (!rot.needed(al, be, ga, tol2)) continue;
+        rot.angle(al, be);
+        if (lane == 0 && rot.gg > quad) s_rot = 1;
+        for (int r = lane; r < sw; r += 32) {
+          const Cx<R> x = cp[r], y = cq[r];
+          Cx<R> nx = rot.cs * x, ny = rot.cs * y;
+          cfma(nx, -conj(rot.sne), y);
+          cfma(ny, rot.sne, x);
+          cp[r] = nx;
+          cq[r] = ny;
+        }
       }
-      s_keep = keep;
+      __syncthreads();
     }
+    if (s_rot == 0) break;
+  }
+  for (int j = warp; j < q; j += nw) {
+    R acc = 0;
+    for (int r = lane; r < sw; r += 32) acc += abs2(Om[j * sw + r]);
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) sig[j] = acc;
+  }
+  if (tid == 0) s_keep = 0;
+  __syncthreads();
+  if (tid < q) {
+    int rk = 0;
+    R smax = 0;
+    for (int l = 0; l < q; ++l) {
+      rk += (sig[l] > sig[tid] || (sig[l] == sig[tid] && l < tid)) ? 1 : 0;
+      smax = fmax(smax, sig[l]);
+    }
+    order[rk] = tid;
+    const R floor_rel = sizeof(R) == 4 ? R(1e-12) : R(1e-27);     // clear of the columns left unrotated
+    if (rk < fa.R && sig[tid] > smax * fmax(eps * eps, floor_rel)) atomicMax(&s_keep, rk + 1);
   }
   __syncthreads();
   const int keep = s_keep;
-  // left = Q V[:, kept] sigma^(1/2) -> F'_a[rows u]; right = Bt conj(V[:, kept]) sigma^(-1/2) -> F'_b[rows w]
+  // F'_b[rows w] = P Sigma^(1/2), F'_a[rows u] = S conj(P) Sigma^(-1/2); column i of Om is
+  // P sigma / scale, sigma = scale sqrt(sig)
+  const R scale = scale2 * iscale;
   Cx<R>* Oa = Fout + fa.gfo[a] + ru0;
   Cx<R>* Ob = Fout + fa.gfo[b] + rw0;
-  for (int e = tid; e < su * keep; e += blockDim.x) {
-    const int r = e % su, i = e / su, oi = order[i];
-    double re = 0, im = 0;
-    for (int p = 0; p < q; ++p) {
-      const Cx<R> y = Y[(long long)p * su + r];
-      const double vr = Vre[p * kPMax + oi], vi = Vim[p * kPMax + oi];
-      re += y.re * vr - y.im * vi;
-      im += y.re * vi + y.im * vr;
-    }
-    Oa[(long long)(col + i) * lda + r] = Cx<R>(R(re * scl[i]), R(im * scl[i]));
-  }
   for (int e = tid; e < sw * keep; e += blockDim.x) {
-    const int r = e % sw, i = e / sw, oi = order[i];
-    double re = 0, im = 0;
-    for (int p = 0; p < q; ++p) {
-      const Cx<R> y = Om[(long long)p * sw + r];
-      const double vr = Vre[p * kPMax + oi], vi = -Vim[p * kPMax + oi];
-      re += y.re * vr - y.im * vi;
-      im += y.re * vi + y.im * vr;
-    }
-    Ob[(long long)(col + i) * ldb + r] = Cx<R>(R(re / scl[i]), R(im / scl[i]));
+    const int r = e % sw, i = e / sw;
+    const R sg = sqrt(sig[order[i]]);
+    Ob[(long long)(col + i) * ldb + r] = sqrt(scale / sg) * Om[order[i] * sw + r];
   }
+  __syncthreads();
+  for (int i = 0; i < keep; ++i) columns_dot<true>(Fb, ldb, k, Om + order[i] * sw, sw, 1, Z + i * kKMax);
+  __syncthreads();
+  rows_times(Fa, lda, k, Z, su, keep, [&](int r, int i, Cx<R> v) {
+    const R sg = sqrt(sig[order[i]]);
+    Oa[(long long)(col + i) * lda + r] = (R(1) / (sg * sqrt(scale * sg))) * v;
+  });
 }
 
 struct NearArgs {
@@ -360,6 +399,7 @@ struct StrongWork {
   int* d_near = nullptr;
   int* d_rank = nullptr;        // expanded rank per node
   void* scratch = nullptr;
+  size_t smem = 0;              // dynamic shared memory for the largest block's vectors (0: scratch)
 };
 
 int hsw_strong_expansion_rank(int R, int L, int leaf) { return 3 * R * (L > 0 ? L - 1 : 0) + leaf; }
@@ -409,10 +449,14 @@ static int strong_prepare(hsweep_s* h, size_t es) {
     if (nrank[v] > h->r_max) return HSWEEP_ERR_ARG;
   std::vector<long long> soff;
   long long so = 0;
+  size_t most = 0;
   for (size_t i = 0; i < far.size(); i += 8) {
+    most = std::max(most, (size_t)(far[i + 4] + far[i + 5]) * s->P * es);
     soff.push_back(so);
     so += (long long)(far[i + 4] + far[i + 5]) * s->P;
   }
+  // (Z and the tables take up to 15 KB of static shared memory beside it)
+  s->smem = most <= 160 * 1024 ? most : 0;
   s->nfar = (int)soff.size();
   s->nnear = (int)(near.size() / 6);
   int rc;
@@ -456,7 +500,10 @@ static int project_impl(hsweep_s* h, int m, const Cx<R>* G_F, int* G_rank, Cx<R>
     FarArgs fa;
     fa.nblk = s->nfar; fa.R = h->strong_R; fa.P = s->P; fa.seed = h->opt.rsvd_seed;
     fa.info = s->d_far; fa.soff = s->d_soff; fa.gfo = d_gfo; fa.sz = h->d_sz;
-    strong_far<R><<<s->nfar, kThreads, 0, st>>>(fa, m, h->eps_H, G_F, G_rank, G_F2, (Cx<R>*)s->scratch);
+    fa.shared = s->smem > 0;
+    if (s->smem > 0)
+      HSW_CUDA(cudaFuncSetAttribute(strong_far<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->smem));
+    strong_far<R><<<s->nfar, kThreads, s->smem, st>>>(fa, m, (R)h->eps_H, G_F, G_rank, G_F2, (Cx<R>*)s->scratch);
     h->nlaunch += 1;
   }
   if (s->nnear > 0) {
