@@ -47,25 +47,31 @@ __global__ void assemble_kernel(int n, double h, double eta, double pref, double
   diag[p] = k2 - (((e_l + e_r) + n_l) + n_r);
 }
 
-// y[s] = A x[s] (f null) or the residual y[s] = f[s] - A x[s], for right-hand sides
-// s0 .. s0 + 7: one thread per node, the five coefficients loaded once (negated for the
-// residual), the 8 x 5 neighbour values of all eight right-hand sides in flight together
+// true when every bit but the sign of x is zero (an integer test: an FP64 comparison takes the
+// FP64 unit, which bounds this kernel)
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
+
+// y[s] = A x[s] (RES false) or the residual y[s] = f[s] - A x[s], for right-hand sides
+// s0 .. s0 + 7: one thread per node, the five coefficients loaded once (the residual's sign is
+// an operand modifier of the multiply-adds), the 8 x 5 neighbour values of all eight
+// right-hand sides in flight together.  FP64 multiply-adds bound it (half a lane a clock and
+// scheduler): ten per node and right-hand side where the coefficients are real.
 constexpr int kMvRhs = 8;
-template <typename T>
+template <typename T, bool RES>
 __global__ void matvec_kernel(int n, long long N, int nrhs, const c128* __restrict__ diag,
                               const c128* __restrict__ east, const c128* __restrict__ north,
                               const c128* __restrict__ x, c128* __restrict__ y, const c128* __restrict__ f) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= N) return;
-  const int j = (int)(p / n), i = (int)(p - (long long)j * n);
+  const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;      // N < 2^30
+  if (p >= (unsigned)N) return;
+  const int j = (int)(p / (unsigned)n), i = (int)(p - (unsigned)j * n);
   const int s0 = blockIdx.y * kMvRhs;
   const c128 zero(0.0, 0.0);
-  const T sg = f ? T(-1) : T(1);
-  const Cx<T> d = sg * cvt<T>(diag[p]);
-  const Cx<T> el = sg * cvt<T>(i > 0 ? east[(long long)j * (n + 1) + i] : zero);
-  const Cx<T> er = sg * cvt<T>(i < n - 1 ? east[(long long)j * (n + 1) + i + 1] : zero);
-  const Cx<T> nl = sg * cvt<T>(j > 0 ? north[(long long)j * n + i] : zero);
-  const Cx<T> nr = sg * cvt<T>(j < n - 1 ? north[(long long)(j + 1) * n + i] : zero);
+  const Cx<T> d = cvt<T>(diag[p]);
+  const Cx<T> el = cvt<T>(i > 0 ? east[(long long)j * (n + 1) + i] : zero);
+  const Cx<T> er = cvt<T>(i < n - 1 ? east[(long long)j * (n + 1) + i + 1] : zero);
+  const Cx<T> nl = cvt<T>(j > 0 ? north[(long long)j * n + i] : zero);
+  const Cx<T> nr = cvt<T>(j < n - 1 ? north[(long long)(j + 1) * n + i] : zero);
   const long long pl = i > 0 ? p - 1 : p, pr = i < n - 1 ? p + 1 : p;
   const long long pd = j > 0 ? p - n : p, pu = j < n - 1 ? p + n : p;
   Cx<T> v[kMvRhs][5];
@@ -80,34 +86,31 @@ __global__ void matvec_kernel(int n, long long N, int nrhs, const c128* __restri
       v[u][4] = cvt<T>(xs[pu]);
     }
   }
+  // acc +- a b
+  auto madd = [](T a, T b, T acc) { return RES ? fma(-a, b, acc) : fma(a, b, acc); };
   // away from the PML every coefficient is real: complex x real multiply-adds give the
-  // same values with half the FP64 operations (FP64 throughput bounds this kernel)
-  const bool real_coef = d.im == 0.0 && el.im == 0.0 && er.im == 0.0 && nl.im == 0.0 && nr.im == 0.0;
-  if (real_coef) {
-#pragma unroll
-    for (int u = 0; u < kMvRhs; ++u) {
-      if (s0 + u < nrhs) {
-        const Cx<T> f0 = f ? cvt<T>(f[(long long)(s0 + u) * N + p]) : Cx<T>(0, 0);
-        T re = fma(d.re, v[u][0].re, f0.re), im = fma(d.re, v[u][0].im, f0.im);
-        re = fma(el.re, v[u][1].re, re); im = fma(el.re, v[u][1].im, im);
-        re = fma(er.re, v[u][2].re, re); im = fma(er.re, v[u][2].im, im);
-        re = fma(nl.re, v[u][3].re, re); im = fma(nl.re, v[u][3].im, im);
-        re = fma(nr.re, v[u][4].re, re); im = fma(nr.re, v[u][4].im, im);
-        y[(long long)(s0 + u) * N + p] = c128(re, im);
-      }
-    }
-    return;
-  }
+  // same values with half the FP64 operations
+  const bool real_coef = is_zero(d.im) && is_zero(el.im) && is_zero(er.im) && is_zero(nl.im) && is_zero(nr.im);
+  const Cx<T> co[5] = {d, el, er, nl, nr};
 #pragma unroll
   for (int u = 0; u < kMvRhs; ++u) {
     if (s0 + u < nrhs) {
-      Cx<T> acc = f ? cvt<T>(f[(long long)(s0 + u) * N + p]) : Cx<T>(0, 0);
-      cfma(acc, d, v[u][0]);
-      cfma(acc, el, v[u][1]);
-      cfma(acc, er, v[u][2]);
-      cfma(acc, nl, v[u][3]);
-      cfma(acc, nr, v[u][4]);
-      y[(long long)(s0 + u) * N + p] = cvt<double>(acc);
+      const Cx<T> f0 = RES ? cvt<T>(f[(long long)(s0 + u) * N + p]) : Cx<T>(0, 0);
+      T re = f0.re, im = f0.im;
+      if (real_coef) {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          re = madd(co[k].re, v[u][k].re, re);
+          im = madd(co[k].re, v[u][k].im, im);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          re = madd(co[k].re, v[u][k].re, madd(-co[k].im, v[u][k].im, re));
+          im = madd(co[k].re, v[u][k].im, madd(co[k].im, v[u][k].re, im));
+        }
+      }
+      y[(long long)(s0 + u) * N + p] = cvt<double>(Cx<T>(re, im));
     }
   }
 }
@@ -129,12 +132,9 @@ int hsw_assemble(hsweep_s* h, double pml_C, int pml_form, int pml_sides, c128* d
 static int matvec_launch(hsweep_s* h, const c128* x, c128* y, const c128* f, int nrhs, bool lowp) {
   if (nrhs <= 0) return HSWEEP_OK;
   dim3 grid(div_up(h->N, 256), div_up(nrhs, kMvRhs));
-  if (lowp)
-    matvec_kernel<float><<<grid, 256, 0, h->stream>>>(h->n, (long long)h->N, nrhs, h->d_diag, h->d_east,
-                                                      h->d_north, x, y, f);
-  else
-    matvec_kernel<double><<<grid, 256, 0, h->stream>>>(h->n, (long long)h->N, nrhs, h->d_diag, h->d_east,
-                                                       h->d_north, x, y, f);
+  auto kern = lowp ? (f ? matvec_kernel<float, true> : matvec_kernel<float, false>)
+                   : (f ? matvec_kernel<double, true> : matvec_kernel<double, false>);
+  kern<<<grid, 256, 0, h->stream>>>(h->n, (long long)h->N, nrhs, h->d_diag, h->d_east, h->d_north, x, y, f);
   h->nlaunch += 1;
   HSW_CUDA(cudaGetLastError());
   return HSWEEP_OK;

@@ -25,7 +25,12 @@
 
 namespace {
 
-constexpr int kRedBlocks = 304;   // 2 x 152 SMs of partial sums per vector
+constexpr int kRedBlocks = 304;   // at most 2 x 152 SMs of partial sums per vector
+
+// Blocks per vector of the reductions: all of kRedBlocks for a few vectors, fewer for a batch,
+// down to 32 (the sums across a warp are FP64 additions too: with 304 blocks for each of 64
+// vectors of 1023 x 1023 they cost half as much as the products)
+static int red_blocks(int nvec) { return std::max(32, std::min(kRedBlocks, 2432 / std::max(1, nvec))); }
 
 constexpr int kDotChunk = 4;      // basis vectors per pass over w
 
@@ -69,11 +74,11 @@ __global__ void dots_kernel(const c128* const* __restrict__ V, int nv, int nt, c
     }
     c128 acc[kDotChunk];
 #pragma unroll
-    for (int i = 0; i < kDotChunk; ++i) {
-      acc[i] = cvt<double>(acct[i]);
-      for (int o = 16; o > 0; o >>= 1) acc[i] += shfl_xor(acc[i], o);
-      if ((threadIdx.x & 31) == 0) red[i][threadIdx.x >> 5] = acc[i];
-    }
+    for (int i = 0; i < kDotChunk; ++i) acc[i] = cvt<double>(acct[i]);
+    int lane_i;
+    bool first;
+    scatter_sum<double, kDotChunk, 32, 1>(acc, threadIdx.x & 31, lane_i, first);   // a lane ends with output lane_i
+    if (first) red[lane_i][threadIdx.x >> 5] = acc[0];
     __syncthreads();
     if (threadIdx.x < nc) {
       c128 t(0, 0);
@@ -293,10 +298,11 @@ static int batched_dots(hsweep_s* h, int first, int nv, const c128* w, int nrhs,
                         bool lowp, bool with_norm = false) {
   KrylovWork* k = h->kw;
   const int nt = nv + (with_norm ? 1 : 0);
-  if (lowp) dots_kernel<float><<<dim3(kRedBlocks, nrhs), 256, 0, h->stream>>>(k->d_V + first, nv, nt, w, h->N, k->partial);
-  else dots_kernel<double><<<dim3(kRedBlocks, nrhs), 256, 0, h->stream>>>(k->d_V + first, nv, nt, w, h->N, k->partial);
+  const int B = red_blocks(nrhs);
+  if (lowp) dots_kernel<float><<<dim3(B, nrhs), 256, 0, h->stream>>>(k->d_V + first, nv, nt, w, h->N, k->partial);
+  else dots_kernel<double><<<dim3(B, nrhs), 256, 0, h->stream>>>(k->d_V + first, nv, nt, w, h->N, k->partial);
   h->nlaunch += 1;
-  reduce_partials<<<nrhs * nt, 256, 0, h->stream>>>(k->partial, kRedBlocks, k->dots);
+  reduce_partials<<<nrhs * nt, 256, 0, h->stream>>>(k->partial, B, k->dots);
   h->nlaunch += 1;
   HSW_CUDA(cudaGetLastError());
   hd.resize((size_t)nrhs * nt);
@@ -306,10 +312,11 @@ static int batched_dots(hsweep_s* h, int first, int nv, const c128* w, int nrhs,
 // ||x[s]|| for every s, on the host
 static int norms(hsweep_s* h, const c128* x, int nrhs, std::vector<double>& out, bool lowp = false) {
   KrylovWork* k = h->kw;
-  if (lowp) sqnorm_kernel<float><<<dim3(kRedBlocks, nrhs), 256, 0, h->stream>>>(x, h->N, k->partial);
-  else sqnorm_kernel<double><<<dim3(kRedBlocks, nrhs), 256, 0, h->stream>>>(x, h->N, k->partial);
+  const int B = red_blocks(nrhs);
+  if (lowp) sqnorm_kernel<float><<<dim3(B, nrhs), 256, 0, h->stream>>>(x, h->N, k->partial);
+  else sqnorm_kernel<double><<<dim3(B, nrhs), 256, 0, h->stream>>>(x, h->N, k->partial);
   h->nlaunch += 1;
-  reduce_partials<<<nrhs, 256, 0, h->stream>>>(k->partial, kRedBlocks, k->dots);
+  reduce_partials<<<nrhs, 256, 0, h->stream>>>(k->partial, B, k->dots);
   h->nlaunch += 1;
   HSW_CUDA(cudaGetLastError());
   std::vector<std::complex<double>> hd(nrhs);
