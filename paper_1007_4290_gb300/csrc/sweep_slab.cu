@@ -33,8 +33,8 @@
 // for this CTA's messages of step t + 1, which were sent after step t was read.  (Every pair
 // of CTAs exchanges at least one column in every step: empty blocks get a zero column.)
 // Bulk copies bring the next layer's F (two stages) and D (two, or one when shared memory
-// is short: D is free from the second barrier on).  The update's global inputs are loaded
-// one step ahead into registers.
+// is short: D is free from the second barrier on).  The update's global inputs are copied
+// one step ahead into shared memory.
 //
 // Clusters of 16 CTAs are at most seven at a time (one per GPC with 16 free SMs), and the
 // receive buffer grows with G.  Where more teams fit side by side without clusters (n = 1023
@@ -42,9 +42,13 @@
 // and exchanges tagged words through L2 (sweep_team.cu's protocol; L2X below).
 //
 // Measured (random media, eps_H 1e-6), per step, against the team sweep of sweep_team.cu:
-// complex64, n = 511: 2.25 us with one right-hand side (5.0), 3.2 with 16 (5.6), 5.6 with 64
-// (7.5); n = 1023: 3.2 with one (6.2), 5.8 with 16 (7.2), 9.4 with 64 (12.4); complex128, n =
-// 255: 5.3 with one (8.6).
+// complex64, n = 511: 2.0 us with one right-hand side (5.0), 2.9 with 16 (5.6), 4.5 with 64
+// (7.5); n = 1023: 2.8 with one (6.2), 4.3 with 16 (7.2), 7.7 with 64 (12.4); complex128, n =
+// 255: 5.1 with one (8.6).  What a step takes is instruction latency: with one right-hand
+// side 600 instructions a warp at one in four clocks and scheduler; with eight about 5 us of
+// FP32 multiply-adds and shared-memory reads.  Not kept: two half-CTAs with four right-hand
+// sides each on the same stages (register spills: 10.2 us against 8.0), and the paired FP32
+// instruction in the tiles (77 % of the FP32 rate where plain multiply-adds reach 88 %).
 #include <algorithm>
 #include <cstdlib>
 #include <type_traits>
@@ -132,9 +136,6 @@ __device__ __forceinline__ void send(unsigned addr, Cx<double> v, unsigned bar) 
                "l"((u64)__double_as_longlong(v.re)), "l"((u64)__double_as_longlong(v.im)), "r"(bar)
                : "memory");
 }
-// keeps the compiler from moving work on v above this point
-__device__ __forceinline__ void pin(Cx<float>& v) { asm volatile("" : "+f"(v.re), "+f"(v.im)); }
-__device__ __forceinline__ void pin(Cx<double>& v) { asm volatile("" : "+d"(v.re), "+d"(v.im)); }
 // two neighbouring complex64 values, 16-byte aligned
 __device__ __forceinline__ void send2(unsigned addr, Cx<float> v, Cx<float> w, unsigned bar) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
@@ -187,10 +188,11 @@ struct SlabArgs {
   long long wait_limit;         // iterations of the waits for other CTAs
   int withhold;                 // test only: this CTA never arrives (-1: none)
   unsigned o_F[2], o_D[2], o_x, o_q, o_p[2], o_y, o_bar, o_meta;
+  unsigned o_in, o_inc;         // the update's inputs: r or w of every (row, rhs), couplings of every row
 };
 
 template <typename R, int G, int RA, int CS, int NT, bool L2X>
-__global__ void __launch_bounds__(NT, 1) sweep_slab_kernel(SlabArgs<R> a) {
+__global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_kernel(SlabArgs<R> a) {
   extern __shared__ __align__(128) unsigned char sm[];
   constexpr int GS = vstride<R>(G);
   using TL = Tile<R, G>;
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(NT, 1) sweep_slab_kernel(SlabArgs<R> a) {
       }
   };
 
-  // this thread's (row, right-hand side) of the update, and its inputs one step ahead
+  // this thread's (row, right-hand side) of the update
   const int row0 = (warp * RG + lane / (CS * GL)) * RA;     // first row of this lane's group
   const int gl4 = (lane / CS) % GL;
   int urow, ug;
@@ -293,20 +295,31 @@ __global__ void __launch_bounds__(NT, 1) sweep_slab_kernel(SlabArgs<R> a) {
   const bool ux = uown && urow < ns;
   uown = ux && ug < gcount;
   const long long upos = (long long)(g0 + ug) * a.N + lo_c + urow;
-  c128 in_r(0.0, 0.0);
-  Cx<R> in_w(0, 0), in_c(0, 0);
+  // Its inputs come a step ahead by cp.async (registers loaded a step ahead were waited for at
+  // once: 15 % of a step): r (forward) or w (backward) of every (row, right-hand side) by and for
+  // its own thread, in one place, and the coupling of a row by its first lane
+  const int slot = urow * G + ug;
+  c128* in_r = reinterpret_cast<c128*>(sm + a.o_in) + slot;
+  Cx<R>* in_w = reinterpret_cast<Cx<R>*>(in_r);
+  Cx<R>* in_c = reinterpret_cast<Cx<R>*>(sm + a.o_inc) + urow;
+  if (ux) *in_r = c128(0.0, 0.0);
+  auto copy_in = [](Cx<R>* dst, const Cx<R>* src) {
+    if constexpr (sizeof(R) == 4) cp_async8(dst, src);
+    else cp_async16(dst, src);
+  };
   auto load_inputs = [&](int s) {
     const bool fwd = s < n;
     const int m = layer_of(s);
     const int mn = (fwd && m < n - 1) ? m + 1 : m;
-    if (ux) in_c = a.cpl[(long long)mn * n + lo_c + urow];
+    if (ux && ug == 0) copy_in(in_c, a.cpl + (long long)mn * n + lo_c + urow);
     if (uown) {
       if (fwd) {
-        if (m < n - 1) in_r = a.r[upos + (long long)(m + 1) * n];
+        if (m < n - 1) cp_async16(in_r, a.r + upos + (long long)(m + 1) * n);
       } else {
-        in_w = a.w[upos + (long long)m * n];
+        copy_in(in_w, a.w + upos + (long long)m * n);
       }
     }
+    cp_async_commit();
   };
 
   // the copies are issued by the last warp, which has the fewest column chunks
@@ -565,25 +578,23 @@ __global__ void __launch_bounds__(NT, 1) sweep_slab_kernel(SlabArgs<R> a) {
       int idx;
       bool first;
       scatter_sum<R, RA * B, CS, 1>(o, lane, idx, first);
+      cp_async_wait0();
+      __syncwarp();
       if (ux) {
-        // the inputs are first touched here: their loads stay in flight over the whole step
-        pin(in_r);
-        pin(in_c);
-        pin(in_w);
         const Cx<R> y = o[0] + yl[urow * GS + ug];
-        const Cx<R> cpl = in_c;
+        const Cx<R> cpl = *in_c;
         const long long pos = upos + (long long)m * n;
         Cx<R> xn;
         if (fwd) {
           if (m < n - 1) {
             if (uown) a.w[pos] = y;
-            xn = cvt<R>(in_r) - cpl * y;
+            xn = cvt<R>(*in_r) - cpl * y;
           } else {
             if (uown) a.z[pos] = cvt<double>(y);
             xn = cpl * y;
           }
         } else {
-          const Cx<R> uu = uown ? in_w - y : Cx<R>(0, 0);
+          const Cx<R> uu = uown ? *in_w - y : Cx<R>(0, 0);
           if (uown) a.z[pos] = cvt<double>(uu);
           xn = cpl * uu;
         }
@@ -595,6 +606,7 @@ __global__ void __launch_bounds__(NT, 1) sweep_slab_kernel(SlabArgs<R> a) {
     __syncthreads();
   }
   // a CTA that stopped early still owns the copies it issued: wait for them
+  cp_async_wait0();
   if (producer && t < nsteps) {
     for (int s = t; s < issuedF; ++s) {
       long long spins = 0;
@@ -699,6 +711,8 @@ static size_t slab_plan(const hsweep_s* h, int G, int dbufs, bool l2x, SlabArgs<
   a.o_q = (unsigned)o; o += al((long long)std::max(1, h->slab_W) * GS * es, 16);
   for (int b = 0; b < 2; ++b) { a.o_p[b] = (unsigned)o; o += l2x ? 0 : al((long long)h->slab_X * G * es, 16); }
   a.o_y = (unsigned)o; o += al((long long)nsm * GS * es, 16);
+  a.o_in = (unsigned)o; o += (size_t)nsm * G * sizeof(c128);
+  a.o_inc = (unsigned)o; o += al((long long)nsm * es, 16);
   a.o_bar = (unsigned)o; o += 64;
   a.o_meta = (unsigned)o; o += al((long long)h->n * sizeof(uchar4), 16);
   a.dC = h->slab_dC;
@@ -711,18 +725,21 @@ static size_t slab_plan(const hsweep_s* h, int G, int dbufs, bool l2x, SlabArgs<
 
 template <typename R> using SlabKernel = void (*)(SlabArgs<R>);
 
-// threads per CTA: a step of one or two right-hand sides is a few hundred instructions a
-// warp, most of them overhead that every further warp repeats
-static int slab_threads(int G, bool fp64) { return fp64 || G <= 2 ? 256 : 512; }
+// Threads per CTA: a step of one or two right-hand sides is a few hundred instructions a
+// warp, most of them overhead that every further warp repeats; with four on a slab of at most
+// 32 rows, two CTAs of 256 threads share an SM and cover each other's waits (n = 511, 64
+// right-hand sides: 4.5 us a step against 4.7 with eight in one CTA).
+constexpr int slab_threads(int G, int rows, bool fp64) { return fp64 || G <= 2 || (G == 4 && rows <= 32) ? 256 : 512; }
 
 template <typename R, int G, bool L2X>
 static SlabKernel<R> slab_kernel_g(int rows) {
   if constexpr (sizeof(R) == 4) {
     // step 4: a warp per group of RA rows, every lane a column slice; all warps busy
-    constexpr int CS = 32 / (G / Tile<float, G>::B), NT = G <= 2 ? 256 : 512, W = 512 / NT;
-    if (rows <= 16) return sweep_slab_kernel<float, G, 1 * W, CS, NT, L2X>;
-    if (rows <= 32) return sweep_slab_kernel<float, G, 2 * W, CS, NT, L2X>;
-    return sweep_slab_kernel<float, G, 4 * W, CS, NT, L2X>;
+    constexpr int CS = 32 / (G / Tile<float, G>::B);
+    constexpr int NT = slab_threads(G, 32, false), NT64 = slab_threads(G, 64, false);
+    if (rows <= 16) return sweep_slab_kernel<float, G, 512 / NT, CS, NT, L2X>;
+    if (rows <= 32) return sweep_slab_kernel<float, G, 2 * 512 / NT, CS, NT, L2X>;
+    return sweep_slab_kernel<float, G, 4 * 512 / NT64, CS, NT64, L2X>;
   } else {
     // four warps, one a sub-core, whatever the slab: the FP64 unit is the bound, and fewer
     // lanes a row mean fewer additions to join them
@@ -753,7 +770,7 @@ static bool launch_config(const hsweep_s* h, SlabKernel<R> kern, const SlabConfi
     return false;
   }
   lc = cudaLaunchConfig_t{};
-  lc.blockDim = dim3(slab_threads(c.G, sizeof(R) == 8));
+  lc.blockDim = dim3(slab_threads(c.G, h->tree.maxsz(h->slab_dC), sizeof(R) == 8));
   lc.gridDim = dim3(C * groups);
   lc.dynamicSmemBytes = c.smem;
   lc.stream = h->stream;
@@ -777,51 +794,59 @@ static SlabConfig choose_slab_uncached(const hsweep_s* h, int nrhs) {
   if (!h->slab_valid) return best;
   const int C = 1 << h->slab_dC, rows = h->tree.maxsz(h->slab_dC);
   double best_cost = 1e300;
-  for (int l2x = 0; l2x < (sizeof(R) == 4 && C > 1 ? 2 : 1); ++l2x)
-    for (int G : {8, 4, 2, 1}) {
-      // complex128 is bound by the FP64 units, which the team sweep's smaller teams load
-      // better once a cluster would carry more than two right-hand sides (n = 255, 16 of
-      // them: 12.7 against 10.8 us a step)
-      if ((G > 2 && sizeof(R) == 8) || (l2x && G < 4)) continue;
-      for (int dbufs : {2, 1}) {
-        SlabArgs<R> a;
-        SlabConfig c;
-        c.l2x = l2x != 0;
-        c.G = G;
-        c.dbufs = dbufs;
-        c.smem = slab_plan<R>(h, G, dbufs, c.l2x, a);
-        if (c.smem > 227 * 1024) continue;
-        cudaLaunchConfig_t lc;
-        cudaLaunchAttribute at[1];
-        SlabKernel<R> kern = slab_kernel<R>(G, rows, c.l2x);
-        if (!launch_config<R>(h, kern, c, 1, lc, at)) continue;
-        int act = 0;     // teams that run at a time
-        if (c.l2x) {
-          int per_sm = 0;
-          if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)lc.blockDim.x, c.smem) != cudaSuccess) {
-            cudaGetLastError();
-            continue;
-          }
-          act = per_sm * h->num_sms / C;
-        } else if (cudaOccupancyMaxActiveClusters(&act, kern, &lc) != cudaSuccess) {
-          cudaGetLastError();
-          continue;
-        }
-        if (act < 1) continue;
-        c.groups = (nrhs + G - 1) / G;
-        c.per_launch = c.l2x ? std::min(c.groups, act) : c.groups;
-        const int rounds = (c.groups + act - 1) / act;
-        if (sizeof(R) == 8 && rounds > 1) continue;
-        const double es = sizeof(R) == 4 ? 1.0 : 15.0;
-        const double step = 1.2 + (c.l2x ? 1.0 : 0.0) + es * 1.5e-5 * G * rows * (2.0 * h->slab_W + rows);
-        if (rounds * step < best_cost - 1e-9) {
-          best_cost = rounds * step;
-          best = c;
-          best.ok = true;
-        }
-        break;      // two D stages where they fit
+  struct Try { bool l2x; int G; };
+  const Try tries[] = {{false, 8}, {false, 4}, {false, 2}, {false, 1}, {true, 8}, {true, 4}};
+  for (const Try& y : tries) {
+    // complex128 is bound by the FP64 units, which the team sweep's smaller teams load
+    // better once a cluster would carry more than two right-hand sides (n = 255, 16 of
+    // them: 12.7 against 10.8 us a step)
+    if (sizeof(R) == 8 && (y.G > 2 || y.l2x)) continue;
+    if (y.l2x && C == 1) continue;
+    for (int dbufs : {2, 1}) {
+      SlabArgs<R> a;
+      SlabConfig c;
+      c.l2x = y.l2x;
+      c.G = y.G;
+      c.dbufs = dbufs;
+      c.smem = slab_plan<R>(h, c.G, dbufs, c.l2x, a);
+      if (c.smem > 227 * 1024) continue;
+      cudaLaunchConfig_t lc;
+      cudaLaunchAttribute at[1];
+      SlabKernel<R> kern = slab_kernel<R>(c.G, rows, c.l2x);
+      if (!launch_config<R>(h, kern, c, 1, lc, at)) continue;
+      int act = 0, per_sm = 0;     // teams that run at a time
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)lc.blockDim.x, c.smem) != cudaSuccess) {
+        cudaGetLastError();
+        continue;
       }
+      if (c.l2x) {
+        act = per_sm * h->num_sms / C;
+      } else if (cudaOccupancyMaxActiveClusters(&act, kern, &lc) != cudaSuccess) {
+        cudaGetLastError();
+        continue;
+      }
+      if (act < 1) continue;
+      c.groups = (nrhs + c.G - 1) / c.G;
+      c.per_launch = c.l2x ? std::min(c.groups, act) : c.groups;
+      const int rounds = (c.groups + act - 1) / act;
+      if (sizeof(R) == 8 && rounds > 1) continue;
+      // Microseconds a step (complex64, fitted to n = 127, 300, 511, 700 and 1023 with 1 to 64
+      // right-hand sides): a latency, 0.35 more for an exchange through L2, and work per
+      // right-hand side that two CTAs on an SM share it for (clusters double up as soon as
+      // there are more than fit with an SM each)
+      const double rc = rows * (2.0 * h->slab_W + rows);
+      const int alone = c.l2x ? h->num_sms / C : std::max(1, act / per_sm);
+      const int shared = (std::min(c.groups, act) + alone - 1) / alone;
+      const double work = (0.12 + 1.8e-5 * rc) * c.G * (sizeof(R) == 4 ? 1.0 : 15.0);
+      const double cost = rounds * (1.75 + 2.5e-5 * rc + (c.l2x ? 0.35 : 0.0) + shared * work);
+      if (cost < best_cost - 1e-9) {
+        best_cost = cost;
+        best = c;
+        best.ok = true;
+      }
+      break;      // two D stages where they fit
     }
+  }
   return best;
 }
 
@@ -990,7 +1015,7 @@ int hsw_slab_plan(hsweep_s* h, int nrhs, long long* out) {
   if (!s.ok) return 0;
   const int rows = h->tree.maxsz(h->slab_dC);
   const int st = h->prec == HSWEEP_FP64 ? slab_stride<double>(h->slab_W) : slab_stride<float>(h->slab_W);
-  out[0] = 2; out[1] = 1 << h->slab_dC; out[2] = s.G; out[3] = s.per_launch; out[4] = slab_threads(s.G, h->prec == HSWEEP_FP64);
+  out[0] = 2; out[1] = 1 << h->slab_dC; out[2] = s.G; out[3] = s.per_launch; out[4] = slab_threads(s.G, h->tree.maxsz(h->slab_dC), h->prec == HSWEEP_FP64);
   out[5] = (long long)s.smem; out[6] = (long long)rows * (st + h->slab_rsD) * (long long)h->fac_elem(); out[7] = s.l2x ? 1 : 0;
   return 1;
 }
