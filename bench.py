@@ -656,7 +656,8 @@ def main():
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["traffic"] = recorded_traffic(args.workload, nrhs)
     plan = h.sweep_plan(nrhs)
-    roof["kernel"] = {2: "sweep_team_kernel"}.get(plan["tma"], "sweep_kernel") + "<c64>"
+    slabs = plan["tma"] == 2 and plan["leaves_per_chunk"] <= 1    # dense-diagonal slabs (hsweep_sweep_plan)
+    roof["kernel"] = {2: "sweep_slab_kernel" if slabs else "sweep_team_kernel"}.get(plan["tma"], "sweep_kernel") + "<c64>"
     roof["plan"] = plan
     roof["launch_ms"] = avg_s * 1e3
     roof["hbm_gbs_achieved"] = bytes_ / avg_s / 1e9

@@ -76,7 +76,8 @@ typedef struct {
   int team;          /* CTAs per sweep team (power of two, 0 = automatic) */
   int groups;        /* right-hand sides per sweep team (1, 2, 4, 5 or 8; 0 = automatic) */
   int sweep_kernel;  /* 0: automatic (default): with strong_rank > 0 the sweep on the strongly
-                           admissible format (hsweep_strong_export) where its plan fits, then
+                           admissible format (its records, hsweep_strong_export, or the same
+                           layers as dense-diagonal slabs) where its plan fits, then
                            the bulk-copy-staged sweep on teams of CTAs (dense-diagonal
                            slabs, else the sibling-pair factors) where its shared-memory
                            plan fits, else the basic sweep;
@@ -358,9 +359,11 @@ HSWEEP_API int hsweep_stats(hsweep_t h, int reset, long long* launches, long lon
  * out[3] teams of a launch, out[4] for the basic kernel 1 when its team is the whole grid (a grid barrier),
  * for the team kernels the threads per CTA (512: one CTA per SM, 256: two), out[5] dynamic shared
  * memory per CTA in bytes, out[6] largest per-step factor record of one CTA in bytes,
- * out[7] column slices per row in the expansion (0 for the basic kernel); for kernel 2 on
- * dense-diagonal slabs, the automatic choice up to n = 1024 (complex64) or 512 (complex128,
- * few right-hand sides), 0 when its teams are clusters and 1 when they exchange through L2.
+ * out[7] column slices per row in the expansion (0 for the basic kernel); for kernels 2 and 3
+ * on dense-diagonal slabs, 0 when their teams are clusters and 1 when they exchange through
+ * L2.  Those are the automatic choice of kernel 2 up to n = 1024 (complex64) or 512
+ * (complex128, few right-hand sides), and of kernel 3 up to n = 1024 in complex64 for as few
+ * right-hand sides as they are the faster for (all up to n = 255, about 10 at n = 511).
  */
 HSWEEP_API int hsweep_sweep_plan(hsweep_t h, int nrhs, long long* out8);
 

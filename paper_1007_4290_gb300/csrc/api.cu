@@ -505,7 +505,10 @@ extern "C" int hsweep_setup_tuning(hsweep_t h, double* out6) {
 
 extern "C" int hsweep_sweep_plan(hsweep_t h, int nrhs, long long* out8) {
   if (!h || !out8 || nrhs < 1) return HSWEEP_ERR_ARG;
-  if (h->opt.sweep_kernel == 0 && h->strong_R > 0 && hsw_strong_plan_sweep(h, nrhs, out8)) return HSWEEP_OK;
+  if (h->opt.sweep_kernel == 0 && h->strong_R > 0) {
+    if (hsw_strong_prefers_slabs(h, nrhs) && hsw_slab_plan(h, nrhs, out8)) return HSWEEP_OK;
+    if (hsw_strong_plan_sweep(h, nrhs, out8)) return HSWEEP_OK;
+  }
   if (h->opt.sweep_kernel != 1 && hsw_slab_plan(h, nrhs, out8)) return HSWEEP_OK;
   if (h->opt.sweep_kernel != 1 && hsw_team_plan(h, nrhs, out8)) return HSWEEP_OK;
   for (int i = 0; i < 8; ++i) out8[i] = 0;

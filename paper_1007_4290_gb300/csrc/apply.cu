@@ -448,6 +448,10 @@ int hsw_apply(hsweep_s* h, const c128* r, c128* z, int nrhs) {
   if (nrhs <= 0) return HSWEEP_OK;
   if (h->opt.sweep_kernel == 0 && h->strong_R > 0) {
     bool used = false;
+    if (hsw_strong_prefers_slabs(h, nrhs)) {
+      int rc = hsw_apply_slab(h, r, z, nrhs, &used);
+      if (rc != HSWEEP_OK || used) return rc;
+    }
     int rc = hsw_apply_strong(h, r, z, nrhs, &used);
     if (rc != HSWEEP_OK || used) return rc;
   }
@@ -530,6 +534,10 @@ int hsw_apply_scratch(hsweep_s* h, const c128* r, c128* z, int nrhs, void* scrat
   if (hsw_apply_scratch_bytes(h, nrhs) > bytes) return HSWEEP_ERR_ARG;
   if (h->opt.sweep_kernel == 0 && h->strong_R > 0) {      // the same kernel hsw_apply would use
     bool used = false;
+    if (hsw_strong_prefers_slabs(h, nrhs)) {
+      int rc = hsw_apply_slab(h, r, z, nrhs, &used, scratch, bytes);
+      if (rc != HSWEEP_OK || used) return rc;
+    }
     int rc = hsw_apply_strong(h, r, z, nrhs, &used, scratch, bytes);
     if (rc != HSWEEP_OK || used) return rc;
   }

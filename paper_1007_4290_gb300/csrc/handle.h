@@ -100,8 +100,10 @@ struct hsweep_s {
   int slab_dC = 0, slab_rsD = 0, slab_W = 0, slab_X = 0;   // most columns / received sums of a layer
   long long slab_cap = 0;
   bool slab_valid = false;
-  // its launch plans already chosen: {nrhs, ok, L2 teams, G, D stages, groups, groups per launch, smem}
-  std::vector<std::array<long long, 8>> slab_plans;
+  bool slab_strong = false;   // the slabs hold the strongly admissible T~_m (hsw_strong_slabs)
+  // its launch plans already chosen: {nrhs, ok, L2 teams, G, D stages, groups, groups per launch, smem,
+  // estimated ns a right-hand-side batch step}
+  std::vector<std::array<long long, 9>> slab_plans;
 
   int* d_status = nullptr;     // [2]
   unsigned* d_bar = nullptr;   // grid barrier words [2]
@@ -194,6 +196,10 @@ int hsw_pack_slabs(hsweep_s* h, int m0, int m1, const std::vector<int>& rk);
 int hsw_apply_slab(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* used, void* scratch = nullptr,
                    size_t scratch_bytes = 0);
 int hsw_slab_plan(hsweep_s* h, int nrhs, long long* out8);   // 1 if the slab sweep would run
+// the slabs of layer m from the expanded strongly admissible factors (setup layout); 1 if the
+// sweep on them is the faster of the two on that format
+int hsw_strong_slabs(hsweep_s* h, int m, const void* G_F, const void* G_leaf, const long long* d_gfo, const int* G_rank);
+int hsw_strong_prefers_slabs(hsweep_s* h, int nrhs);
 // direction.cu: reversal of the layer order (x2 -> 1 - x2)
 int hsw_flip_reserve(hsweep_s* h, size_t bytes);
 int hsw_flip_c128(hsweep_s* h, const c128* in, c128* out, int nvec);
@@ -213,6 +219,9 @@ int hsw_apply_strong(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* used, 
                      size_t scratch_bytes = 0);
 size_t hsw_apply_strong_scratch_bytes(hsweep_s* h, int nrhs);
 int hsw_strong_plan_sweep(hsweep_s* h, int nrhs, long long* out8);   // 1 if the strong sweep would run
+long long hsw_strong_cost(hsweep_s* h, int nrhs);         // its estimate, ns a step of the batch; 0 if it would not run
+long long hsw_strong_exchange_bound(const hsweep_s* h, int nrhs);   // bytes: any plan for at most nrhs
+long long hsw_slab_exchange_bound(const hsweep_s* h);               // bytes: any plan
 __host__ __device__ void hsw_philox4x32_10(const uint32_t ctr[4], const uint32_t key[2], uint32_t out[4]);
 // setup.cu
 int hsw_factor(hsweep_s* h);

@@ -1785,6 +1785,8 @@ static int factor_impl(hsweep_s* h) {
       // the records of the strong sweep, from the exact strongly admissible factors
       rc = hsw_spack_layer(h, m, G_F, G_leaf, w->d_gfo);
       if (rc) return rc;
+      rc = hsw_strong_slabs(h, m, G_F, G_leaf, w->d_gfo, w->G_rank);
+      if (rc) return rc;
       rc = recompress(w->all_nodes_off, w->all_nodes, w->all_pairs_off, w->all_pairs, 1, direct ? store : nullptr,
                       store_rank);
       if (rc) return rc;

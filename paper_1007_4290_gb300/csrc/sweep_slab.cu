@@ -626,37 +626,41 @@ __global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_ke
 }
 
 // ---- packing: the slab records of layers m0 .. from the factor store ---------------------------
-// One CTA per (slab, layer).  D^t[j][i] = T(i, j): the leaf block, or the product of the
+// One CTA per (slab, layer), or eight when one layer is packed at a time.  D^t[j][i] = T(i, j): the leaf block, or the product of the
 // factors of the two children that part rows i and j (rank(v) terms).
 template <typename R>
 __global__ void __launch_bounds__(256) pack_slabs(int m0, int L, int leaf, int nnodes, int dC, int rsD,
                                                   const int* __restrict__ lo, const int* __restrict__ sz,
-                                                  const long long* __restrict__ off, const Cx<R>* __restrict__ fac,
-                                                  long long layer_stride, const int* __restrict__ rank,
+                                                  const long long* __restrict__ off, const Cx<R>* __restrict__ leaves,
+                                                  const Cx<R>* __restrict__ fac, long long layer_stride,
+                                                  const int* __restrict__ rank,
                                                   Cx<R>* __restrict__ pack, long long cap, int n, uchar4* __restrict__ meta) {
   const int c = blockIdx.x, C = 1 << dC, m = m0 + blockIdx.y;
   const int vc = C + c, lo_c = lo[vc], ns = sz[vc];
-  const int* rk = rank + (long long)m * nnodes;
+  const int t0 = blockIdx.z * blockDim.x + threadIdx.x, nt = gridDim.z * blockDim.x;
+  // layer_stride = 0: a single layer (the setup's buffers), ranks and factors at their start
+  const int* rk = layer_stride ? rank + (long long)m * nnodes : rank;
   const Cx<R>* F = fac + (long long)m * layer_stride;
+  const Cx<R>* D = leaves + (long long)m * layer_stride;
   Cx<R>* out = pack + ((long long)m * C + c) * cap;
   int e[4] = {0, 0, 0, 0}, W = 0;
   for (int d = 1; d <= dC; ++d) {
     W += max(1, rk[vc >> (dC - d)]);
     e[d - 1] = W;
   }
-  if (threadIdx.x == 0) meta[(long long)c * n + m] = make_uchar4(e[0], e[1], e[2], e[3]);
+  if (t0 == 0) meta[(long long)c * n + m] = make_uchar4(e[0], e[1], e[2], e[3]);
   auto leaf_of = [&](int i) {
     int v = vc;
     for (int d = dC; d < L; ++d) v = 2 * v + ((lo_c + i) >= lo[2 * v + 1] ? 1 : 0);
     return v;
   };
-  for (int it = threadIdx.x; it < ns * rsD; it += blockDim.x) {
+  for (int it = t0; it < ns * rsD; it += nt) {
     const int j = it / rsD, i = it - j * rsD;
     Cx<R> val(0, 0);
     if (i < ns) {
       int vi = leaf_of(i), vj = leaf_of(j);
       if (vi == vj) {
-        val = F[(long long)(vi - (1 << L)) * leaf * leaf + (long long)(lo_c + j - lo[vj]) * leaf + (lo_c + i - lo[vi])];
+        val = D[(long long)(vi - (1 << L)) * leaf * leaf + (long long)(lo_c + j - lo[vj]) * leaf + (lo_c + i - lo[vi])];
       } else {
         while ((vi >> 1) != (vj >> 1)) { vi >>= 1; vj >>= 1; }
         const Cx<R>* Fi = F + off[vi] + (lo_c + i - lo[vi]);
@@ -669,7 +673,7 @@ __global__ void __launch_bounds__(256) pack_slabs(int m0, int L, int leaf, int n
   }
   const int rs = slab_stride<R>(W);
   Cx<R>* fo = out + (long long)ns * rsD;
-  for (int it = threadIdx.x; it < ns * rs; it += blockDim.x) {
+  for (int it = t0; it < ns * rs; it += nt) {
     const int i = it / rs, k = it - i * rs;
     Cx<R> val(0, 0);
     if (k < W) {
@@ -693,6 +697,7 @@ struct SlabConfig {
   bool ok = false, l2x = false;
   int G = 0, dbufs = 0, groups = 0, per_launch = 0;   // groups of G right-hand sides; of them one launch runs
   size_t smem = 0;
+  long long cost = 0;                                 // estimated ns a step of the batch
 };
 
 // shared-memory plan for G right-hand sides; returns total bytes
@@ -843,6 +848,7 @@ static SlabConfig choose_slab_uncached(const hsweep_s* h, int nrhs) {
         best_cost = cost;
         best = c;
         best.ok = true;
+        best.cost = (long long)(1e3 * cost);
       }
       break;      // two D stages where they fit
     }
@@ -856,12 +862,13 @@ static SlabConfig choose_slab(hsweep_s* h, int nrhs) {
     if (e[0] == nrhs) {
       SlabConfig s;
       s.ok = e[1] != 0; s.l2x = e[2] != 0; s.G = (int)e[3]; s.dbufs = (int)e[4]; s.groups = (int)e[5];
-      s.per_launch = (int)e[6]; s.smem = (size_t)e[7];
+      s.per_launch = (int)e[6]; s.smem = (size_t)e[7]; s.cost = e[8];
       return s;
     }
   const SlabConfig s = choose_slab_uncached<R>(h, nrhs);
   if (h->slab_plans.size() >= 64) h->slab_plans.erase(h->slab_plans.begin());
-  h->slab_plans.push_back({nrhs, s.ok ? 1 : 0, s.l2x ? 1 : 0, s.G, s.dbufs, s.groups, s.per_launch, (long long)s.smem});
+  h->slab_plans.push_back({nrhs, s.ok ? 1 : 0, s.l2x ? 1 : 0, s.G, s.dbufs, s.groups, s.per_launch, (long long)s.smem,
+                           s.cost});
   return s;
 }
 
@@ -876,7 +883,8 @@ static int apply_slab_impl(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* 
   void* wptr = scratch;
   void* xptr = static_cast<unsigned char*>(scratch) + wb;
   if (scratch) {
-    if (wb + xb > (long long)scratch_bytes) return HSWEEP_ERR_ARG;
+    // a caller's buffer too small for the exchange slots: the team sweep, which it was sized for
+    if (wb + xb > (long long)scratch_bytes) return HSWEEP_OK;
   } else {
     const long long need_w = (long long)nrhs * h->N;
     if (need_w > h->wcache_cap) {
@@ -887,13 +895,18 @@ static int apply_slab_impl(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* 
       }
       h->wcache_cap = need_w;
     }
-    if (xb / es > h->xch_cap) {
-      int rc = hsw_regrow(h, &h->d_xch, (size_t)xb);
+    // room for the largest exchange of any plan for as many right-hand sides or fewer,
+    // although this call may need none: a captured call with fewer of them can have a plan
+    // that exchanges through L2, and must not allocate
+    const long long xcap = std::max(hsw_slab_exchange_bound(h), hsw_strong_exchange_bound(h, nrhs));
+    const long long need_x = std::max(xb, xcap) / es;
+    if (need_x > h->xch_cap) {
+      int rc = hsw_regrow(h, &h->d_xch, (size_t)(need_x * es));
       if (rc) {
         if (!h->d_xch) h->xch_cap = 0;
         return rc;
       }
-      h->xch_cap = xb / es;
+      h->xch_cap = need_x;
     }
     wptr = h->d_wcache;
     xptr = h->d_xch;
@@ -981,13 +994,19 @@ int hsw_slab_create(hsweep_s* h) {
 
 int hsw_pack_slabs(hsweep_s* h, int m0, int m1, const std::vector<int>& rk) {
   if (!h->d_slab || m1 <= m0) return HSWEEP_OK;
+  if (h->slab_strong) {
+    if (h->spack_valid) return HSWEEP_OK;     // the setup wrote them (hsw_strong_slabs)
+    h->slab_strong = false;                   // a layer was replaced: all of them from the store
+    m0 = 0;
+    m1 = h->n;
+  }
   const dim3 grid(1 << h->slab_dC, m1 - m0);
   if (h->prec == HSWEEP_FP64)
     pack_slabs<double><<<grid, 256, 0, h->stream>>>(m0, h->L, h->leaf, h->nnodes, h->slab_dC, h->slab_rsD, h->d_lo, h->d_sz,
-        h->d_off, (const c128*)h->d_fac, h->layer_stride, h->d_rank, (c128*)h->d_slab, h->slab_cap, h->n, (uchar4*)h->d_slab_meta);
+        h->d_off, (const c128*)h->d_fac, (const c128*)h->d_fac, h->layer_stride, h->d_rank, (c128*)h->d_slab, h->slab_cap, h->n, (uchar4*)h->d_slab_meta);
   else
     pack_slabs<float><<<grid, 256, 0, h->stream>>>(m0, h->L, h->leaf, h->nnodes, h->slab_dC, h->slab_rsD, h->d_lo, h->d_sz,
-        h->d_off, (const c64*)h->d_fac, h->layer_stride, h->d_rank, (c64*)h->d_slab, h->slab_cap, h->n, (uchar4*)h->d_slab_meta);
+        h->d_off, (const c64*)h->d_fac, (const c64*)h->d_fac, h->layer_stride, h->d_rank, (c64*)h->d_slab, h->slab_cap, h->n, (uchar4*)h->d_slab_meta);
   h->nlaunch += 1;
   HSW_CUDA(cudaGetLastError());
   // the most columns of any layer and slab, for the shared-memory plan
@@ -1009,13 +1028,65 @@ int hsw_pack_slabs(hsweep_s* h, int m0, int m1, const std::vector<int>& rk) {
   return HSWEEP_OK;
 }
 
+// The strongly admissible T~_m as slabs, from the expanded factors of the setup (sibling-pair
+// factors of rank 3R(L - l) + one leaf at depth l, zero outside each column's own cluster).
+// The sweep on them does more arithmetic than the one on the records of sweep_strong.cu, which
+// skips those zeros, but has one exchange and fewer barriers a step where that one gathers
+// every cluster's interaction list.  Microseconds a step, complex64, R = 2 (records, slabs):
+// n = 255, 1 RHS 2.95, 1.96; n = 511, 1 RHS 3.21, 2.47; 8 RHS 3.50, 2.81; 16 RHS 3.50, 3.54;
+// 24 RHS 3.87, 3.55; 64 RHS 4.69, 5.62; n = 1023, 1 RHS 3.67, 2.99; 64 RHS 7.07, 9.07.
+// complex128 keeps the records: the FP64 units pay for the zeros (n = 127, 1 RHS 5.02, 5.68;
+// n = 511 7.86, 13.66).
+int hsw_strong_slabs(hsweep_s* h, int m, const void* G_F, const void* G_leaf, const long long* d_gfo, const int* G_rank) {
+  if (!h->d_slab || h->opt.sweep_kernel != 0 || h->L < 2 || h->prec == HSWEEP_FP64) return HSWEEP_OK;
+  pack_slabs<float><<<dim3(1 << h->slab_dC, 1, 8), 256, 0, h->stream>>>(m, h->L, h->leaf, h->nnodes, h->slab_dC,
+      h->slab_rsD, h->d_lo, h->d_sz, d_gfo, (const c64*)G_leaf, (const c64*)G_F, 0, G_rank, (c64*)h->d_slab,
+      h->slab_cap, h->n, (uchar4*)h->d_slab_meta);
+  h->nlaunch += 1;
+  HSW_CUDA(cudaGetLastError());
+  if (m < h->n - 1) return HSWEEP_OK;
+  const int dC = h->slab_dC, C = 1 << dC;
+  h->slab_W = h->slab_X = 0;
+  for (int c = 0; c < C; ++c) {
+    int W = 0, X = 0;
+    for (int d = 1; d <= dC; ++d) {
+      int b = ((C + c) >> (dC - d)) | 1;                    // the pair's right child, and its first leaf
+      while (b < h->nleaves) b *= 2;
+      const int r = 3 * h->strong_R * (h->L - d) + h->tree.sz[b];
+      W += r;
+      X += r << (dC - d);
+    }
+    h->slab_W = std::max(h->slab_W, W);
+    h->slab_X = std::max(h->slab_X, X);
+  }
+  h->slab_plans.clear();
+  h->slab_strong = h->slab_valid = true;
+  return HSWEEP_OK;
+}
+
+// The faster of the two sweeps on the strongly admissible format, by the estimates that chose
+// their plans (over n = 63 to 1023 and 1 to 64 RHS it misses the faster one only where the two
+// are within 8 %)
+int hsw_strong_prefers_slabs(hsweep_s* h, int nrhs) {
+  if (!h->slab_strong || !h->spack_valid || !slab_usable(h)) return 0;
+  const SlabConfig s = choose_slab<float>(h, nrhs);
+  const long long other = s.ok ? hsw_strong_cost(h, nrhs) : 0;
+  return s.ok && (other == 0 || s.cost < other);
+}
+
+// two CTAs on every SM, eight right-hand sides a team
+long long hsw_slab_exchange_bound(const hsweep_s* h) {
+  if (!h->slab_valid || h->prec == HSWEEP_FP64 || h->slab_dC == 0) return 0;
+  return 2LL * 2 * h->num_sms * h->slab_W * 8 * (long long)h->fac_elem();
+}
+
 int hsw_slab_plan(hsweep_s* h, int nrhs, long long* out) {
   if (!slab_usable(h)) return 0;
   const SlabConfig s = h->prec == HSWEEP_FP64 ? choose_slab<double>(h, nrhs) : choose_slab<float>(h, nrhs);
   if (!s.ok) return 0;
   const int rows = h->tree.maxsz(h->slab_dC);
   const int st = h->prec == HSWEEP_FP64 ? slab_stride<double>(h->slab_W) : slab_stride<float>(h->slab_W);
-  out[0] = 2; out[1] = 1 << h->slab_dC; out[2] = s.G; out[3] = s.per_launch; out[4] = slab_threads(s.G, h->tree.maxsz(h->slab_dC), h->prec == HSWEEP_FP64);
+  out[0] = h->slab_strong ? 3 : 2; out[1] = 1 << h->slab_dC; out[2] = s.G; out[3] = s.per_launch; out[4] = slab_threads(s.G, h->tree.maxsz(h->slab_dC), h->prec == HSWEEP_FP64);
   out[5] = (long long)s.smem; out[6] = (long long)rows * (st + h->slab_rsD) * (long long)h->fac_elem(); out[7] = s.l2x ? 1 : 0;
   return 1;
 }

@@ -599,7 +599,7 @@ struct StrongPack {
   int* d_src = nullptr;
   int* d_near = nullptr;
   void* d_pack = nullptr;
-  std::vector<std::array<long long, 9>> plans;   // {nrhs, ok, dC, C, G, teams, smem, ntask, threads}
+  std::vector<std::array<long long, 10>> plans;  // {nrhs, ok, dC, C, G, teams, smem, ntask, threads, cost}
 };
 
 namespace {
@@ -720,6 +720,7 @@ struct StrongConfig {
   int dC, C, G, nteams, ntask;
   size_t smem;
   int nt;              // threads per CTA (kST or kST2)
+  long long cost;      // estimated ns a step of the batch
 };
 
 // shared-memory plan and exchange layout for (dC, G); 0 if not supported
@@ -812,7 +813,8 @@ StrongConfig choose_strong(hsweep_s* h, int nrhs) {
   StrongPack* p = h->spk;
   for (const auto& e : p->plans)
     if (e[0] == nrhs)
-      return StrongConfig{e[1] != 0, (int)e[2], (int)e[3], (int)e[4], (int)e[5], (int)e[7], (size_t)e[6], (int)e[8]};
+      return StrongConfig{e[1] != 0, (int)e[2], (int)e[3], (int)e[4], (int)e[5], (int)e[7], (size_t)e[6], (int)e[8],
+                          e[9]};
   StrongConfig best{};
   best.ok = false;
   double best_cost = 1e300;
@@ -842,14 +844,14 @@ StrongConfig choose_strong(hsweep_s* h, int nrhs) {
         const double cost = rounds * step;
         if (cost < best_cost - 1e-9) {
           best_cost = cost;
-          best = StrongConfig{true, dC, C, G, teams, a.ntask, smem, nt};
+          best = StrongConfig{true, dC, C, G, teams, a.ntask, smem, nt, (long long)(1e3 * cost)};
         }
       }
     }
   }
   if (p->plans.size() >= 64) p->plans.erase(p->plans.begin());
   p->plans.push_back({nrhs, best.ok ? 1 : 0, best.dC, best.C, best.G, best.nteams, (long long)best.smem, best.ntask,
-                      best.nt});
+                      best.nt, best.cost});
   return best;
 }
 
@@ -918,7 +920,9 @@ int apply_strong_impl(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* used,
       }
       h->wcache_cap = need_w;
     }
-    const long long need_x = (xb + (long long)es - 1) / (long long)es;
+    // as in sweep_slab.cu: any plan for as many right-hand sides or fewer, of either sweep
+    const long long xcap = std::max(hsw_slab_exchange_bound(h), hsw_strong_exchange_bound(h, nrhs));
+    const long long need_x = (std::max(xb, xcap) + (long long)es - 1) / (long long)es;
     if (need_x > h->xch_cap) {
       int rc = hsw_regrow(h, &h->d_xch, (size_t)need_x * es);
       if (rc) {
@@ -998,6 +1002,30 @@ size_t hsw_apply_strong_scratch_bytes(hsweep_s* h, int nrhs) {
     strong_scratch_need<float>(h, nrhs, cfg, &wb, &xb);
   }
   return (size_t)(al256s(wb) + al256s(xb));
+}
+
+long long hsw_strong_cost(hsweep_s* h, int nrhs) {
+  if (!h->spack_valid || !h->spk) return 0;
+  const StrongConfig cfg = h->prec == HSWEEP_FP64 ? choose_strong<double>(h, nrhs) : choose_strong<float>(h, nrhs);
+  return cfg.ok ? cfg.cost : 0;
+}
+
+template <typename R>
+static long long strong_exchange_bound(const hsweep_s* h, int nrhs) {
+  long long most = 0;
+  for (int C = 1, dC = 0; C <= h->nleaves && C <= 2 * h->num_sms; C *= 2, ++dC)
+    for (int G : {8, 4, 2, 1}) {
+      StrongArgs<R> a;
+      if (plan_strong<R>(h, dC, G, a) == 0) continue;
+      const long long teams = std::min<long long>((nrhs + G - 1) / G, 2 * h->num_sms / C);   // at most two CTAs per SM
+      most = std::max(most, 2 * teams * C * a.xwords * G * (long long)sizeof(typename Tagged<R>::W));
+    }
+  return most;
+}
+
+long long hsw_strong_exchange_bound(const hsweep_s* h, int nrhs) {
+  if (!h->spack_valid || !h->spk) return 0;
+  return h->prec == HSWEEP_FP64 ? strong_exchange_bound<double>(h, nrhs) : strong_exchange_bound<float>(h, nrhs);
 }
 
 int hsw_strong_plan_sweep(hsweep_s* h, int nrhs, long long* out) {

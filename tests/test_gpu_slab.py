@@ -88,3 +88,38 @@ def test_withheld_sums_time_out_and_every_cta_returns(hs, n, prec, nrhs, monkeyp
     assert h.status()[0] == 0
     assert torch.equal(z, ref)
     h.free()
+
+
+# n, R, right-hand sides: ragged slabs of 2, 4, 8 and 16 CTAs, the rank from 1 to the largest
+# that n = 127 takes, remainders of the right-hand-side groups
+@pytest.mark.parametrize("n,R,nrhs", [(40, 2, 1), (63, 5, 3), (127, 1, 9), (127, 5, 2), (200, 2, 35), (260, 3, 5)])
+def test_strong_format_slabs_match_the_exact_sweep_of_their_layers(hs, n, R, nrhs):
+    # the slabs that the setup packs from the strongly admissible factors (plan kernel 3, plan
+    # entry 7 at most 1), the records of the same layers, and the slabs packed anew from the
+    # store once a layer is imported
+    from tests.helpers import strong_to_dense
+    import synth
+    c, omega, pml = synth.velocity_lens(n), 2 * np.pi * (n + 1) / 8, 6
+    h = hs.hsweep_setup(torch.tensor(c, device="cuda"), omega, pml, 1e-6, hs.default_opts(strong_rank=R))
+    p = h.sweep_plan(nrhs)
+    assert p["tma"] == 3 and p["leaves_per_chunk"] <= 1, p
+    rng = np.random.default_rng(n + R)
+    V = rng.standard_normal((nrhs, n * n)) + 1j * rng.standard_normal((nrhs, n * n))
+    Vt = torch.tensor(V, device="cuda")
+    Z = h.apply(Vt).cpu().numpy()
+    assert h.status()[0] == 0
+    Ts = [strong_to_dense(n, 8, R, *h.strong_export(m)) for m in range(n)]
+    disc = Discretization(c, omega, pml)
+    for s in {0, nrhs - 1}:
+        ref = solve_exact(disc, Ts, V[s])
+        assert np.linalg.norm(Z[s] - ref) / np.linalg.norm(ref) < 2e-5, s
+    h.import_layer(0, *h.export_layer(0))
+    p = h.sweep_plan(nrhs)
+    assert p["tma"] == 2 and p["leaves_per_chunk"] <= 1, p
+    Zs = h.apply(Vt)
+    h.free()
+    h = hs.hsweep_setup(torch.tensor(c, device="cuda"), omega, pml, 1e-6, hs.default_opts(strong_rank=R, sweep_kernel=2))
+    Zw = h.apply(Vt)
+    assert h.status()[0] == 0
+    h.free()
+    assert ((Zs - Zw).norm() / Zw.norm()).item() < 4e-5      # two sweeps, 2e-5 each
