@@ -36,8 +36,8 @@ namespace {
 constexpr int kBlk = 256;
 
 // Dense path of the recompression in complex64: up to this many rows the pivoted Gram-Schmidt
-// of the block itself (svd_jacobi, about 0.3 us for each of the block's 20 to 40 significant
-// columns) is shorter than the QR of its factors (3.6 us for each of up to 98 columns).  A
+// of the block itself (svd_jacobi: one barrier for each of the block's 20 to 40 significant
+// columns) is shorter than the QR of its factors (one for each of up to 98 columns).  A
 // 128 x 128 core is 131 KB of shared memory.  In complex128 the QR is the cheaper.
 constexpr int kDenseRows = 128;
 
@@ -128,7 +128,7 @@ __device__ __forceinline__ int depth_of(int v) { return 31 - __clz(v); }
 // ---------------------------------------------------------------------------------
 // S~_m, one launch: blocks 0 .. nleaves - 1 (of slice 0) form a leaf A_mm[leaf] - D T_leaf D
 // and invert it, FP64 Gauss-Jordan with partial pivoting in both precisions (a serial chain
-// of FP64 instructions, 15 us, with the factors beside it); the others form the factors
+// of FP64 instructions, 17 us, with the factors beside it; 35 us in three launches before); the others form the factors
 // [-D F_a, a e_last] / [D F_b, e_first] of node v = 2 + blockIdx.x - nleaves, in gridDim.y slices.
 template <typename R>
 __global__ void __launch_bounds__(kBlk) schur_layer(Geo g, int m, const c128* __restrict__ diag,
@@ -263,7 +263,8 @@ __global__ void __launch_bounds__(kBlk) schur_layer(Geo g, int m, const c128* __
 // Qr_u = F_u^t X restricted to u) followed by an expansion.  Both are chains of dependent
 // loads; they are cut short by spreading them over more CTAs and warps: the reductions take
 // eight columns of X per CTA, the expansion 32 rows and four columns with the sum over the
-// factor columns split over the eight warps (23 -> 5 us and 11 -> 4 us a launch at n = 511).
+// factor columns split over the eight warps (26.3 -> 8.9 us and 13.5 -> 6.4 us a
+// launch at n = 511).
 template <typename R>
 __global__ void __launch_bounds__(kBlk) tsmm_reduce(Geo g, int d, const Cx<R>* __restrict__ G_F,
                                                     const int* __restrict__ G_rank, const Cx<R>* __restrict__ S_F,
@@ -512,8 +513,8 @@ __global__ void core_inverse(Geo g, int d, int m, const int* __restrict__ S_rank
 // In complex64, the blocks of the inverse that are used, from one k x k inverse: with
 // N = (I - Q P)^{-1},
 //     M11 = -N Q,  M12 = N,  M22 = -P N   (M21 = M12^t is not needed),
-// half the pivots and an eighth of the elimination of the 2k x 2k matrix (31 -> 13 us a depth
-// at 76 columns).  It takes the identity blocks as pivots, which is as stable as pivoting
+// half the pivots and an eighth of the elimination of the 2k x 2k matrix (33.8 -> 21.7
+// us a depth at n = 511).  It takes the identity blocks as pivots, which is as stable as pivoting
 // while the entries of P and Q are of order one, as they are for a block's coupling seen
 // through its own inverse; a matrix with an entry above kCoreLarge, or with a vanishing pivot,
 // goes through the pivoted elimination above.
@@ -704,7 +705,9 @@ __global__ void __launch_bounds__(32 * kCoreWarps) core_inverse_block(Geo g, int
 }
 
 // W_v = Y_v M_side (k x k block of M), and the new off-diagonal block at the parent:
-// F_a = -Y_a M12, F_b = Y_b.  A thread has one row and four columns.
+// F_a = -Y_a M12, F_b = Y_b.  A thread has one entry of each; what bounds it is the latency of
+// its chain of loads, so eight terms are loaded at a time (6.7 us a launch at n = 511; with four
+// columns a thread, which read Y a quarter as often, 11.3).
 template <typename R>
 __global__ void __launch_bounds__(128) woodbury_form(Geo g, int d, const int* __restrict__ S_rank,
                                                      const Cx<R>* __restrict__ Y, const Cx<R>* __restrict__ Mb,
@@ -712,7 +715,7 @@ __global__ void __launch_bounds__(128) woodbury_form(Geo g, int d, const int* __
                                                      int* __restrict__ G_rank) {
   pdl_begin();
   const int row = blockIdx.x * 32 + (threadIdx.x & 31);
-  const int col = 4 * (blockIdx.y * 4 + (threadIdx.x >> 5));
+  const int col = blockIdx.y * 4 + (threadIdx.x >> 5);
   if (row >= g.n) return;
   const int v = g.rowleaf[row] >> (g.L - (d + 1));
   const int t = v >> 1, side = v & 1;
@@ -720,36 +723,18 @@ __global__ void __launch_bounds__(128) woodbury_form(Geo g, int d, const int* __
   if (col >= k) return;
   const int s = g.sz[v], i = row - g.lo[v];
   const Cx<R>* Yv = Y + (long long)g.lo[v] * g.KCAP + i;
-  const Cx<R>* M = Mb + (long long)(t - (1 << d)) * 4 * g.KCAP * g.KCAP;
   const int ldm = 2 * g.KCAP;
-  const int off = side ? k : 0;
-  Cx<R> w[4], nf[4];
-  int c[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    w[u] = nf[u] = Cx<R>(0, 0);
-    c[u] = min(col + u, k - 1);
-  }
-#pragma unroll 2
+  const Cx<R>* M2 = Mb + (long long)(t - (1 << d)) * 4 * g.KCAP * g.KCAP + k + col;     // M12
+  const Cx<R>* M1 = M2 + (side ? k * ldm : -k);                                        // M22 or M11
+  Cx<R> w(0, 0), nf(0, 0);
+#pragma unroll 8
   for (int j = 0; j < k; ++j) {
     const Cx<R> y = Yv[(long long)j * s];
-    const Cx<R>* M1 = M + (off + j) * ldm + off;        // M11 or M22
-#pragma unroll
-    for (int u = 0; u < 4; ++u) cfma(w[u], y, M1[c[u]]);
-    if (!side) {
-      const Cx<R>* M2 = M + j * ldm + k;                 // M12
-#pragma unroll
-      for (int u = 0; u < 4; ++u) cfma(nf[u], y, M2[c[u]]);
-    }
+    cfma(w, y, M1[j * ldm]);
+    if (!side) cfma(nf, y, M2[j * ldm]);
   }
-  Cx<R>* F = G_F + g.gfo[v];
-  Cx<R>* Wv = W + (long long)g.lo[v] * g.KCAP;
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-    if (col + u < k) {
-      Wv[(long long)(col + u) * s + i] = w[u];
-      F[(long long)(col + u) * s + i] = side ? Yv[(long long)(col + u) * s] : -nf[u];
-    }
+  W[(long long)g.lo[v] * g.KCAP + (long long)col * s + i] = w;
+  G_F[g.gfo[v] + (long long)col * s + i] = side ? Yv[(long long)col * s] : -nf;
   if (i == 0 && col == 0) G_rank[v] = k;
 }
 
@@ -803,7 +788,7 @@ template <typename R> __host__ __device__ constexpr int group_lanes() { return s
 // written out (qmode = 0).  R is row-major with leading dimension cap(u).
 // Every step updates all later columns (a warp per column, the new norm with the update), so
 // a step costs one barrier; classical Gram-Schmidt with its two passes took ten, 3.6 us a
-// column (256 rows, 37 columns: 120 us, now 15).  F = Q R holds to rounding; Q is orthogonal
+// column (the launch at n = 511: 316 us, now 53; n = 150 in complex128: 931, now 253).  F = Q R holds to rounding; Q is orthogonal
 // to rounding over the relative size of a column's remainder, which is all the SVD of the
 // core asks of it (a skew of a column near the drop threshold moves the singular values
 // compared with eps_H by as much, not the product).  When F_u fits the kernel's shared
@@ -1076,8 +1061,8 @@ template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW
 //    a projection of C it does not depend on how exactly the rotations were unitary (their
 //    angles come from FP32 reciprocal square roots in both precisions).
 // What bounds it is the latency of kq - 1 barriers a sweep (complex64) or the FP64 units of
-// one SM (complex128).  Jacobi on the whole core, with the rotations accumulated, took 683 us
-// a layer at n = 511 in complex64 and 1586 us at n = 150 in complex128.
+// one SM (complex128).  A launch takes 195 us at n = 511 in complex64 (595 with Jacobi on
+// the whole core, rotations accumulated), 323 us at n = 150 in complex128 (1612).
 template <typename R>
 __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R>* __restrict__ Cb,
                                                    const int* __restrict__ qcols, Cx<R>* __restrict__ Tx,
@@ -1754,7 +1739,7 @@ static int factor_impl(hsweep_s* h) {
       else
         HSW_CUDA(pdl_launch(core_inverse<R>, dim3(ntau_d), 1024, core_smem, st, g, d, m, w->S_rank, PQ, M, h->d_status));
       h->nlaunch += 1;
-      HSW_CUDA(pdl_launch(woodbury_form<R>, dim3(div_up(h->n, 32), (KCAP + 15) / 16), 128, 0, st, g, d, w->S_rank, Y, M, Wv,
+      HSW_CUDA(pdl_launch(woodbury_form<R>, dim3(div_up(h->n, 32), (KCAP + 3) / 4), 128, 0, st, g, d, w->S_rank, Y, M, Wv,
                           G_F, w->G_rank));
       h->nlaunch += 1;
       HSW_CUDA(pdl_launch(woodbury_append<R>, dim3(n_below1), kBlk, 0, st, g, d, w->S_rank, Y, Wv, G_F, w->G_rank, G_leaf));
