@@ -110,6 +110,12 @@ SWEEP_TRAFFIC = {
                         "bytes": 5.5496e9},
 }
 TEAM_KERNEL_SRC = os.path.join(ROOT, "paper_1007_4290_gb300", "csrc", "sweep_team.cu")
+SLAB_KERNEL_SRC = os.path.join(ROOT, "paper_1007_4290_gb300", "csrc", "sweep_slab.cu")
+# the same for the sweep on dense-diagonal slabs
+SLAB_TRAFFIC = {
+    # profiles/sweep_slab_n1023_random_64rhs_dram.md: 4.719 GB read + 1.577 GB written
+    "n1023_random/64": {"sha256": "244113b7075d1e4f334ffaaafe72f0e653a8abbb856fcd843e91d48df96432e8", "bytes": 6.2957e9},
+}
 STRONG_KERNEL_SRC = os.path.join(ROOT, "paper_1007_4290_gb300", "csrc", "sweep_strong.cu")
 # the same for the sweep on the strongly admissible format (R = 2)
 STRONG_TRAFFIC = {
@@ -123,6 +129,14 @@ def recorded_strong_traffic(workload, nrhs):
     if rec is None or not os.path.exists(STRONG_KERNEL_SRC):
         return None
     digest = kernel_source_digest(STRONG_KERNEL_SRC, b"struct StrongPack {")
+    return rec["bytes"] if digest == rec["sha256"] else None
+
+
+def recorded_slab_traffic(workload, nrhs):
+    rec = SLAB_TRAFFIC.get("%s/%d" % (workload, nrhs))
+    if rec is None or not os.path.exists(SLAB_KERNEL_SRC):
+        return None
+    digest = kernel_source_digest(SLAB_KERNEL_SRC, b"struct SlabConfig {")
     return rec["bytes"] if digest == rec["sha256"] else None
 
 
@@ -654,9 +668,9 @@ def main():
         roof = {"bound": "hbm", "achieved": bytes_ / avg_s / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "peak_source": src}
     roof["frac"] = roof["achieved"] / roof["peak"]
-    roof["traffic"] = recorded_traffic(args.workload, nrhs)
     plan = h.sweep_plan(nrhs)
     slabs = plan["tma"] == 2 and plan["leaves_per_chunk"] <= 1    # dense-diagonal slabs (hsweep_sweep_plan)
+    roof["traffic"] = (recorded_slab_traffic if slabs else recorded_traffic)(args.workload, nrhs)
     roof["kernel"] = {2: "sweep_slab_kernel" if slabs else "sweep_team_kernel"}.get(plan["tma"], "sweep_kernel") + "<c64>"
     roof["plan"] = plan
     roof["launch_ms"] = avg_s * 1e3

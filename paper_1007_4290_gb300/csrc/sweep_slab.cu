@@ -41,10 +41,10 @@
 // with 64 right-hand sides: eight teams of 16), the same kernel runs as a cooperative grid
 // and exchanges tagged words through L2 (sweep_team.cu's protocol; L2X below).
 //
-// Measured (random media, eps_H 1e-6), per step, against the team sweep of sweep_team.cu:
-// complex64, n = 511: 2.0 us with one right-hand side (5.0), 2.9 with 16 (5.6), 4.5 with 64
-// (7.5); n = 1023: 2.8 with one (6.2), 4.3 with 16 (7.2), 7.7 with 64 (12.4); complex128, n =
-// 255: 5.1 with one (8.6).  What a step takes is instruction latency: with one right-hand
+// Measured (eps_H 1e-6), per step, against the team sweep of sweep_team.cu: complex64, n = 511,
+// lens: 2.0 us with one right-hand side (5.0), 2.8 with 16 (5.6), 4.5 with 64 (7.5); n = 1023,
+// random medium, the top ranks at 48: 2.9 with one (6.2), 5.3 with 16 (7.2), 8.4 with 64
+// (12.4); complex128, n = 255, random, with four: 4.9 (8.6).  What a step takes is instruction latency: with one right-hand
 // side 600 instructions a warp at one in four clocks and scheduler; with eight about 5 us of
 // FP32 multiply-adds and shared-memory reads.  Not kept: two half-CTAs with four right-hand
 // sides each on the same stages (register spills: 10.2 us against 8.0), and the paired FP32
