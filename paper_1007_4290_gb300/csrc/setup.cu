@@ -58,25 +58,9 @@ template <> struct Tiny<float> {
   static constexpr float quad = 1e-8f;
 };
 
-template <typename R> __device__ __forceinline__ Cx<R> warp_sum(Cx<R> v) {
-  for (int o = 16; o > 0; o >>= 1) v += shfl_xor(v, o);
-  return v;
-}
 template <typename R> __device__ __forceinline__ R warp_sum_r(R v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// Block-wide sum of a real value (result broadcast to all threads).
-template <typename R> __device__ R block_sum(R v, R* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  v = warp_sum_r(v);
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  R t = 0;
-  for (int i = 0; i < nw; ++i) t += red[i];
-  return t;
 }
 
 // 1 / a, by the Newton reciprocal where |a|^2 is well inside FP32's range
