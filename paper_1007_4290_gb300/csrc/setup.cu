@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, c
   const int s = g.sz[u], w = G_rank[u], ld = g.cap[u];
   Cx<R>* F = G_F + g.gfo[u];
   Cx<R>* Rm = Rb + g.rbo[u];                               // row-major qc x w, ld cap(u)
-  if ((w >= s && s <= g.QCAP) || s <= g.dense_max) {
+  if (s <= g.QCAP && (w >= s || s <= g.dense_max)) {
     for (int e = threadIdx.x; e < s * w; e += blockDim.x) {
       const int i = e % s, l = e / s;
       Rm[(long long)i * ld + l] = F[e];
@@ -1466,10 +1466,11 @@ static int setup_alloc(hsweep_s* h) {
   auto small_depth = [&](int d) { return deferred_core(d) <= qlim; };
   w->QCAP = w->WCAP;
   w->dense_max = es == sizeof(c64) ? kDenseRows : 0;
-  for (int d = 1; d <= L; ++d) {
+  for (int d = 1; d <= L; ++d)
     if (small_depth(d)) w->QCAP = std::max(w->QCAP, deferred_core(d));
-    if (h->tree.maxsz(d) <= w->dense_max) w->QCAP = std::max(w->QCAP, h->tree.maxsz(d));
-  }
+  // (node by node: n = 257 or 513 has depths with blocks of 128 and of 129 rows)
+  for (int v = 2; v < nn; ++v)
+    if (h->tree.sz[v] <= w->dense_max) w->QCAP = std::max(w->QCAP, h->tree.sz[v]);
   w->sfo.assign(nn, 0);
   w->gfo.assign(nn, 0);
   w->qro.assign(nn, 0);
