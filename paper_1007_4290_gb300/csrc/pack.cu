@@ -69,6 +69,10 @@ __global__ void pack_layers(int m0, int n, int L, int leaf, int nnodes, const in
 
 int hsw_pack(hsweep_s* h, int m0, int m1) {
   if (m1 <= m0) return HSWEEP_OK;
+  if (!h->pack_valid) {     // the first import: the other layers are empty, not what the allocation held
+    m0 = 0;
+    m1 = h->n;
+  }
   const size_t smem = (size_t)(h->nleaves + 1) * sizeof(long long);
   if (smem > 48 * 1024) return HSWEEP_ERR_ARG;
   if (h->prec == HSWEEP_FP64)
