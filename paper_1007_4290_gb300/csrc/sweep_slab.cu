@@ -1009,6 +1009,8 @@ int hsw_pack_slabs(hsweep_s* h, int m0, int m1, const std::vector<int>& rk) {
         h->d_off, (const c64*)h->d_fac, (const c64*)h->d_fac, h->layer_stride, h->d_rank, (c64*)h->d_slab, h->slab_cap, h->n, (uchar4*)h->d_slab_meta);
   h->nlaunch += 1;
   HSW_CUDA(cudaGetLastError());
+  // the setup and the import return with the work done: another stream may be set next
+  HSW_CUDA(cudaStreamSynchronize(h->stream));
   // the most columns of any layer and slab, for the shared-memory plan
   const int dC = h->slab_dC, C = 1 << dC;
   h->slab_W = h->slab_X = 0;
