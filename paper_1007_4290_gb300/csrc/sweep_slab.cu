@@ -601,6 +601,7 @@ __global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_ke
         x[urow * GS + ug] = xn;
       }
       }
+      __syncwarp();       // a row's lanes have read its coupling: its first lane may replace it
       if (t + 1 < nsteps) load_inputs(t + 1);
     }
     __syncthreads();
