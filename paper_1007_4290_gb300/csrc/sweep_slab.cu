@@ -957,10 +957,11 @@ static int apply_slab_impl(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* 
   return HSWEEP_OK;
 }
 
-// the slab sweep serves the automatic plan: an explicit team, group or thread choice, and
-// the tensor-core option, ask for the team sweep of sweep_team.cu
+// the slab sweep serves the automatic plan: sweep_kernel 2, an explicit team, group or thread
+// choice, and the tensor-core option, ask for the team sweep of sweep_team.cu
 static bool slab_usable(const hsweep_s* h) {
-  return h->slab_valid && h->opt.team == 0 && h->opt.groups == 0 && h->opt.team_threads == 0 && h->opt.sweep_tc == 0;
+  return h->slab_valid && h->opt.sweep_kernel == 0 && h->opt.team == 0 && h->opt.groups == 0 && h->opt.team_threads == 0 &&
+         h->opt.sweep_tc == 0;
 }
 
 }  // namespace
