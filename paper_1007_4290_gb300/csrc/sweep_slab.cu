@@ -957,18 +957,22 @@ static int apply_slab_impl(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* 
   return HSWEEP_OK;
 }
 
-// the slab sweep serves the automatic plan: sweep_kernel 2, an explicit team, group or thread
-// choice, and the tensor-core option, ask for the team sweep of sweep_team.cu
-static bool slab_usable(const hsweep_s* h) {
-  return h->slab_valid && h->opt.sweep_kernel == 0 && h->opt.team == 0 && h->opt.groups == 0 && h->opt.team_threads == 0 &&
-         h->opt.sweep_tc == 0;
-}
-
 }  // namespace
+
+// The slab sweep serves the automatic plan: sweep_kernel 1 or 2, an explicit team, group or
+// thread choice, and the tensor-core option, ask for other sweeps; the strongly admissible
+// format in complex128 runs on its records.  Such a handle reserves and packs no slabs (at
+// n = 1023 in complex64 they are 2.2 GB).
+static bool slab_wanted(const hsweep_s* h) {
+  const hsweep_opts& o = h->opt;
+  return o.sweep_kernel == 0 && o.team == 0 && o.groups == 0 && o.team_threads == 0 && o.sweep_tc == 0 &&
+         !(h->strong_R > 0 && h->prec == HSWEEP_FP64);
+}
 
 // The slab geometry: clusters of at most 16 CTAs (the largest that sm_103 schedules) and at
 // most 64 rows per slab in complex64, 32 in complex128.
 int hsw_slab_create(hsweep_s* h) {
+  if (!slab_wanted(h)) return HSWEEP_OK;
   const size_t es = h->fac_elem();
   const int cap_rows = h->prec == HSWEEP_FP64 ? 32 : 64;
   int target = h->prec == HSWEEP_FP64 ? 16 : 32;
@@ -1042,7 +1046,7 @@ int hsw_pack_slabs(hsweep_s* h, int m0, int m1, const std::vector<int>& rk) {
 // complex128 keeps the records: the FP64 units pay for the zeros (n = 127, 1 RHS 5.02, 5.68;
 // n = 511 7.86, 13.66).
 int hsw_strong_slabs(hsweep_s* h, int m, const void* G_F, const void* G_leaf, const long long* d_gfo, const int* G_rank) {
-  if (!h->d_slab || h->opt.sweep_kernel != 0 || h->L < 2 || h->prec == HSWEEP_FP64) return HSWEEP_OK;
+  if (!h->d_slab || h->L < 2) return HSWEEP_OK;
   pack_slabs<float><<<dim3(1 << h->slab_dC, 1, 8), 256, 0, h->stream>>>(m, h->L, h->leaf, h->nnodes, h->slab_dC,
       h->slab_rsD, h->d_lo, h->d_sz, d_gfo, (const c64*)G_leaf, (const c64*)G_F, 0, G_rank, (c64*)h->d_slab,
       h->slab_cap, h->n, (uchar4*)h->d_slab_meta);
@@ -1072,7 +1076,7 @@ int hsw_strong_slabs(hsweep_s* h, int m, const void* G_F, const void* G_leaf, co
 // their plans (over n = 63 to 1023 and 1 to 64 RHS it misses the faster one only where the two
 // are within 8 %)
 int hsw_strong_prefers_slabs(hsweep_s* h, int nrhs) {
-  if (!h->slab_strong || !h->spack_valid || !slab_usable(h)) return 0;
+  if (!h->slab_strong || !h->spack_valid) return 0;
   const SlabConfig s = choose_slab<float>(h, nrhs);
   const long long other = s.ok ? hsw_strong_cost(h, nrhs) : 0;
   return s.ok && (other == 0 || s.cost < other);
@@ -1085,7 +1089,6 @@ long long hsw_slab_exchange_bound(const hsweep_s* h) {
 }
 
 int hsw_slab_plan(hsweep_s* h, int nrhs, long long* out) {
-  if (!slab_usable(h)) return 0;
   const SlabConfig s = h->prec == HSWEEP_FP64 ? choose_slab<double>(h, nrhs) : choose_slab<float>(h, nrhs);
   if (!s.ok) return 0;
   const int rows = h->tree.maxsz(h->slab_dC);
@@ -1097,7 +1100,6 @@ int hsw_slab_plan(hsweep_s* h, int nrhs, long long* out) {
 
 int hsw_apply_slab(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* used, void* scratch, size_t scratch_bytes) {
   *used = false;
-  if (!slab_usable(h)) return HSWEEP_OK;
   if (h->prec == HSWEEP_FP64) return apply_slab_impl<double>(h, r, z, nrhs, used, scratch, scratch_bytes);
   return apply_slab_impl<float>(h, r, z, nrhs, used, scratch, scratch_bytes);
 }
