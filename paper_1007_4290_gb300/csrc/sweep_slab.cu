@@ -857,6 +857,20 @@ static SlabConfig choose_slab_uncached(const hsweep_s* h, int nrhs) {
   return best;
 }
 
+// complex128 with two right-hand sides a cluster against the team sweep, by estimates fitted to
+// n = 130 to 511, ranks 16 to 56 at the top and 8 to 14 right-hand sides.  Microseconds a step
+// (slabs, teams): n = 255, 8 RHS 7.1, 8.2, 10 RHS 7.1, 10.3; n = 300, 8 RHS 9.5, 9.4, 10 RHS 9.5, 12.7;
+// n = 511, 8 RHS 14.8, 12.3, 10 RHS 14.8, 20.7 (eps_H = 1e-6); the slabs' lead falls with the rank
+// (n = 257, top rank 46: 8 RHS 17.4, 11.3; 10 RHS 17.4, 16.4), so beyond 16 rows a slab has to be
+// ahead by 15 %.  One a cluster was never the slower (n = 64 to 511: 0.50 to 0.98 of the teams' time).
+static bool slower_than_teams(hsweep_s* h, int nrhs) {
+  const double other = 1e-3 * (double)hsw_team_cost(h, nrhs);
+  if (other <= 0) return false;
+  const int rows = h->tree.maxsz(h->slab_dC);
+  const double W = h->slab_W, rc = rows * (2.0 * W + rows);
+  return rows <= 16 ? 2.5 + 0.028 * W + 1.72e-3 * rc > 1.1 * other : 1.15 * (3.65 + 0.0563 * W + 1.24e-3 * rc) > other;
+}
+
 template <typename R>
 static SlabConfig choose_slab(hsweep_s* h, int nrhs) {
   for (const auto& e : h->slab_plans)
@@ -866,7 +880,8 @@ static SlabConfig choose_slab(hsweep_s* h, int nrhs) {
       s.per_launch = (int)e[6]; s.smem = (size_t)e[7]; s.cost = e[8];
       return s;
     }
-  const SlabConfig s = choose_slab_uncached<R>(h, nrhs);
+  SlabConfig s = choose_slab_uncached<R>(h, nrhs);
+  if (sizeof(R) == 8 && s.ok && s.G == 2 && slower_than_teams(h, nrhs)) s.ok = false;
   if (h->slab_plans.size() >= 64) h->slab_plans.erase(h->slab_plans.begin());
   h->slab_plans.push_back({nrhs, s.ok ? 1 : 0, s.l2x ? 1 : 0, s.G, s.dbufs, s.groups, s.per_launch, (long long)s.smem,
                            s.cost});
@@ -899,7 +914,9 @@ static int apply_slab_impl(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* 
     // room for the largest exchange of any plan for as many right-hand sides or fewer,
     // although this call may need none: a captured call with fewer of them can have a plan
     // that exchanges through L2, and must not allocate
-    const long long xcap = std::max(hsw_slab_exchange_bound(h), hsw_strong_exchange_bound(h, nrhs));
+    // (in complex128 the team sweep serves some counts between those of the slabs)
+    const long long xcap = std::max({hsw_slab_exchange_bound(h), hsw_strong_exchange_bound(h, nrhs),
+                                     sizeof(R) == 8 ? hsw_team_exchange_bound(h, nrhs) : 0LL});
     const long long need_x = std::max(xb, xcap) / es;
     if (need_x > h->xch_cap) {
       int rc = hsw_regrow(h, &h->d_xch, (size_t)(need_x * es));

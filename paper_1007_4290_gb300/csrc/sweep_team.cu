@@ -1096,6 +1096,32 @@ int hsw_team_plan(hsweep_s* h, int nrhs, long long* out) {
   return 1;
 }
 
+// complex128, ns a step of the batch (fitted to n = 130 to 511, top ranks 16 to 56, teams of 8 and
+// 16 CTAs, within 15 %); 0 if the team sweep would not run
+long long hsw_team_cost(hsweep_s* h, int nrhs) {
+  if (!team_usable(h) || h->prec != HSWEEP_FP64) return 0;
+  const TeamConfig cfg = choose_team<double>(h, nrhs);
+  if (!cfg.ok) return 0;
+  const int ngroups = (nrhs + cfg.G - 1) / cfg.G, rounds = (ngroups + cfg.nteams - 1) / cfg.nteams;
+  return (long long)(rounds * (5500.0 + 0.133 * (double)h->slab_bytes_max[cfg.dC] * cfg.G));
+}
+
+long long hsw_team_exchange_bound(const hsweep_s* h, int nrhs) {
+  if (!team_usable(h)) return 0;
+  long long most = 0;
+  for (int C = 1; C <= h->nleaves && C <= 2 * h->num_sms; C *= 2)
+    for (int G : {8, 5, 4, 2, 1}) {
+      TeamConfig cfg{};
+      cfg.C = C; cfg.dC = ilog2t(C); cfg.G = G;
+      cfg.nteams = std::min((nrhs + G - 1) / G, 2 * h->num_sms / C);      // at most two CTAs per SM
+      long long wb, xb;
+      if (h->prec == HSWEEP_FP64) team_scratch_need<double>(h, nrhs, cfg, &wb, &xb);
+      else team_scratch_need<float>(h, nrhs, cfg, &wb, &xb);
+      most = std::max(most, xb);
+    }
+  return most;
+}
+
 int hsw_apply_team(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* used, void* scratch, size_t scratch_bytes) {
   *used = false;
   if (!team_usable(h)) return HSWEEP_OK;

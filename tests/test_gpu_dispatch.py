@@ -37,3 +37,40 @@ def test_sweep_kernel_2_is_the_team_sweep(hs, n, prec, strong, nrhs):
         err = np.linalg.norm(z[s] - ref) / np.linalg.norm(ref)
         assert err < (1e-11 if prec == 0 else 1e-4), (s, err)      # as for the automatic choice
     h.free()
+
+
+# complex128 with more right-hand sides than clusters of 16 fit: eight and nine beyond 16 rows a
+# slab run as teams of one right-hand side each, ten on slabs again; each can be captured after a
+# call with more of them
+@pytest.mark.parametrize("n,plans", [(255, {7: 0, 8: 0, 10: 0, 16: 8}), (300, {7: 0, 8: 8, 9: 8, 10: 0, 14: 0, 16: 8}),
+                                     (511, {4: 0, 8: 8, 10: 0})])
+def test_complex128_plans_between_slabs_and_teams(hs, n, plans):
+    c, omega, pml = _problem(n, 3, ppw=16)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        h = hs.hsweep_setup(torch.tensor(c, device="cuda"), omega, pml, 1e-6, hs.default_opts(precision=0))
+        got = {k: h.sweep_plan(k)["leaves_per_chunk"] for k in plans}
+        assert got == plans
+        r = torch.randn(max(plans), n * n, dtype=torch.complex128, device="cuda")
+        top = max(k for k in plans if plans[k] == 0)
+        z = h.apply(r[:top])
+    s.synchronize()
+    for k in plans:
+        if k > top:
+            continue
+        with torch.cuda.stream(s):
+            rk = r[:k].clone()
+            zk = torch.zeros_like(rk)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            code = hs._lib.hsweep_apply(h.raw, hs._ptr(rk, torch.complex128), hs._ptr(zk, torch.complex128), k)
+        assert code == hs.OK
+        with torch.cuda.stream(s):
+            g.replay()
+            ref = h.apply(rk)
+        s.synchronize()
+        assert torch.equal(zk, ref), k
+        # any two plans: rounding apart (the sweeps' parity bound in complex128, each)
+        assert ((zk - z[:k]).norm() / z[:k].norm()).item() < 2e-11, k
+    assert h.status()[0] == 0
+    h.free()
