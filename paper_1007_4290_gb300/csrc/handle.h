@@ -189,6 +189,7 @@ int hsw_apply_team(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* used, vo
                    size_t scratch_bytes = 0);
 size_t hsw_apply_team_scratch_bytes(hsweep_s* h, int nrhs);
 int hsw_team_plan(hsweep_s* h, int nrhs, long long* out8);   // 1 if the team kernel would run
+void hsw_team_load(const hsweep_s* h);                   // loads the kernels that its planning looks at
 long long hsw_team_cost(hsweep_s* h, int nrhs);           // complex128: its estimate, ns a step of the batch; 0 if it would not run
 long long hsw_team_exchange_bound(const hsweep_s* h, int nrhs);     // bytes: any plan for at most nrhs
 // sweep_slab.cu: geometry and buffers of the dense-diagonal slabs, their packing (rk: the

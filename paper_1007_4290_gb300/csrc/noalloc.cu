@@ -24,6 +24,7 @@ void hsw_noalloc_bind(hsweep_s* h) {
     p = nullptr;
   }
   h->noalloc_scratch = p;
+  hsw_team_load(h);
 }
 
 extern "C" int hsweep_apply_noalloc(hsweep_t h, const hsw_c128* r, hsw_c128* z, int nrhs) {

@@ -33,6 +33,7 @@
 // b = sum (Im f) x, f x = (Re a - Im b, Im a + Re b).
 #include <cstdlib>
 #include <type_traits>
+#include <atomic>
 #include "handle.h"
 #include "sweep_common.cuh"
 #include "tma.cuh"
@@ -882,6 +883,15 @@ static int resident_for(const hsweep_s* h, int G, size_t smem, int nt) {
   return nt == kThreads2 ? resident_for_nt<R, kThreads2>(h, G, smem) : resident_for_nt<R, kThreads>(h, G, smem);
 }
 
+template <typename R, int... G>
+static void load_kernels() {
+  cudaFuncAttributes fa;
+  const cudaError_t e[] = {cudaFuncGetAttributes(&fa, sweep_team_kernel<R, G, 0, kThreads>)...,
+                           cudaFuncGetAttributes(&fa, sweep_team_kernel<R, G, 0, kThreads2>)...};
+  for (cudaError_t x : e)
+    if (x != cudaSuccess) cudaGetLastError();      // the plan that asks for the kernel reports it
+}
+
 // Team size C, right-hand sides per team G and threads per CTA: the fewest rounds of 2n-1
 // dependent steps, a step costing a fixed latency (exchange through L2, barriers, growing
 // slowly with the team's depth) plus work that grows with the slab's rows times G per thread.
@@ -1120,6 +1130,17 @@ long long hsw_team_exchange_bound(const hsweep_s* h, int nrhs) {
       most = std::max(most, xb);
     }
   return most;
+}
+
+// CUDA loads a kernel into device memory when it is first used.  hsweep_apply_noalloc asks what a
+// team plan would need also where hsweep_apply runs another sweep, so the kernels that planning
+// looks at are loaded when a handle is created (once a device and precision).
+void hsw_team_load(const hsweep_s* h) {
+  static std::atomic<unsigned long long> loaded[2];
+  const unsigned long long bit = 1ULL << (h->device & 63);
+  if (loaded[h->prec == HSWEEP_FP64].fetch_or(bit) & bit) return;
+  if (h->prec == HSWEEP_FP64) load_kernels<double, 1, 2, 4, 5, 8>();
+  else load_kernels<float, 1, 2, 4, 5, 8>();
 }
 
 int hsw_apply_team(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* used, void* scratch, size_t scratch_bytes) {
