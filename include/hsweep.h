@@ -387,15 +387,16 @@ HSWEEP_API int hsweep_setup_tuning(hsweep_t h, double* out6);
  * property of the library, not of the method.)
  *   - Scratch comes from one fixed device array inside the library, of
  *     HSWEEP_NOALLOC_SCRATCH_BYTES bytes (32 MiB), which every GPU that loads the
- *     library reserves until the process exits.  A call whose scratch need
+ *     library reserves until the process exits (with 9 MiB more for the slots through
+ *     which the CTAs of a batch exchange partial sums).  A call whose scratch need
  *     (about nrhs * n*n * 8 bytes in HSWEEP_MIXED, * 16 in HSWEEP_FP64, plus a few MiB)
  *     exceeds it returns HSWEEP_ERR_ARG and does nothing.
- *   - The array's device address is looked up when the handle is created
+ *   - The arrays' device addresses are looked up when the handle is created
  *     (hsweep_setup / hsweep_create, on the handle's device) and kept in the handle;
  *     this call makes no lookup.  The current device must be the handle's device.
  *   - Downward handles (sweep_dir = -1) are refused with HSWEEP_ERR_ARG (their apply
  *     needs reflected copies of r and z).
- *   - Every call shares the one array and it keeps the last call's contents; calls
+ *   - Every call shares these arrays and they keep the last call's contents; calls
  *     whose GPU work overlaps (other streams, other handles, other threads) race on it.
  *   - r and z are as in hsweep_apply.  No cudaMalloc, cudaFree or allocating library
  *     routine is called.  Stream-ordered; returns after enqueue.

@@ -137,9 +137,12 @@ struct hsweep_s {
   int core_mode[2] = {-1, -1};
   float core_ms[2][2] = {{0, 0}, {0, 0}};
 
-  // device address of the library's fixed scratch array for hsweep_apply_noalloc, looked
-  // up on the handle's device when the handle is created (noalloc.cu); null if that failed
+  // device addresses of the library's fixed arrays for hsweep_apply_noalloc (scratch, and the
+  // slab sweep's exchange slots), looked up on the handle's device when the handle is created
+  // (noalloc.cu); null if that failed
   void* noalloc_scratch = nullptr;
+  void* noalloc_slots = nullptr;
+  size_t noalloc_slot_bytes = 0;
 
   // instrumentation: kernel launches made by this handle, and (when prof is set) a
   // pair of CUDA events around every sweep-kernel launch on the handle's stream

@@ -897,10 +897,9 @@ static int apply_slab_impl(hsweep_s* h, const c128* r, c128* z, int nrhs, bool* 
   const long long wb = al((long long)nrhs * h->N * es, 256);
   const long long xb = cfg.l2x ? 2LL * cfg.per_launch * C * h->slab_W * cfg.G * es : 0;
   void* wptr = scratch;
-  void* xptr = static_cast<unsigned char*>(scratch) + wb;
-  if (scratch) {
-    // a caller's buffer too small for the exchange slots: the team sweep, which it was sized for
-    if (wb + xb > (long long)scratch_bytes) return HSWEEP_OK;
+  void* xptr = h->noalloc_slots;
+  if (scratch) {      // the scratch of hsweep_apply_noalloc, and its array for the exchange slots
+    if (wb > (long long)scratch_bytes || xb > (long long)h->noalloc_slot_bytes) return HSWEEP_OK;
   } else {
     const long long need_w = (long long)nrhs * h->N;
     if (need_w > h->wcache_cap) {
