@@ -29,8 +29,11 @@ constexpr int kRedBlocks = 304;   // at most 2 x 152 SMs of partial sums per vec
 
 // Blocks per vector of the reductions: all of kRedBlocks for a few vectors, fewer for a batch,
 // down to 32 (the sums across a warp are FP64 additions too: with 304 blocks for each of 64
-// vectors of 1023 x 1023 they cost half as much as the products)
-static int red_blocks(int nvec) { return std::max(32, std::min(kRedBlocks, 2432 / std::max(1, nvec))); }
+// vectors of 1023 x 1023 they cost half as much as the products).  With krylov_lowp the sums of a
+// thread are FP32, and fewer blocks would make them longer (109 entries for 14 at n = 1023 with 64).
+static int red_blocks(int nvec, bool lowp) {
+  return lowp ? kRedBlocks : std::max(32, std::min(kRedBlocks, 2432 / std::max(1, nvec)));
+}
 
 constexpr int kDotChunk = 4;      // basis vectors per pass over w
 
@@ -298,7 +301,7 @@ static int batched_dots(hsweep_s* h, int first, int nv, const c128* w, int nrhs,
                         bool lowp, bool with_norm = false) {
   KrylovWork* k = h->kw;
   const int nt = nv + (with_norm ? 1 : 0);
-  const int B = red_blocks(nrhs);
+  const int B = red_blocks(nrhs, lowp);
   if (lowp) dots_kernel<float><<<dim3(B, nrhs), 256, 0, h->stream>>>(k->d_V + first, nv, nt, w, h->N, k->partial);
   else dots_kernel<double><<<dim3(B, nrhs), 256, 0, h->stream>>>(k->d_V + first, nv, nt, w, h->N, k->partial);
   h->nlaunch += 1;
@@ -312,7 +315,7 @@ static int batched_dots(hsweep_s* h, int first, int nv, const c128* w, int nrhs,
 // ||x[s]|| for every s, on the host
 static int norms(hsweep_s* h, const c128* x, int nrhs, std::vector<double>& out, bool lowp = false) {
   KrylovWork* k = h->kw;
-  const int B = red_blocks(nrhs);
+  const int B = red_blocks(nrhs, lowp);
   if (lowp) sqnorm_kernel<float><<<dim3(B, nrhs), 256, 0, h->stream>>>(x, h->N, k->partial);
   else sqnorm_kernel<double><<<dim3(B, nrhs), 256, 0, h->stream>>>(x, h->N, k->partial);
   h->nlaunch += 1;
