@@ -58,6 +58,27 @@ template <> struct Tiny<float> {
   static constexpr float quad = 1e-8f;
 };
 
+// Thresholds and shared memory of svd_jacobi for cores of at most qcap x qcap.
+//   thr: columns with smaller squared norms (relative to the largest column's) are not rotated.
+//   rem: the pivoted Gram-Schmidt ends when the squares of all that is left sum to this.
+// Both are fractions of the truncation threshold eps.  A quarter and a hundredth in complex64: what is
+// left holds no singular value above eps / 2 (a sixteenth for rem takes two columns more at the top
+// of n = 255 in the strong format, 286 for 266 ms a setup; columns alone against eps / 4, without a bound on
+// their sum, 252 ms, but 128 aligned ones hold a value of 2.8 eps).
+template <typename R>
+struct SvdPlan {
+  int entries;       // of the core
+  size_t smem;       // the core, two rows of R, norms, singular values and index tables
+  R thr;
+  float rem;
+  SvdPlan(int qcap, double eps) {
+    entries = qcap * qcap;
+    smem = ((size_t)entries + 2 * qcap) * sizeof(Cx<R>) + (size_t)(3 * qcap + 1) * sizeof(R) + (size_t)2 * qcap * sizeof(int) + 16;
+    thr = (R)std::max((double)Tiny<R>::neg, (sizeof(R) == 4 ? 0.01 : 0.0025) * eps * eps);
+    rem = (float)((sizeof(R) == 4 ? 0.25 : 0.0025) * eps * eps);
+  }
+};
+
 template <typename R> __device__ __forceinline__ R warp_sum_r(R v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
@@ -1034,9 +1055,11 @@ template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW
 //   T_b = conj(P) Sigma^(1/2) (qb x k'),  T_a = C P Sigma^(-1/2) (qa x k'),
 // P the right singular vectors kept: T_a T_b^t = C P P^*, the projection of C.
 //
-// 1. Gram-Schmidt with column pivoting, C = Q R, stopped when every remaining column is
-//    below the threshold thr (relative to the largest): the block's numerical rank is a third
-//    to a half of the core's size.  Each warp picks the pivot from the column norms (no
+// 1. Gram-Schmidt with column pivoting, C = Q R, stopped when the squared norms of the
+//    remaining columns sum to at most rem (relative to the largest column's), or to the rounding
+//    noise of the core: no singular value above sqrt(rem) is left behind, however the remaining
+//    columns are aligned.  The block's numerical rank is a third to a half of the core's size.
+//    Each warp picks the pivot from the column norms (no
 //    broadcast), takes its columns' inner products with the pivot column, updates them and
 //    leaves their new norms: one barrier a step.  Q is not kept: row k of R, conjugated, goes
 //    into the storage of the k-th pivot column.
@@ -1050,7 +1073,7 @@ template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW
 template <typename R>
 __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R>* __restrict__ Cb,
                                                    const int* __restrict__ qcols, Cx<R>* __restrict__ Tx,
-                                                   int* __restrict__ newrank, int smem_entries, R thr) {
+                                                   int* __restrict__ newrank, int smem_entries, R thr, float rem) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char sm[];
   const int a = g.list[blockIdx.x], b = a + 1, t = a >> 1;
@@ -1081,14 +1104,21 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
   }
   __syncthreads();
   // normalise by the largest column norm
-  R mx = 0;
-  for (int j = lane; j < qb; j += 32) mx = fmax(mx, nrm[j]);
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  R mx = 0, tot = 0;
+  for (int j = lane; j < qb; j += 32) {
+    mx = fmax(mx, nrm[j]);
+    tot += nrm[j];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  }
   if (!(mx > 0)) {
     if (threadIdx.x == 0) { newrank[a] = 0; newrank[b] = 0; }
     return;
   }
   const R scale = sqrt(mx), iscale = R(1) / scale;
+  rem = fmaxf(rem, (float)(R(Tiny<R>::neg) * (tot / mx)));
   __syncthreads();
   for (int j = warp; j < qb; j += nw) {
     for (int i = lane; i < qa; i += 32) C[j * ld + i] = iscale * C[j * ld + i];
@@ -1112,7 +1142,12 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
       const int op = __shfl_xor_sync(0xffffffffu, p, o);
       if (ob > best || (ob == best && op < p)) { best = ob; p = op; }
     }
-    if (!(best > thr)) break;
+    if (!((float)best > rem)) {
+      float left = 0;      // (FP32: the FP64 unit is slow, and a threshold is compared)
+      for (int j = lane; j < qb; j += 32) left += fmaxf(0.f, (float)nr[j]);
+      left = warp_sum_r(left);
+      if (!(left > rem)) break;
+    }
     const R rs = rsqrt_of(best), ib = rcp_of(best);
     const Cx<R>* cp = C + p * ld;
     // kGL lanes a column: a warp in complex64, eight lanes in complex128 (an FP64 instruction
@@ -1266,9 +1301,9 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
       smax = fmax(smax, sig[l]);
     }
     order[rk] = j;
-    // (a column below thr may have been left unrotated: only those clear of it are orthogonal
-    // to the others; at eps below the rounding noise this is what ends the expansion)
-    if (rk < g.r_max && sig[j] > R(eps) * smax && sig[j] * sig[j] > R(4) * thr) atomicMax(&s_keep, rk + 1);
+    // (a column below thr was left unrotated and need not be orthogonal to the others: at eps
+    // below the rounding noise this is what ends the expansion)
+    if (rk < g.r_max && sig[j] > R(eps) * smax && sig[j] * sig[j] > R(1.01) * thr) atomicMax(&s_keep, rk + 1);
   }
   __syncthreads();
   const int keep = s_keep;
@@ -1595,10 +1630,7 @@ static int factor_impl(hsweep_s* h) {
   const size_t qr_base = ((size_t)g.cap_max * (2 * sizeof(R) + sizeof(int)) + 15) & ~size_t(15);
   const int qs_entries = qr_base < 226 * 1024 ? (int)((226 * 1024 - qr_base) / es) : 0;
   const size_t qr_smem = qr_base + (size_t)qs_entries * es;
-  // the SVD's shared memory: C, two rows of R, norms, singular values and index tables
-  const size_t svd_tail = (size_t)2 * QCAP * es + (size_t)(3 * QCAP + 1) * sizeof(R) + (size_t)2 * QCAP * sizeof(int) + 16;
-  const int svd_entries = QCAP * QCAP;
-  const size_t svd_smem = (size_t)svd_entries * es + svd_tail;
+  const SvdPlan<R> svd(QCAP, h->eps_H);
   // one shared-memory carveout for every kernel of the layer loop, so that consecutive
   // launches do not reconfigure the SMs' L1/shared split
   {
@@ -1615,8 +1647,8 @@ static int factor_impl(hsweep_s* h) {
   HSW_CUDA(cudaFuncSetAttribute(core_inverse_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)core_smem));
   HSW_CUDA(cudaFuncSetAttribute(core_inverse_block, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   HSW_CUDA(cudaFuncSetAttribute(qr_mgs<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qr_smem));
-  HSW_CUDA(cudaFuncSetAttribute(svd_jacobi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)svd_smem));
-  if (core_smem > 227 * 1024 || qr_smem > 227 * 1024 || svd_smem > 227 * 1024)
+  HSW_CUDA(cudaFuncSetAttribute(svd_jacobi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)svd.smem));
+  if (core_smem > 227 * 1024 || qr_smem > 227 * 1024 || svd.smem > 227 * 1024)
     return HSWEEP_ERR_ARG;
 
   // Autotuning of the core products (step 2a), complex64 only: on layer tune_m, the first
@@ -1624,9 +1656,6 @@ static int factor_impl(hsweep_s* h) {
   // recompression) runs both kernels, timed with CUDA events, and the faster one serves that
   // kind of launch from then on; before it, and in complex128, the CUDA-core kernel runs.
   const int tune_m = h->n / 2;
-  // SVD: columns below a fraction of the truncation threshold (squared, relative) are left out:
-  // a quarter in complex64 (rounding noise lies just below), a twentieth in complex128
-  const R thr = (R)std::max((double)Tiny<R>::neg, (sizeof(R) == 4 ? 0.0625 : 0.0025) * h->eps_H * h->eps_H);
   constexpr int kCT = core_tile_edge<R>();
   const int core_tiles = ((QCAP + kCT - 1) / kCT) * ((QCAP + kCT - 1) / kCT);
   const int gemm_tiles = ((h->tree.maxsz(1) + kCT - 1) / kCT) * ((h->r_max + kCT - 1) / kCT);
@@ -1685,7 +1714,7 @@ static int factor_impl(hsweep_s* h) {
     gp.list = w->d_lists + pair_off;
     int rc = core_product(gp, np_list, kind);
     if (rc) return rc;
-    HSW_CUDA(pdl_launch(svd_jacobi<R>, dim3(np_list), 1024, svd_smem, st, gp, h->eps_H, Cb, w->qcols, Tx, w->newrank, svd_entries, thr));
+    HSW_CUDA(pdl_launch(svd_jacobi<R>, dim3(np_list), 1024, svd.smem, st, gp, h->eps_H, Cb, w->qcols, Tx, w->newrank, svd.entries, svd.thr, svd.rem));
     if (store) {
       HSW_CUDA(pdl_launch(recompress_gemm<R>, dim3(gemm_tiles, nn_list), 256, 0, st, gl, G_F, w->qcols, w->qmode, Tx, w->newrank, store, h->d_off, store_rank));
       h->nlaunch += 3;

@@ -1,0 +1,50 @@
+// C entry points that launch single kernels of csrc/setup.cu and device helpers of csrc/common.cuh on
+// the caller's data (host arrays), for tests/test_gpu_setup_kernels.py.
+#include "../../paper_1007_4290_gb300/csrc/setup.cu"
+
+#define ENTRY extern "C" __attribute__((visibility("default"))) int
+
+namespace {
+
+template <typename T>
+struct Dev {
+  T* p = nullptr;
+  size_t n;
+  explicit Dev(size_t n_, const T* src = nullptr) : n(n_) {
+    if (cudaMalloc(&p, n * sizeof(T)) != cudaSuccess) p = nullptr;
+    if (p && src) cudaMemcpy(p, src, n * sizeof(T), cudaMemcpyHostToDevice);
+    else if (p) cudaMemset(p, 0, n * sizeof(T));
+  }
+  ~Dev() { cudaFree(p); }
+  bool get(T* dst) { return cudaMemcpy(dst, p, n * sizeof(T), cudaMemcpyDeviceToHost) == cudaSuccess; }
+};
+
+// the truncated SVD of one core C (qa x qb, column-major): T_a (ld qcap, r_max columns), T_b, rank
+template <typename R>
+int svd(int qa, int qb, int qcap, int r_max, double eps, const Cx<R>* C, Cx<R>* Ta, Cx<R>* Tb, int* rank) {
+  if (qa > qcap || qb > qcap) return 1;
+  const int list[1] = {0}, qcols[2] = {qa, qb};
+  Dev<int> dl(1, list), dq(2, qcols), dr(2);
+  Dev<Cx<R>> dC((size_t)qcap * qcap), dT((size_t)2 * qcap * r_max);
+  if (!dl.p || !dq.p || !dr.p || !dC.p || !dT.p) return 2;
+  cudaMemcpy(dC.p, C, sizeof(Cx<R>) * qa * qb, cudaMemcpyHostToDevice);
+  Geo g{};
+  g.QCAP = qcap; g.r_max = r_max; g.list = dl.p;
+  const SvdPlan<R> s(qcap, eps);
+  if (s.smem > 227 * 1024) return 3;
+  cudaFuncSetAttribute(svd_jacobi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
+  svd_jacobi<R><<<1, 1024, s.smem>>>(g, eps, dC.p, dq.p, dT.p, dr.p, s.entries, s.thr, s.rem);
+  if (cudaDeviceSynchronize() != cudaSuccess) return 4;
+  cudaMemcpy(Ta, dT.p, sizeof(Cx<R>) * qcap * r_max, cudaMemcpyDeviceToHost);
+  cudaMemcpy(Tb, dT.p + (size_t)qcap * r_max, sizeof(Cx<R>) * qcap * r_max, cudaMemcpyDeviceToHost);
+  return cudaMemcpy(rank, dr.p, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess ? 0 : 5;
+}
+
+}  // namespace
+
+ENTRY svd_f32(int qa, int qb, int qcap, int r_max, double eps, const Cx<float>* C, Cx<float>* Ta, Cx<float>* Tb, int* rank) {
+  return svd<float>(qa, qb, qcap, r_max, eps, C, Ta, Tb, rank);
+}
+ENTRY svd_f64(int qa, int qb, int qcap, int r_max, double eps, const Cx<double>* C, Cx<double>* Ta, Cx<double>* Tb, int* rank) {
+  return svd<double>(qa, qb, qcap, r_max, eps, C, Ta, Tb, rank);
+}

@@ -1,0 +1,89 @@
+"""Single kernels of the setup on constructed inputs, against NumPy in complex128: launched through
+tests/kernels/setup_entries.cu, which is compiled with the library's own flags and objects."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+U32, U64 = 2.0 ** -24, 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    import __graft_entry__ as g
+    b = g._build_module()
+    objs = os.path.join(b.HERE, "_build")
+    if not os.path.exists(os.path.join(objs, "setup.o")):
+        b.build()
+    out = str(tmp_path_factory.mktemp("kernels") / "entries.so")
+    rest = [o for o in sorted(glob.glob(os.path.join(objs, "*.o"))) if os.path.basename(o) != "setup.o"]
+    cmd = [b.nvcc(), *b.ARCH, *b.FLAGS, "-shared", "-o", out, os.path.join(HERE, "kernels", "setup_entries.cu"), *rest, "-ldl"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    torch.zeros(1, device="cuda")
+    return ctypes.CDLL(out)
+
+
+def _types(prec):
+    return (np.complex64, U32) if prec == 32 else (np.complex128, U64)
+
+
+def _svd(lib, prec, C, eps, r_max=56, qcap=None):
+    ct, _ = _types(prec)
+    qa, qb = C.shape
+    qcap = qcap or max(qa, qb)
+    Cf = np.asfortranarray(C.astype(ct))
+    Ta, Tb = np.zeros((r_max, qcap), ct), np.zeros((r_max, qcap), ct)
+    rank = ctypes.c_int(-1)
+    fn = lib.svd_f32 if prec == 32 else lib.svd_f64
+    rc = fn(qa, qb, qcap, r_max, ctypes.c_double(eps), Cf.ctypes.data_as(ctypes.c_void_p),
+            Ta.ctypes.data_as(ctypes.c_void_p), Tb.ctypes.data_as(ctypes.c_void_p), ctypes.byref(rank))
+    assert rc == 0, rc
+    k = rank.value
+    return Ta[:k, :qa].T.astype(complex), Tb[:k, :qb].T.astype(complex), np.array(Cf, dtype=complex)
+
+
+def _unitary(rng, n, k):
+    return np.linalg.qr(rng.standard_normal((n, k)) + 1j * rng.standard_normal((n, k)))[0]
+
+
+# eps, and sizes: one column, a leaf pair, ragged cores, the largest dense core of complex64
+@pytest.mark.parametrize("prec,eps", [(32, 1e-6), (32, 1e-7), (32, 1e-3), (64, 1e-6), (64, 1e-12)])
+@pytest.mark.parametrize("qa,qb", [(1, 1), (8, 7), (49, 98), (98, 49), (97, 97), (112, 112), (128, 127)])
+def test_svd_keeps_the_singular_values_above_eps(lib, prec, eps, qa, qb):
+    if prec == 64 and max(qa, qb) > 112:
+        pytest.skip("beyond the cores of complex128")
+    _, u = _types(prec)
+    rng = np.random.default_rng(qa * 1000 + qb)
+    q = min(qa, qb)
+    s = 0.5 ** np.arange(q)
+    C = (_unitary(rng, qa, q) * s) @ _unitary(rng, qb, q).conj().T
+    Ta, Tb, C = _svd(lib, prec, C, eps)
+    s = np.linalg.svd(C, compute_uv=False)
+    # rounding of a column update and of a rotation: a few u of the largest value, each of up to 40
+    noise = 40 * u
+    k = Ta.shape[1]
+    # at most eps / 2 is out of the expansion's reach: sqrt(1 + 1/4) < 1.2
+    assert k >= min(56, np.sum(s > 1.2 * eps * s[0] + noise * s[0])), (k, s[:k + 3])
+    assert k <= np.sum(s > 0.9 * eps * s[0] - noise * s[0])
+    left = s[k] if k < q else 0.0
+    assert np.linalg.norm(C - Ta @ Tb.T, 2) <= 1.2 * left + (noise + (0.5 * eps if k < q else 0)) * s[0]
+
+
+@pytest.mark.parametrize("prec,eps", [(32, 1e-6), (64, 1e-6), (64, 1e-10)])
+def test_svd_keeps_a_value_spread_over_many_small_columns(lib, prec, eps):
+    # every column but the first is a fifth of eps; 100 of them aligned make a singular value of 2 eps
+    C = np.zeros((112, 112), complex)
+    C[0, 0] = 1
+    C[1, 1:101] = 0.2 * eps
+    Ta, Tb, C = _svd(lib, prec, C, eps)
+    assert Ta.shape[1] == 2
+    assert np.linalg.norm(C - Ta @ Tb.T, 2) < 0.1 * eps
+
