@@ -154,7 +154,7 @@ __device__ __forceinline__ double rsqrt_any(double x) {
 // cs and the phase are refined to the storage precision.
 template <typename R>
 struct JacobiRotation {
-  float gg;
+  float gg, t;      // the squared cosine; the tangent
   R cs, dn;
   Cx<R> sne;
   __device__ __forceinline__ bool needed(R al, R be, Cx<R> ga, float tol2) {
@@ -167,8 +167,9 @@ struct JacobiRotation {
     const float ig = rsqrtf(gg);
     const float z = 0.5f * (float)((be - al) * s) * ig;
     // (z reaches 1e29 in complex128, where its square would overflow)
-    const float za = fabsf(z), tt = copysignf(1.0f, z) / (za + (za < 1e9f ? sqrtf(fmaf(z, z, 1.0f)) : za));
-    const R tr = (R)tt;
+    const float za = fabsf(z);
+    t = copysignf(1.0f, z) / (za + (za < 1e9f ? sqrtf(fmaf(z, z, 1.0f)) : za));
+    const R tr = (R)t;
     cs = rsqrt_of(fma(tr, tr, R(1)));
     R igr = (R)ig;
     if (sizeof(R) == 8) igr = igr * fma(R(-0.5) * abs2(gn) * igr, igr, R(1.5));

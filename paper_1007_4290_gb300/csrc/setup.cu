@@ -1044,6 +1044,14 @@ __global__ void __launch_bounds__(256) core_product_tc(Geo g, const Cx<float>* _
   }
 }
 
+// One-sided Jacobi ends after a sweep whose cosines were at most sqrt(quad), if the rotations
+// cannot have left more than the orthogonality tolerance: a rotation by tan t mixes the other
+// inner products of its two columns, so up to t times the largest cosine is left, t being small
+// between well-separated singular values (the quadratic convergence) but not within a cluster.
+template <typename R> __device__ __forceinline__ bool rotations_done(float gg, float t) {
+  return t * sqrtf(gg) <= 2.0f * sqrtf(Tiny<R>::jac2);
+}
+
 // Shuffle-sum within aligned groups of GW lanes (GW = 16 or 32).
 template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW) {
   for (int o = GW >> 1; o > 0; o >>= 1) v += shfl_xor(v, o);
@@ -1085,7 +1093,7 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
   R* sig = nrm + 2 * g.QCAP;                                       // [QCAP + 1]
   int* slot = reinterpret_cast<int*>(sig + g.QCAP + 1);            // [QCAP] column storage of row k
   int* order = slot + g.QCAP;                                      // [QCAP]
-  __shared__ int s_rot, s_keep;
+  __shared__ int s_rot, s_gg, s_t, s_keep;
   if (qa == 0 || qb == 0) {
     if (threadIdx.x == 0) { newrank[a] = 0; newrank[b] = 0; }
     return;
@@ -1200,7 +1208,7 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
   const int gpw = 32 / GW;                    // groups per warp
   for (int sweep = 0; sweep < 40; ++sweep) {
     __syncthreads();
-    if (threadIdx.x == 0) s_rot = 0;
+    if (threadIdx.x == 0) s_rot = s_gg = s_t = 0;
     // squared column norms, exact at the start of every sweep and carried through its
     // rounds by the rotation's own update (a rotation by tan t of the pair (p, q) with
     // <p, q> = g maps |p|^2 to |p|^2 - t |g| and |q|^2 to |q|^2 + t |g|), so a pair's test
@@ -1251,7 +1259,12 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
           const R cs = rot.cs;
           const Cx<R> sne = rot.sne, snc = conj(sne);
           if (gl == 0) {
-            if (rot.gg > Tiny<R>::quad) s_rot = 1;
+            if (rot.gg > Tiny<R>::quad) {
+              s_rot = 1;
+            } else {
+              atomicMax(&s_gg, __float_as_int(rot.gg));      // (nonnegative floats order as integers)
+              atomicMax(&s_t, __float_as_int(fabsf(rot.t)));
+            }
             sig[ip] = fmax(R(0), al - rot.dn);
             sig[iq] = be + rot.dn;
           }
@@ -1281,7 +1294,7 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
       }
       __syncthreads();
     }
-    if (s_rot == 0) break;       // every cosine of this sweep was rounding noise or nearly so
+    if (s_rot == 0 && rotations_done<R>(__int_as_float(s_gg), __int_as_float(s_t))) break;
   }
   // singular values, ordering, truncation
   for (int j = warp; j < kq; j += nw) {

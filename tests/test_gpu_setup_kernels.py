@@ -87,3 +87,20 @@ def test_svd_keeps_a_value_spread_over_many_small_columns(lib, prec, eps):
     assert Ta.shape[1] == 2
     assert np.linalg.norm(C - Ta @ Tb.T, 2) < 0.1 * eps
 
+
+# cosines between the columns of T_b: the rotations' tolerance (4e-7, 1e-15), twice, and the rounding
+# of the sweeps' rotations, a few u each of at most 20 sweeps
+@pytest.mark.parametrize("prec,spread", [(32, 1e-4), (32, 1e-2), (32, 0.0), (64, 1e-8), (64, 1e-4), (64, 0.0)])
+def test_svd_columns_of_a_cluster_are_orthogonal(lib, prec, spread):
+    _, u = _types(prec)
+    rng = np.random.default_rng(7)
+    q, m = 96, 40
+    s = np.concatenate([1 + spread * rng.standard_normal(m), 1e-2 * (1 + spread * rng.standard_normal(m // 2))])
+    k = len(s)
+    C = (_unitary(rng, q, k) * s) @ _unitary(rng, q, k).conj().T
+    Ta, Tb, C = _svd(lib, prec, C, 1e-4, r_max=56)
+    assert Ta.shape[1] == 56
+    P = Tb / np.linalg.norm(Tb, axis=0)
+    G = np.abs(P.conj().T @ P - np.eye(56))
+    tol = 2 * (4e-7 if prec == 32 else 1e-15) + 60 * u
+    assert G.max() < tol, (G.max(), tol)
