@@ -22,8 +22,8 @@
 // is truncated once, in its final form.  Blocks whose core would not fit (large blocks
 // in complex128) are recompressed after every depth that changed them.  A small block whose factors have at least as
 // many columns as rows takes the dense path: its core is the block itself, C = F_a F_b^t,
-// and its new factors come straight from the SVD of C (no QR).  QR is classical
-// Gram-Schmidt with re-orthogonalisation; the SVD is a column-pivoted Gram-Schmidt down to
+// and its new factors come straight from the SVD of C (no QR).  QR is modified
+// Gram-Schmidt, repeated for columns that lose most of themselves; the SVD is a column-pivoted Gram-Schmidt down to
 // the numerical rank followed by one-sided (Hestenes) Jacobi on what remains.
 // The leaf inverses are computed in FP64 with partial pivoting in both precisions.
 #include <algorithm>
@@ -793,11 +793,18 @@ template <typename R> __host__ __device__ constexpr int group_lanes() { return s
 // written out (qmode = 0).  R is row-major with leading dimension cap(u).
 // Every step updates all later columns (a warp per column, the new norm with the update), so
 // a step costs one barrier; classical Gram-Schmidt with its two passes took ten, 3.6 us a
-// column (the launch at n = 511: 316 us, now 53; n = 150 in complex128: 931, now 253).  F = Q R holds to rounding; Q is orthogonal
-// to rounding over the relative size of a column's remainder, which is all the SVD of the
-// core asks of it (a skew of a column near the drop threshold moves the singular values
-// compared with eps_H by as much, not the product).  When F_u fits the kernel's shared
-// memory (qs_entries) the columns stay there.
+// column (the launch at n = 511: 316 us, now 53; n = 150 in complex128: 931, now 253).  A column
+// of which less than kReorth is left when its turn comes is orthogonalised once more against all
+// Q columns before it (two barriers).  Without that the skews compound: each column takes over
+// those of the columns subtracted from it, enlarged by what it lost, and cosines of 0.05 to 0.8
+// were reached on columns with remainders of a tenth each.  F = Q R holds to rounding either way;
+// the singular values of the core are those of the block only as far as Q is orthogonal.  When F_u
+// fits the kernel's shared memory (qs_entries) the columns stay there.
+constexpr float kReorth = 0.5f;
+// bytes of the tables in front of the columns
+template <typename R> __host__ __device__ constexpr size_t qr_tables(int wcap) {
+  return ((size_t)wcap * (3 * sizeof(R) + sizeof(Cx<R>) + sizeof(int)) + 15) & ~size_t(15);
+}
 template <typename R>
 __global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, const int* __restrict__ G_rank,
                                                Cx<R>* __restrict__ Rb, int* __restrict__ qcols, int* __restrict__ qmode,
@@ -817,12 +824,14 @@ __global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, c
     return;
   }
   const int wcap = g.cap_max;
-  R* cur = reinterpret_cast<R*>(sm);                       // [wcap] squared norm of a column's remainder
+  Cx<R>* co = reinterpret_cast<Cx<R>*>(sm);                // [wcap] coefficients of a second pass
+  R* cur = reinterpret_cast<R*>(co + wcap);                // [wcap] squared norm of a column's remainder
   R* org = cur + wcap;                                     // [wcap] and of the column itself
-  int* pos = reinterpret_cast<int*>(org + wcap);           // [wcap] Q column of a kept column, or -1
-  const size_t qs_off = ((size_t)wcap * (2 * sizeof(R) + sizeof(int)) + 15) & ~size_t(15);
+  R* rn = org + wcap;                                      // [wcap] 1 / norm of a Q column's source
+  int* src = reinterpret_cast<int*>(rn + wcap);            // [wcap] and that source
+  __shared__ R red[32];
   const bool qsh = (long long)s * w <= qs_entries;
-  Cx<R>* Fq = qsh ? reinterpret_cast<Cx<R>*>(sm + qs_off) : F;   // the columns being orthogonalised
+  Cx<R>* Fq = qsh ? reinterpret_cast<Cx<R>*>(sm + qr_tables<R>(wcap)) : F;   // the columns being orthogonalised
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int rows = min(s, ld);
   for (int e = threadIdx.x; e < rows * w; e += blockDim.x) Rm[(long long)(e / w) * ld + e % w] = Cx<R>(0, 0);
@@ -840,8 +849,45 @@ __global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, c
   constexpr int kGL = group_lanes<R>(), kCPW = 32 / kGL;
   int qc = 0;
   for (int j = 0; j < w; ++j) {
-    const R nr = cur[j];
-    const bool kept = nr > Tiny<R>::dep * Tiny<R>::dep * org[j] && nr > 0 && qc < rows;
+    R nr = cur[j];
+    bool kept = nr > Tiny<R>::dep * Tiny<R>::dep * org[j] && nr > 0 && qc < rows;
+    if (kept && qc > 0 && nr < R(kReorth * kReorth) * org[j]) {
+      Cx<R>* cj = Fq + (long long)j * s;
+      for (int kb = warp * kCPW; kb < qc; kb += nw * kCPW) {
+        const int k = kb + lane / kGL, gl = lane % kGL;
+        const bool act = k < qc;
+        const Cx<R>* ck = Fq + (long long)src[act ? k : 0] * s;
+        Cx<R> d(0, 0);
+        if (act)
+          for (int i = gl; i < s; i += kGL) cfma_conj(d, ck[i], cj[i]);
+        for (int o = kGL / 2; o > 0; o >>= 1) d += shfl_xor(d, o);
+        if (act && gl == 0) {
+          d = rn[k] * d;
+          co[k] = -(rn[k] * d);
+          Rm[(long long)k * ld + j] += d;
+        }
+      }
+      __syncthreads();
+      // four rows a warp, the columns over eight lanes
+      R part = 0;
+      for (int i0 = 4 * warp; i0 < s; i0 += 4 * nw) {
+        const int i = i0 + lane / 8;
+        Cx<R> v(0, 0);
+        if (i < s)
+          for (int k = lane % 8; k < qc; k += 8) cfma(v, co[k], Fq[(long long)src[k] * s + i]);
+        for (int o = 4; o > 0; o >>= 1) v += shfl_xor(v, o);
+        if (i < s && lane % 8 == 0) {
+          v += cj[i];
+          cj[i] = v;
+          part += abs2(v);
+        }
+      }
+      for (int o = 8; o < 32; o <<= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+      if (lane == 0) red[warp] = part;
+      __syncthreads();
+      nr = warp_sum_r(lane < nw ? red[lane] : R(0));
+      kept = nr > Tiny<R>::dep * Tiny<R>::dep * org[j] && nr > 0;
+    }
     if (kept) {
       const R inv = rcp_any(nr), rs = rsqrt_any(nr), nn = nr * rs;
       const Cx<R>* cj = Fq + (long long)j * s;
@@ -868,17 +914,19 @@ __global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, c
           Rm[(long long)qc * ld + l] = rs * d;
         }
       }
-      if (threadIdx.x == 0) Rm[(long long)qc * ld + j] = Cx<R>(nn, 0);
+      if (threadIdx.x == 0) {
+        Rm[(long long)qc * ld + j] = Cx<R>(nn, 0);
+        src[qc] = j;
+        rn[qc] = rs;
+      }
+      ++qc;
     }
-    if (threadIdx.x == 0) pos[j] = kept ? qc : -1;
-    if (kept) ++qc;
     __syncthreads();
   }
   // the kept columns, normalised, to the front (a Q column never lies behind its source)
-  for (int j = 0; j < w; ++j) {
-    const int c = pos[j];
-    if (c < 0) continue;
-    const R rs = rsqrt_any(cur[j]);
+  for (int c = 0; c < qc; ++c) {
+    const int j = src[c];
+    const R rs = rn[c];
     for (int i = threadIdx.x; i < s; i += blockDim.x) F[(long long)c * s + i] = rs * Fq[(long long)j * s + i];
     if (!qsh) __syncthreads();
   }
@@ -1640,7 +1688,7 @@ static int factor_impl(hsweep_s* h) {
   const int L = h->L, nn = h->nnodes, KCAP = w->KCAP, QCAP = w->QCAP;
   const size_t core_smem = (size_t)(2 * KCAP) * (2 * KCAP) * es + 32 * sizeof(R) + (2 * KCAP + 1) * sizeof(int) + 16;
   // QR: norms and positions, then as many entries of F_u as fit (226 KB in all)
-  const size_t qr_base = ((size_t)g.cap_max * (2 * sizeof(R) + sizeof(int)) + 15) & ~size_t(15);
+  const size_t qr_base = qr_tables<R>(g.cap_max);
   const int qs_entries = qr_base < 226 * 1024 ? (int)((226 * 1024 - qr_base) / es) : 0;
   const size_t qr_smem = qr_base + (size_t)qs_entries * es;
   const SvdPlan<R> svd(QCAP, h->eps_H);

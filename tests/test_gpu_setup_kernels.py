@@ -104,3 +104,41 @@ def test_svd_columns_of_a_cluster_are_orthogonal(lib, prec, spread):
     G = np.abs(P.conj().T @ P - np.eye(56))
     tol = 2 * (4e-7 if prec == 32 else 1e-15) + 60 * u
     assert G.max() < tol, (G.max(), tol)
+
+
+def _qr(lib, prec, F, qsh):
+    ct, _ = _types(prec)
+    s, w = F.shape
+    Fq = np.asfortranarray(F.astype(ct))
+    Rm, qc = np.zeros((w, w), ct), ctypes.c_int(-1)
+    fn = lib.qr_f32 if prec == 32 else lib.qr_f64
+    F0 = np.array(Fq, dtype=complex)
+    rc = fn(s, w, int(qsh), Fq.ctypes.data_as(ctypes.c_void_p), Rm.ctypes.data_as(ctypes.c_void_p), ctypes.byref(qc))
+    assert rc == 0, rc
+    return F0, Fq[:, :qc.value].astype(complex), Rm[:qc.value].astype(complex)
+
+
+# remainders of the columns down to near the drop threshold (2e-6, 1e-13), and below it
+@pytest.mark.parametrize("prec,least", [(32, 1e-1), (32, 5e-6), (32, 1e-9), (64, 1e-1), (64, 5e-13), (64, 1e-18)])
+@pytest.mark.parametrize("s,w,qsh", [(9, 3, True), (130, 57, True), (256, 98, True), (130, 57, False), (512, 49, False)])
+def test_qr_is_orthogonal_also_for_columns_with_small_remainders(lib, prec, least, s, w, qsh):
+    _, u = _types(prec)
+    if qsh and s * w * (8 if prec == 32 else 16) > 220 * 1024:
+        qsh = False
+    rng = np.random.default_rng(s + w)
+    B = _unitary(rng, s, w)
+    F = np.empty((s, w), complex)
+    for j in range(w):
+        v = B[:, :j] @ (rng.standard_normal(j) + 1j * rng.standard_normal(j)) if j else B[:, 0]
+        F[:, j] = (v / np.linalg.norm(v) + np.exp(rng.uniform(np.log(least), 0)) * B[:, j]) * np.exp(rng.uniform(-3, 3))
+    F, Q, R = _qr(lib, prec, F, qsh)
+    # a column keeps at least half of itself in its last pass: 2 u for each rounding, a few of them,
+    # from up to w updates added at random, and as much again a few times over from the columns before
+    tol = 2 * u * 3 * np.sqrt(w) * 5
+    assert np.abs(Q.conj().T @ Q - np.eye(Q.shape[1])).max() < tol
+    # rounding of w updates, and the dropped remainders
+    drop = 4e-6 if prec == 32 else 2e-13
+    err = np.linalg.norm(F - Q @ R, axis=0) / np.linalg.norm(F, axis=0)
+    assert err.max() < 4 * np.sqrt(w) * u + (drop if Q.shape[1] < w else 0)
+    if least > drop:
+        assert Q.shape[1] == w
