@@ -60,8 +60,8 @@ __host__ __device__ void hsw_philox4x32_10(const uint32_t ctr[4], const uint32_t
 namespace {
 
 // Two complex standard normals (real and imaginary parts independent N(0, 1)) from one
-// Philox block, by the Box-Muller transform, in the precision that stores them (the FP64
-// logarithms and sines took longer than the products with the test vectors).
+// Philox block, by the Box-Muller transform in FP64: the stored vectors are those of
+// hsweep_rsvd_normals, rounded.
 template <typename R>
 __device__ inline void gauss2(uint32_t row, uint32_t pair, uint32_t blk, uint32_t m, uint32_t seed, Cx<R>& z0,
                               Cx<R>& z1) {
@@ -69,20 +69,15 @@ __device__ inline void gauss2(uint32_t row, uint32_t pair, uint32_t blk, uint32_
   const uint32_t key[2] = {seed, 0x5EEDu};
   uint32_t x[4];
   hsw_philox4x32_10(ctr, key, x);
-  const R s = R(2.3283064365386963e-10);   // 2^-32
-  const R u0 = (R(x[0]) + R(0.5)) * s, u1 = R(x[1]) * s;
-  const R u2 = (R(x[2]) + R(0.5)) * s, u3 = R(x[3]) * s;
-  const R r0 = sqrt(R(-2) * log(u0)), r1 = sqrt(R(-2) * log(u2));
-  R s0, c0, s1, c1;
-  if constexpr (sizeof(R) == 4) {
-    sincospif(2.0f * u1, &s0, &c0);
-    sincospif(2.0f * u3, &s1, &c1);
-  } else {
-    sincospi(2.0 * u1, &s0, &c0);
-    sincospi(2.0 * u3, &s1, &c1);
-  }
-  z0 = Cx<R>(r0 * c0, r0 * s0);
-  z1 = Cx<R>(r1 * c1, r1 * s1);
+  const double s = 2.3283064365386963e-10;   // 2^-32
+  const double u0 = ((double)x[0] + 0.5) * s, u1 = (double)x[1] * s;
+  const double u2 = ((double)x[2] + 0.5) * s, u3 = (double)x[3] * s;
+  const double r0 = sqrt(-2.0 * log(u0)), r1 = sqrt(-2.0 * log(u2));
+  double s0, c0, s1, c1;
+  sincospi(2.0 * u1, &s0, &c0);
+  sincospi(2.0 * u3, &s1, &c1);
+  z0 = Cx<R>(R(r0 * c0), R(r0 * s0));
+  z1 = Cx<R>(R(r1 * c1), R(r1 * s1));
 }
 
 struct FarArgs {
@@ -94,6 +89,21 @@ struct FarArgs {
   const int* sz;            // node sizes
   int shared;               // the scratch of every block fits in dynamic shared memory
 };
+
+// Omega of every block, complex Gaussian test vectors (sw x P, column-major) into its scratch: the
+// FP64 logarithms and sines of the largest block take one SM longer than the block's products, so
+// they are spread over the GPU first.
+template <typename R>
+__global__ void __launch_bounds__(128) strong_normals(FarArgs fa, int m, Cx<R>* __restrict__ scratch) {
+  const int bi = blockIdx.x, sw = fa.info[8 * bi + 5], e = blockIdx.y * blockDim.x + threadIdx.x;
+  if (e >= sw * (fa.P / 2)) return;
+  const int row = e % sw, pr = e / sw;
+  Cx<R> z0, z1;
+  gauss2<R>((uint32_t)row, (uint32_t)pr, (uint32_t)bi, (uint32_t)m, fa.seed, z0, z1);
+  Cx<R>* Om = scratch + fa.soff[bi];
+  Om[(2 * pr) * sw + row] = z0;
+  Om[(2 * pr + 1) * sw + row] = z1;
+}
 
 // Z[p][c] (ld kKMax) = sum_r F[r, c] v_p[r] (CONJ: conj(v_p[r])), c < k, p < np: a warp per
 // column c and eight vectors
@@ -154,7 +164,7 @@ __device__ __forceinline__ void rows_times(const Cx<R>* __restrict__ F, int ldf,
 // latency of these short chains; with classical Gram-Schmidt (a block-wide sum per inner
 // product) and FP64 Jacobi on the Gram matrix by one warp a layer at n = 255 took 931 us, now 71.
 template <typename R>
-__global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, int m, R eps, const Cx<R>* __restrict__ F,
+__global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, R eps, const Cx<R>* __restrict__ F,
                                                        const int* __restrict__ rank, Cx<R>* __restrict__ Fout,
                                                        Cx<R>* __restrict__ scratch) {
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -176,15 +186,11 @@ __global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, int m, R eps,
   Cx<R>* Om = fa.shared ? reinterpret_cast<Cx<R>*>(dyn) : scratch + fa.soff[bi];   // sw x P (Omega, later Bt)
   Cx<R>* Y = Om + sw * P;                                                            // su x P (Y, then Q)
 
-  // Omega: complex Gaussian test vectors
-  for (int e = tid; e < sw * (P / 2); e += blockDim.x) {
-    const int row = e % sw, pr = e / sw;
-    Cx<R> z0, z1;
-    gauss2<R>((uint32_t)row, (uint32_t)pr, (uint32_t)bi, (uint32_t)m, fa.seed, z0, z1);
-    Om[(2 * pr) * sw + row] = z0;
-    Om[(2 * pr + 1) * sw + row] = z1;
+  if (fa.shared) {
+    const Cx<R>* src = scratch + fa.soff[bi];
+    for (int e = tid; e < sw * P; e += blockDim.x) Om[e] = src[e];
+    __syncthreads();
   }
-  __syncthreads();
   // Y = S Omega = F_a[rows u] (F_b[rows w]^t Omega)
   columns_dot<false>(Fb, ldb, k, Om, sw, P, Z);
   __syncthreads();
@@ -394,6 +400,7 @@ int depth_of_host(int v) { int d = 0; while (v > 1) { v >>= 1; ++d; } return d; 
 
 struct StrongWork {
   int nfar = 0, nnear = 0, P = 0;
+  int ngrid = 0;                // CTAs of strong_normals per block
   int* d_far = nullptr;
   long long* d_soff = nullptr;
   int* d_near = nullptr;
@@ -453,6 +460,7 @@ static int strong_prepare(hsweep_s* h, size_t es) {
   for (size_t i = 0; i < far.size(); i += 8) {
     most = std::max(most, (size_t)(far[i + 4] + far[i + 5]) * s->P * es);
     soff.push_back(so);
+    s->ngrid = std::max(s->ngrid, (far[i + 5] * (s->P / 2) + 127) / 128);
     so += (long long)(far[i + 4] + far[i + 5]) * s->P;
   }
   // (Z and the tables take up to 15 KB of static shared memory beside it)
@@ -503,8 +511,9 @@ static int project_impl(hsweep_s* h, int m, const Cx<R>* G_F, int* G_rank, Cx<R>
     fa.shared = s->smem > 0;
     if (s->smem > 0)
       HSW_CUDA(cudaFuncSetAttribute(strong_far<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->smem));
-    strong_far<R><<<s->nfar, kThreads, s->smem, st>>>(fa, m, (R)h->eps_H, G_F, G_rank, G_F2, (Cx<R>*)s->scratch);
-    h->nlaunch += 1;
+    strong_normals<R><<<dim3(s->nfar, s->ngrid), 128, 0, st>>>(fa, m, (Cx<R>*)s->scratch);
+    strong_far<R><<<s->nfar, kThreads, s->smem, st>>>(fa, (R)h->eps_H, G_F, G_rank, G_F2, (Cx<R>*)s->scratch);
+    h->nlaunch += 2;
   }
   if (s->nnear > 0) {
     NearArgs na;

@@ -1,23 +1,9 @@
-// C entry points that launch single kernels of csrc/setup.cu and device helpers of csrc/common.cuh on
-// the caller's data (host arrays), for tests/test_gpu_setup_kernels.py.
+// C entry points that launch single kernels of csrc/setup.cu on the caller's data (host arrays), for tests/test_gpu_setup_kernels.py.
 #include "../../paper_1007_4290_gb300/csrc/setup.cu"
 
-#define ENTRY extern "C" __attribute__((visibility("default"))) int
+#include "dev.cuh"
 
 namespace {
-
-template <typename T>
-struct Dev {
-  T* p = nullptr;
-  size_t n;
-  explicit Dev(size_t n_, const T* src = nullptr) : n(n_) {
-    if (cudaMalloc(&p, n * sizeof(T)) != cudaSuccess) p = nullptr;
-    if (p && src) cudaMemcpy(p, src, n * sizeof(T), cudaMemcpyHostToDevice);
-    else if (p) cudaMemset(p, 0, n * sizeof(T));
-  }
-  ~Dev() { cudaFree(p); }
-  bool get(T* dst) { return cudaMemcpy(dst, p, n * sizeof(T), cudaMemcpyDeviceToHost) == cudaSuccess; }
-};
 
 // the truncated SVD of one core C (qa x qb, column-major): T_a (ld qcap, r_max columns), T_b, rank
 template <typename R>

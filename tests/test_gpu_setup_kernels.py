@@ -1,34 +1,20 @@
 """Single kernels of the setup on constructed inputs, against NumPy in complex128: launched through
 tests/kernels/setup_entries.cu, which is compiled with the library's own flags and objects."""
 import ctypes
-import glob
-import os
-import subprocess
 
 import numpy as np
 import pytest
-import torch
+
+from tests.kernels import kernel_library
 
 pytestmark = pytest.mark.gpu
 
-HERE = os.path.dirname(os.path.abspath(__file__))
 U32, U64 = 2.0 ** -24, 2.0 ** -53
 
 
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
-    import __graft_entry__ as g
-    b = g._build_module()
-    objs = os.path.join(b.HERE, "_build")
-    if not os.path.exists(os.path.join(objs, "setup.o")):
-        b.build()
-    out = str(tmp_path_factory.mktemp("kernels") / "entries.so")
-    rest = [o for o in sorted(glob.glob(os.path.join(objs, "*.o"))) if os.path.basename(o) != "setup.o"]
-    cmd = [b.nvcc(), *b.ARCH, *b.FLAGS, "-shared", "-o", out, os.path.join(HERE, "kernels", "setup_entries.cu"), *rest, "-ldl"]
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    assert r.returncode == 0, r.stderr
-    torch.zeros(1, device="cuda")
-    return ctypes.CDLL(out)
+    return kernel_library(tmp_path_factory, "setup")
 
 
 def _types(prec):
