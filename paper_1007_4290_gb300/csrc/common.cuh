@@ -182,6 +182,15 @@ struct JacobiRotation {
   Cx<R> gn;
 };
 
+// One-sided Jacobi ends after a sweep whose cosines were all small (1e-4 in complex64, 1e-8 in
+// complex128), if its rotations cannot have left more than the orthogonality tolerance: a rotation
+// by tan t mixes the other inner products of its two columns, so up to t times the largest cosine
+// is left, t being small between well-separated singular values (the quadratic convergence) but
+// not within a cluster.  gg: the largest squared cosine, t: the largest tangent, tol2: the squared tolerance.
+__device__ __forceinline__ bool rotations_done(float gg, float t, float tol2) {
+  return t * sqrtf(gg) <= 2.0f * sqrtf(tol2);
+}
+
 // L2-only loads/stores for data exchanged between CTAs of one sweep team.
 template <typename R> __device__ __forceinline__ Cx<R> ld_cg(const Cx<R>* p);
 template <> __device__ __forceinline__ Cx<float> ld_cg(const Cx<float>* p) {

@@ -1092,14 +1092,6 @@ __global__ void __launch_bounds__(256) core_product_tc(Geo g, const Cx<float>* _
   }
 }
 
-// One-sided Jacobi ends after a sweep whose cosines were at most sqrt(quad), if the rotations
-// cannot have left more than the orthogonality tolerance: a rotation by tan t mixes the other
-// inner products of its two columns, so up to t times the largest cosine is left, t being small
-// between well-separated singular values (the quadratic convergence) but not within a cluster.
-template <typename R> __device__ __forceinline__ bool rotations_done(float gg, float t) {
-  return t * sqrtf(gg) <= 2.0f * sqrtf(Tiny<R>::jac2);
-}
-
 // Shuffle-sum within aligned groups of GW lanes (GW = 16 or 32).
 template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW) {
   for (int o = GW >> 1; o > 0; o >>= 1) v += shfl_xor(v, o);
@@ -1342,7 +1334,7 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
       }
       __syncthreads();
     }
-    if (s_rot == 0 && rotations_done<R>(__int_as_float(s_gg), __int_as_float(s_t))) break;
+    if (s_rot == 0 && rotations_done(__int_as_float(s_gg), __int_as_float(s_t), Tiny<R>::jac2)) break;
   }
   // singular values, ordering, truncation
   for (int j = warp; j < kq; j += nw) {

@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, R eps, const 
   __shared__ Cx<R> Z[kKMax * kPMax];
   __shared__ R cur[kPMax], org[kPMax], sig[kPMax];
   __shared__ int kept[kPMax], order[kPMax];
-  __shared__ int s_rot, s_keep;
+  __shared__ int s_rot, s_gg, s_t, s_keep;
 
   const int bi = blockIdx.x;
   const int* inf = fa.info + 8 * bi;
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, R eps, const 
   const int me = q + (q & 1);
   for (int sweep = 0; sweep < 30; ++sweep) {
     __syncthreads();
-    if (tid == 0) s_rot = 0;
+    if (tid == 0) s_rot = s_gg = s_t = 0;
     __syncthreads();
     for (int round = 0; round < me - 1; ++round) {
       for (int pr = warp; pr < me / 2; pr += nw) {
@@ -309,7 +309,14 @@ __global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, R eps, const 
         JacobiRotation<R> rot;
         if (!rot.needed(al, be, ga, tol2)) continue;
         rot.angle(al, be);
-        if (lane == 0 && rot.gg > quad) s_rot = 1;
+        if (lane == 0) {
+          if (rot.gg > quad) {
+            s_rot = 1;
+          } else {
+            atomicMax(&s_gg, __float_as_int(rot.gg));
+            atomicMax(&s_t, __float_as_int(fabsf(rot.t)));
+          }
+        }
         for (int r = lane; r < sw; r += 32) {
           const Cx<R> x = cp[r], y = cq[r];
           Cx<R> nx = rot.cs * x, ny = rot.cs * y;
@@ -321,7 +328,7 @@ __global__ void __launch_bounds__(kThreads) strong_far(FarArgs fa, R eps, const 
       }
       __syncthreads();
     }
-    if (s_rot == 0) break;
+    if (s_rot == 0 && rotations_done(__int_as_float(s_gg), __int_as_float(s_t), tol2)) break;
   }
   for (int j = warp; j < q; j += nw) {
     R acc = 0;

@@ -40,3 +40,32 @@ def test_test_vectors_are_the_library_s_normals_rounded(lib, P, m, seed):
     assert np.abs(d64 - host).max() < 40 * U64 * 6
     for a, b in ((d32.real, d64.real), (d32.imag, d64.imag)):
         assert np.array_equal(a, b.astype(np.float32))
+
+
+def _far(lib, prec, Fa, Fb, R, eps, shared):
+    ct = np.complex64 if prec == 32 else np.complex128
+    (su, k), sw = Fa.shape, Fb.shape[0]
+    Fa, Fb = Fa.astype(ct), Fb.astype(ct)
+    F = np.concatenate([Fa.T.reshape(-1), Fb.T.reshape(-1)])
+    O = np.zeros((su + sw) * R, ct)
+    fn = lib.far_f32 if prec == 32 else lib.far_f64
+    rc = fn(su, sw, k, R, ctypes.c_double(eps), int(shared), _p(F), _p(O))
+    assert rc == 0, rc
+    O = O.astype(complex)
+    return (Fa.astype(complex) @ Fb.astype(complex).T, O[:su * R].reshape(R, su).T, O[su * R:].reshape(R, sw).T)
+
+
+# a block of exact rank R whose singular values form a cluster: the projection is the block itself, as
+# far as the right factor's columns are orthogonal (the rotations' tolerance, twice, and their rounding)
+@pytest.mark.parametrize("prec,spread", [(32, 1e-4), (32, 1e-3), (32, 0.0), (64, 1e-8), (64, 1e-4), (64, 0.0)])
+@pytest.mark.parametrize("su,sw,R,shared", [(16, 17, 8, True), (64, 60, 8, True), (128, 128, 7, False)])
+def test_projection_of_a_cluster_is_the_block(lib, prec, spread, su, sw, R, shared):
+    u = U32 if prec == 32 else U64
+    rng = np.random.default_rng(su + R)
+    q = [np.linalg.qr(rng.standard_normal((n, R)) + 1j * rng.standard_normal((n, R)))[0] for n in (su, sw)]
+    s = 1 + spread * rng.standard_normal(R)
+    S, A, B = _far(lib, prec, q[0] * s, q[1], R, 1e-9 if prec == 64 else 1e-6, shared)
+    P = B / np.linalg.norm(B, axis=0)
+    tol = 2 * (4e-7 if prec == 32 else 1e-15) + 60 * u
+    assert np.abs(P.conj().T @ P - np.eye(R)).max() < tol
+    assert np.linalg.norm(S - A @ B.T, 2) < R * tol
