@@ -1,5 +1,6 @@
 // Internal state of an hsweep handle, shared by the translation units of the library.
 #pragma once
+#include <atomic>
 #include <array>
 #include <utility>
 #include <vector>

@@ -33,7 +33,6 @@
 // b = sum (Im f) x, f x = (Re a - Im b, Im a + Re b).
 #include <cstdlib>
 #include <type_traits>
-#include <atomic>
 #include "handle.h"
 #include "sweep_common.cuh"
 #include "tma.cuh"
