@@ -79,33 +79,27 @@ template <int G> struct Tile<double, G> {
 };
 constexpr int kKW = 16;       // columns per chunk, in both precisions
 
-// acc += f x for B right-hand sides.  With four or more the paired FP32 instruction pays:
-// f (Re, Re), (Im, Im) against x and x' = (-Im x, Re x); below, the pairs cost as many moves
-// as they save.
-template <typename R, int B> struct TMac {
-  typedef Cx<R> F, X;
-  typedef Cx<R> A;
-  static __device__ __forceinline__ F f(Cx<R> v) { return v; }
-  static __device__ __forceinline__ void mac(A (&s)[B], const F& f, const X (&x)[B]) {
+// acc += f x for B right-hand sides (in pairs, the FP32 instruction on two values costs as many
+// moves as it saves), and their B values of a row
+template <typename R, int B>
+__device__ __forceinline__ void mac(Cx<R> (&s)[B], Cx<R> f, const Cx<R> (&x)[B]) {
 #pragma unroll
-    for (int g = 0; g < B; ++g) cfma(s[g], f, x[g]);
-  }
-  static __device__ __forceinline__ void load(const Cx<R>* p, X (&x)[B]) {
-    if constexpr (sizeof(R) == 4 && B % 2 == 0) {
+  for (int g = 0; g < B; ++g) cfma(s[g], f, x[g]);
+}
+template <typename R, int B>
+__device__ __forceinline__ void load_rhs(const Cx<R>* p, Cx<R> (&x)[B]) {
+  if constexpr (sizeof(R) == 4 && B % 2 == 0) {
 #pragma unroll
-      for (int g = 0; g < B; g += 2) {
-        const float4 v = *reinterpret_cast<const float4*>(p + g);
-        x[g] = Cx<R>(v.x, v.y);
-        x[g + 1] = Cx<R>(v.z, v.w);
-      }
-    } else {
-#pragma unroll
-      for (int g = 0; g < B; ++g) x[g] = p[g];
+    for (int g = 0; g < B; g += 2) {
+      const float4 v = *reinterpret_cast<const float4*>(p + g);
+      x[g] = Cx<R>(v.x, v.y);
+      x[g + 1] = Cx<R>(v.z, v.w);
     }
+  } else {
+#pragma unroll
+    for (int g = 0; g < B; ++g) x[g] = p[g];
   }
-  static __device__ __forceinline__ Cx<R> get(const A& s) { return s; }
-  static __device__ __forceinline__ A zero() { return Cx<R>(0, 0); }
-};
+}
 // entries per row of F (or D) for w columns: a multiple of 8, odd in units of 64 bytes, so
 // that the rows of a warp's access fall into different banks
 template <typename R>
@@ -144,31 +138,14 @@ __device__ __forceinline__ void send2(unsigned addr, Cx<float> v, Cx<float> w, u
                : "memory");
 }
 
-__device__ __forceinline__ void send2(unsigned addr, Cx<double> v, Cx<double> w, unsigned bar) {
-  send(addr, v, bar);
-  send(addr + 16, w, bar);
+// two tagged words (16 bytes); teams exchange through L2 in complex64 only
+__device__ __forceinline__ void load_words(const Tagged<float>::W* p, Tagged<float>::W (&w)[2]) {
+  const ulonglong2 t = __ldcg(reinterpret_cast<const ulonglong2*>(p));
+  w[0] = t.x;
+  w[1] = t.y;
 }
-
-// V tagged words (16 bytes)
-template <typename R, int V>
-__device__ __forceinline__ void load_words(const typename Tagged<R>::W* p, typename Tagged<R>::W (&w)[V]) {
-  if constexpr (V == 2) {
-    const ulonglong2 t = __ldcg(reinterpret_cast<const ulonglong2*>(p));
-    w[0] = t.x;
-    w[1] = t.y;
-  } else {
-    w[0] = Tagged<R>::load(p);
-  }
-}
-
-template <typename R>
-__device__ __forceinline__ void store_words(typename Tagged<R>::W* p, typename Tagged<R>::W w0, typename Tagged<R>::W w1) {
-  if constexpr (sizeof(R) == 4) {
-    __stcg(reinterpret_cast<ulonglong2*>(p), make_ulonglong2(w0, w1));
-  } else {
-    Tagged<R>::store(p, w0);
-    Tagged<R>::store(p + 1, w1);
-  }
+__device__ __forceinline__ void store_words(Tagged<float>::W* p, Tagged<float>::W w0, Tagged<float>::W w1) {
+  __stcg(reinterpret_cast<ulonglong2*>(p), make_ulonglong2(w0, w1));
 }
 
 template <typename R>
@@ -197,7 +174,6 @@ __global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_ke
   constexpr int GS = vstride<R>(G);
   using TL = Tile<R, G>;
   constexpr int A = TL::A, CL = TL::CL, B = TL::B, GL = G / B, RL = 32 / (CL * GL), KW = kKW;
-  using M = TMac<R, B>;
   constexpr int NW = NT / 32;
   constexpr int RG = 32 / (CS * GL);      // step 4: row groups per warp, RA rows each
   constexpr int VG = (sizeof(R) == 4 && G % 2 == 0) ? 2 : 1;    // right-hand sides per 16-byte word
@@ -366,11 +342,11 @@ __global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_ke
     // for the columns below kend
     auto chunk = [&](const Cx<R>* mat, int st, int k0, auto put) {
       const int cl = lane % CL, gl = (lane / CL) % GL, rl = lane / (CL * GL);
-      typename M::A acc[A][B];
+      Cx<R> acc[A][B];
 #pragma unroll
       for (int u = 0; u < A; ++u)
 #pragma unroll
-        for (int g = 0; g < B; ++g) acc[u][g] = M::zero();
+        for (int g = 0; g < B; ++g) acc[u][g] = Cx<R>(0, 0);
       const Cx<R>* bp = mat + rl * st + k0 + (A == 4 ? 2 * cl : cl);
       const Cx<R>* xp = x + rl * GS + gl * B;
 #pragma unroll (G <= 2 ? 4 : 2)
@@ -385,16 +361,16 @@ __global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_ke
         } else {
           f[0] = *bp;
         }
-        typename M::X xv[B];
-        M::load(xp, xv);
+        Cx<R> xv[B];
+        load_rhs(xp, xv);
 #pragma unroll
-        for (int u = 0; u < A; ++u) M::mac(acc[u], M::f(f[u]), xv);
+        for (int u = 0; u < A; ++u) mac(acc[u], f[u], xv);
       }
       Cx<R> o[A * B];
 #pragma unroll
       for (int u = 0; u < A; ++u)
 #pragma unroll
-        for (int g = 0; g < B; ++g) o[u * B + g] = M::get(acc[u][g]);
+        for (int g = 0; g < B; ++g) o[u * B + g] = acc[u][g];
       int idx;
       bool first;
       scatter_sum<R, A * B, RL, CL * GL>(o, lane, idx, first);
@@ -416,22 +392,18 @@ __global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_ke
       // a slot holds this step's value or the one from two steps before, told apart by the tag
       typename T::W* dst = a.xch + (((long long)par * gridDim.x) + blockIdx.x) * a.Wcap * G;
       for (; ci < nFx; ci += NW) {
-        auto put = [&](int k, int g, Cx<R> v0, Cx<R> v1, auto pv) {
+        chunk(F, rs, min(ci, nF - 1) * KW, [&](int kf, int g, Cx<R> v0, Cx<R> v1, auto pv) {
+          static_assert(decltype(pv)::value == 2, "the L2 slots are written in pairs");
+          const int k = kf + (ci - min(ci, nF - 1)) * KW;
           if (k < a.Wcap && (int)blockIdx.x != a.withhold) {
             const bool in = k < W;
-            if constexpr (decltype(pv)::value == 2)
-              store_words<R>(dst + k * G + g, T::pack(in ? v0 : Cx<R>(0, 0), ph), T::pack(in ? v1 : Cx<R>(0, 0), ph));
-            else
-              T::store(dst + k * G + g, T::pack(in ? v0 : Cx<R>(0, 0), ph));
+            store_words(dst + k * G + g, T::pack(in ? v0 : Cx<R>(0, 0), ph), T::pack(in ? v1 : Cx<R>(0, 0), ph));
           }
-        };
-        chunk(F, rs, min(ci, nF - 1) * KW, [&](int k, int g, Cx<R> v0, Cx<R> v1, auto pv) {
-          put(k + (ci - min(ci, nF - 1)) * KW, g, v0, v1, pv);
         });
       }
     } else {
       for (; ci < nF; ci += NW)
-        chunk(F, rs, ci * KW, [&](int k, int g, Cx<R> v0, Cx<R> v1, auto pv) {
+        chunk(F, rs, ci * KW, [&](int k, int g, auto v0, auto v1, auto pv) {
           if (k < W && (int)blockIdx.x != a.withhold) {
             // column k of depth d: to the S CTAs of the sibling subtree, slot (c mod S, k)
             const int d = 1 + (k >= mc.x) + (dC > 1 && k >= mc.y) + (dC > 2 && k >= mc.z);
@@ -504,14 +476,14 @@ __global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_ke
           typename T::W wv[8][VG];
 #pragma unroll
           for (int u = 0; u < 8; ++u)
-            if (u < S) load_words<R, VG>(src + u * cs, wv[u]);
+            if (u < S) load_words(src + u * cs, wv[u]);
           long long spins = 0;
           for (;;) {      // re-read every word not yet written for this step
             bool pending = false;
 #pragma unroll
             for (int u = 0; u < 8; ++u)
               if (u < S && !(T::ok(wv[u][0], ph) && T::ok(wv[u][VG - 1], ph))) {
-                load_words<R, VG>(src + u * cs, wv[u]);
+                load_words(src + u * cs, wv[u]);
                 pending = true;
               }
             if (!pending) break;
@@ -550,11 +522,11 @@ __global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_ke
     {
       if (warp * RG * RA < ns) {
       const int cs = lane % CS;
-      typename M::A acc[RA][B];
+      Cx<R> acc[RA][B];
 #pragma unroll
       for (int u = 0; u < RA; ++u)
 #pragma unroll
-        for (int g = 0; g < B; ++g) acc[u][g] = M::zero();
+        for (int g = 0; g < B; ++g) acc[u][g] = Cx<R>(0, 0);
       {
         const Cx<R>* Fr[RA];
 #pragma unroll
@@ -564,17 +536,17 @@ __global__ void __launch_bounds__(NT, G == 4 && NT == 256 ? 2 : 1) sweep_slab_ke
           Cx<R> f[RA];
 #pragma unroll
           for (int u = 0; u < RA; ++u) f[u] = Fr[u][k];
-          typename M::X v[B];
-          M::load(q + k * GS + gl4 * B, v);
+          Cx<R> v[B];
+          load_rhs(q + k * GS + gl4 * B, v);
 #pragma unroll
-          for (int u = 0; u < RA; ++u) M::mac(acc[u], M::f(f[u]), v);
+          for (int u = 0; u < RA; ++u) mac(acc[u], f[u], v);
         }
       }
       Cx<R> o[RA * B];
 #pragma unroll
       for (int u = 0; u < RA; ++u)
 #pragma unroll
-        for (int g = 0; g < B; ++g) o[u * B + g] = M::get(acc[u][g]);
+        for (int g = 0; g < B; ++g) o[u * B + g] = acc[u][g];
       int idx;
       bool first;
       scatter_sum<R, RA * B, CS, 1>(o, lane, idx, first);
@@ -747,7 +719,7 @@ static SlabKernel<R> slab_kernel_g(int rows) {
     if (rows <= 32) return sweep_slab_kernel<float, G, 2 * 512 / NT, CS, NT, L2X>;
     return sweep_slab_kernel<float, G, 4 * 512 / NT64, CS, NT64, L2X>;
   } else {
-    // four warps, one a sub-core, whatever the slab: the FP64 unit is the bound, and fewer
+    // eight warps, two a sub-core, whatever the slab: the FP64 unit is the bound, and fewer
     // lanes a row mean fewer additions to join them
     if (rows <= 8) return sweep_slab_kernel<double, G, 1, 16, 256, L2X>;
     if (rows <= 16) return sweep_slab_kernel<double, G, 1, 8, 256, L2X>;
