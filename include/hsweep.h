@@ -205,8 +205,8 @@ HSWEEP_API int hsweep_strong_export(hsweep_t h, int m, hsw_c128* records, long l
  * width eta = pml_width * h on all four sides) and run the setup sweep of
  * Algorithm 2.5: for m = 1..n, S~_m from T~_{m-1} (hdiagmul + hsub), T~_m = hinv(S~_m).
  * Off-diagonal blocks keep the singular values above eps_H times the block's largest
- * one (at most r_max of them; in HSWEEP_MIXED one within 15 % of that threshold may go either
- * way); eps_H = 0 keeps every one up to r_max, down to the rounding noise of the arithmetic
+ * one (at most r_max of them; in HSWEEP_MIXED one within a third of that threshold may go
+ * either way); eps_H = 0 keeps every one up to r_max, down to the rounding noise of the arithmetic
  * (about 1e-7 of the block's norm in HSWEEP_MIXED, 1e-14 in HSWEEP_FP64).
  *   c_dev      device, n*n doubles, node layout as above; every value finite and > 0
  *   omega      > 0;  n >= 3;  0 <= pml_width < n/2;  eps_H >= 0

@@ -27,6 +27,7 @@
 // the numerical rank followed by one-sided (Hestenes) Jacobi on what remains.
 // The leaf inverses are computed in FP64 with partial pivoting in both precisions.
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <utility>
 #include "handle.h"
@@ -62,9 +63,10 @@ template <> struct Tiny<float> {
 //   thr: columns with smaller squared norms (relative to the largest column's) are not rotated.
 //   rem: the pivoted Gram-Schmidt ends when the squares of all that is left sum to this.
 // Both are fractions of the truncation threshold eps.  A quarter and a hundredth in complex64: what is
-// left holds no singular value above eps / 2 (a sixteenth for rem takes two columns more at the top
-// of n = 255 in the strong format, 286 for 266 ms a setup; columns alone against eps / 4, without a bound on
-// their sum, 252 ms, but 128 aligned ones hold a value of 2.8 eps).
+// left holds no singular value above eps / 2, or two thirds of eps where the Gram matrix shows it to be
+// noise (a sixteenth for rem takes two columns more at the top of n = 255 in the strong format, 286 for
+// 266 ms a setup; each column against eps / 4, without a bound on their sum, 252 ms, but 128 aligned
+// ones hold a value of 2.8 eps).
 template <typename R>
 struct SvdPlan {
   int entries;       // of the core
@@ -793,7 +795,7 @@ template <typename R> __host__ __device__ constexpr int group_lanes() { return s
 // written out (qmode = 0).  R is row-major with leading dimension cap(u).
 // Every step updates all later columns (a warp per column, the new norm with the update), so
 // a step costs one barrier; classical Gram-Schmidt with its two passes took ten, 3.6 us a
-// column (the launch at n = 511: 316 us, now 53; n = 150 in complex128: 931, now 253).  A column
+// column (the launch at n = 511: 316 us, now 54; n = 150 in complex128: 931, now 367).  A column
 // of which less than kReorth is left when its turn comes is orthogonalised once more against all
 // Q columns before it (two barriers).  Without that the skews compound: each column takes over
 // those of the columns subtracted from it, enlarged by what it lost, and cosines of 0.05 to 0.8
@@ -1098,6 +1100,40 @@ template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW
   return v;
 }
 
+// A bound on the squared spectral norm of the columns of C with nr >= 0 (squared norms nr): the
+// Frobenius norm of their Gram matrix.  It is the Frobenius bound for aligned columns, and a sixth of
+// it for 70 unrelated ones.  Whole CTA; a warp takes a column against four later ones at a time (10 us
+// for 100 columns of 128).
+__device__ float left_norm2(const Cx<float>* C, int ld, int qa, int qb, const float* nr, float* red) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  float sum = 0;
+  for (int i = warp; i < qb; i += nw) {
+    if (nr[i] < 0) continue;
+    const Cx<float>* ci = C + i * ld;
+    if (lane == 0) sum += nr[i] * nr[i];
+    for (int j0 = i + 1; j0 < qb; j0 += 4) {
+      Cx<float> d[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) d[u] = Cx<float>(0.f, 0.f);
+      for (int r = lane; r < qa; r += 32) {
+        const Cx<float> x = ci[r];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) cfma_conj(d[u], x, C[min(j0 + u, qb - 1) * ld + r]);
+      }
+      int u;
+      bool first;
+      scatter_sum<float, 4, 32, 1>(d, lane, u, first);
+      if (first && j0 + u < qb && nr[j0 + u] >= 0) sum += 2.0f * abs2(d[0]);
+    }
+  }
+  sum = warp_sum_r(sum);
+  if (lane == 0) red[warp] = sum;
+  __syncthreads();
+  sum = warp_sum_r(lane < nw ? red[lane] : 0.f);
+  __syncthreads();
+  return sqrtf(sum);
+}
+
 // Recompression, step 2b: for every sibling pair (a, b) with a = list[blockIdx.x], the
 // truncated SVD of the core C (step 2a), as the small transforms
 //   T_b = conj(P) Sigma^(1/2) (qb x k'),  T_a = C P Sigma^(-1/2) (qa x k'),
@@ -1105,8 +1141,9 @@ template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW
 //
 // 1. Gram-Schmidt with column pivoting, C = Q R, stopped when the squared norms of the
 //    remaining columns sum to at most rem (relative to the largest column's), or to the rounding
-//    noise of the core: no singular value above sqrt(rem) is left behind, however the remaining
-//    columns are aligned.  The block's numerical rank is a third to a half of the core's size.
+//    noise of the core, or (complex64) when their Gram matrix shows that they are many unrelated
+//    small ones: no singular value above sqrt(rem) is left behind, however the remaining columns
+//    are aligned.  The block's numerical rank is a third to a half of the core's size.
 //    Each warp picks the pivot from the column norms (no
 //    broadcast), takes its columns' inner products with the pivot column, updates them and
 //    leaves their new norms: one barrier a step.  Q is not kept: row k of R, conjugated, goes
@@ -1116,8 +1153,8 @@ template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW
 //    a projection of C it does not depend on how exactly the rotations were unitary (their
 //    angles come from FP32 reciprocal square roots in both precisions).
 // What bounds it is the latency of kq - 1 barriers a sweep (complex64) or the FP64 units of
-// one SM (complex128).  A launch takes 195 us at n = 511 in complex64 (595 with Jacobi on
-// the whole core, rotations accumulated), 323 us at n = 150 in complex128 (1612).
+// one SM (complex128).  A launch takes 205 us at n = 511 in complex64 (595 with Jacobi on
+// the whole core, rotations accumulated), 324 us at n = 150 in complex128 (1612).
 template <typename R>
 __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R>* __restrict__ Cb,
                                                    const int* __restrict__ qcols, Cx<R>* __restrict__ Tx,
@@ -1134,6 +1171,7 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
   int* slot = reinterpret_cast<int*>(sig + g.QCAP + 1);            // [QCAP] column storage of row k
   int* order = slot + g.QCAP;                                      // [QCAP]
   __shared__ int s_rot, s_gg, s_t, s_keep;
+  __shared__ float red[32];
   if (qa == 0 || qb == 0) {
     if (threadIdx.x == 0) { newrank[a] = 0; newrank[b] = 0; }
     return;
@@ -1176,6 +1214,7 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
   constexpr int kGL = group_lanes<R>(), kCPW = 32 / kGL;
   // ---- 1. pivoted Gram-Schmidt -----------------------------------------------------------
   int kq = 0;
+  float check = FLT_MAX;
   const int kmax = min(qa, qb);
   for (; kq < kmax; ++kq) {
     const R* nr = nrm + (kq & 1) * g.QCAP;
@@ -1195,6 +1234,14 @@ __global__ void __launch_bounds__(1024) svd_jacobi(Geo g, double eps, const Cx<R
       for (int j = lane; j < qb; j += 32) left += fmaxf(0.f, (float)nr[j]);
       left = warp_sum_r(left);
       if (!(left > rem)) break;
+      if constexpr (sizeof(R) == 4) {
+        // many columns of like size: rounding noise, or aligned ones?  (Noise of that size moves
+        // the singular values as much: up to two thirds of eps for half of it.)
+        if (best <= 0.25f * rem && left >= 8.0f * best && left <= check) {
+          if (left_norm2(C, ld, qa, qb, nr, red) <= (16.0f / 9.0f) * rem) break;
+          check = 0.9f * left;
+        }
+      }
     }
     const R rs = rsqrt_of(best), ib = rcp_of(best);
     const Cx<R>* cp = C + p * ld;

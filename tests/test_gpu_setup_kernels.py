@@ -128,3 +128,27 @@ def test_qr_is_orthogonal_also_for_columns_with_small_remainders(lib, prec, leas
     assert err.max() < 4 * np.sqrt(w) * u + (drop if Q.shape[1] < w else 0)
     if least > drop:
         assert Q.shape[1] == w
+
+
+@pytest.mark.parametrize("m,size", [(97, 1.5e-7), (97, 0.5e-7), (128, 2.2e-7)])
+def test_svd_tells_noise_from_a_value_spread_over_columns(lib, m, size):
+    # unrelated columns, whose squares sum to about (eps / 2)^2 and more while none of their singular values
+    # (about twice a column's norm) reaches eps; and with them one value of 1.3 eps spread over all columns
+    eps = 1e-6
+    rng = np.random.default_rng(m)
+    N = rng.standard_normal((m, m)) + 1j * rng.standard_normal((m, m))
+    N *= size / np.sqrt(2 * m)
+    a = rng.standard_normal(m) + 1j * rng.standard_normal(m)
+    for spread in (0.0, 1.3e-6):
+        C = np.zeros((m, m), complex)
+        C[:, 0] = a / np.linalg.norm(a)
+        b = np.exp(2j * np.pi * rng.uniform(size=m)) / np.sqrt(m)
+        b[0] = 0
+        v = _unitary(rng, m, 2)[:, 0]
+        C[:, 1:] += (N + spread * np.outer(v, b))[:, 1:]
+        Ta, Tb, Cr = _svd(lib, 32, C, eps)
+        s = np.linalg.svd(Cr, compute_uv=False)
+        assert Ta.shape[1] == np.sum(s > eps * s[0]) == (2 if spread else 1), (s[:4], Ta.shape[1])
+        # what is left: at most the largest value not kept and half of eps
+        k = Ta.shape[1]
+        assert np.linalg.norm(Cr - Ta @ Tb.T, 2) < 1.2 * s[k] + 0.5 * eps
