@@ -795,7 +795,7 @@ template <typename R> __host__ __device__ constexpr int group_lanes() { return s
 // written out (qmode = 0).  R is row-major with leading dimension cap(u).
 // Every step updates all later columns (a warp per column, the new norm with the update), so
 // a step costs one barrier; classical Gram-Schmidt with its two passes took ten, 3.6 us a
-// column (the launch at n = 511: 316 us, now 54; n = 150 in complex128: 931, now 367).  A column
+// column (the launch at n = 511: 316 us, now 54; n = 150 in complex128: 931, now 360).  A column
 // of which less than kReorth is left when its turn comes is orthogonalised once more against all
 // Q columns before it (two barriers).  Without that the skews compound: each column takes over
 // those of the columns subtracted from it, enlarged by what it lost, and cosines of 0.05 to 0.8
@@ -870,21 +870,25 @@ __global__ void __launch_bounds__(1024) qr_mgs(Geo g, Cx<R>* __restrict__ G_F, c
         }
       }
       __syncthreads();
-      // four rows a warp, the columns over eight lanes
+      // kRW neighbouring rows a warp (their words are in different banks whatever the column's
+      // place), the columns over 32 / kRW groups of lanes
+      constexpr int kRW = sizeof(R) == 8 ? 8 : 16;
       R part = 0;
-      for (int i0 = 4 * warp; i0 < s; i0 += 4 * nw) {
-        const int i = i0 + lane / 8;
+      for (int i0 = kRW * warp; i0 < s; i0 += kRW * nw) {
+        const int i = i0 + lane % kRW;
         Cx<R> v(0, 0);
-        if (i < s)
-          for (int k = lane % 8; k < qc; k += 8) cfma(v, co[k], Fq[(long long)src[k] * s + i]);
-        for (int o = 4; o > 0; o >>= 1) v += shfl_xor(v, o);
-        if (i < s && lane % 8 == 0) {
+        if (i < s) {
+#pragma unroll 4
+          for (int k = lane / kRW; k < qc; k += 32 / kRW) cfma(v, co[k], Fq[(long long)src[k] * s + i]);
+        }
+        for (int o = kRW; o < 32; o <<= 1) v += shfl_xor(v, o);
+        if (i < s && lane < kRW) {
           v += cj[i];
           cj[i] = v;
           part += abs2(v);
         }
       }
-      for (int o = 8; o < 32; o <<= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+      for (int o = 1; o < kRW; o <<= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
       if (lane == 0) red[warp] = part;
       __syncthreads();
       nr = warp_sum_r(lane < nw ? red[lane] : R(0));
