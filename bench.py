@@ -113,8 +113,8 @@ TEAM_KERNEL_SRC = os.path.join(ROOT, "paper_1007_4290_gb300", "csrc", "sweep_tea
 SLAB_KERNEL_SRC = os.path.join(ROOT, "paper_1007_4290_gb300", "csrc", "sweep_slab.cu")
 # the same for the sweep on dense-diagonal slabs
 SLAB_TRAFFIC = {
-    # profiles/sweep_slab_n1023_random_64rhs_dram.md: 4.719 GB read + 1.577 GB written
-    "n1023_random/64": {"sha256": "244113b7075d1e4f334ffaaafe72f0e653a8abbb856fcd843e91d48df96432e8", "bytes": 6.2957e9},
+    # profiles/sweep_slab_n1023_random_64rhs_dram.md: 4.718 GB read + 1.577 GB written
+    "n1023_random/64": {"sha256": "5f031a112871be22e448f0089fc1a1335a5b7ebc37e8bcaa567f7ba6b086f20f", "bytes": 6.2944e9},
 }
 STRONG_KERNEL_SRC = os.path.join(ROOT, "paper_1007_4290_gb300", "csrc", "sweep_strong.cu")
 # the same for the sweep on the strongly admissible format (R = 2)
