@@ -1108,7 +1108,7 @@ template <typename R> __device__ __forceinline__ Cx<R> group_sum(Cx<R> v, int GW
 // Frobenius norm of their Gram matrix.  It is the Frobenius bound for aligned columns, and a sixth of
 // it for 70 unrelated ones.  Whole CTA; a warp takes a column against four later ones at a time (10 us
 // for 100 columns of 128).
-__device__ float left_norm2(const Cx<float>* C, int ld, int qa, int qb, const float* nr, float* red) {
+__device__ __noinline__ float left_norm2(const Cx<float>* C, int ld, int qa, int qb, const float* nr, float* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   float sum = 0;
   for (int i = warp; i < qb; i += nw) {
